@@ -478,6 +478,51 @@ void fold_constants(InstHost &h) {
   }
 }
 
+// c 2^58 rounded, in limbs ch 2^29 + cl with balanced cl (|c| <= 1).
+int2 limbs58(ld c) {
+  const long long C = llrintl(c * 288230376151711744.0L);
+  long long lo = C & 0x1FFFFFFF;
+  if (lo >= 0x10000000) lo -= 0x20000000;
+  return make_int2((int)((C - lo) >> 29), (int)lo);
+}
+
+// The Burgers operator on mirrored nodes (BurgersFixed) for the integer step.
+void fold_burgers(InstHost &h) {
+  const Ops &o = h.ops;
+  const int Np = o.Np, p = Np - 1, H = Np / 2, mid = Np % 2;
+  adg::BurgersFixed &B = h.I.bf;
+  std::memset(&B, 0, sizeof(B));
+  const ld c2 = -2.0L * (ld)h.dt / (ld)h.dx;
+  auto W = [&](int i, int j) {
+    ld w = o.D[i * Np + j];
+    if (j == 0) w += o.Minv[i * Np];
+    if (j == p) w -= o.Minv[i * Np + p];
+    return 0.5L * c2 * w;
+  };
+  auto a = [&](int i) { return -c2 * o.Minv[i * Np]; };
+  ld S[3][3] = {}, D[2][4] = {}, big = 0;
+  for (int i = 0; i < H + mid; ++i) {
+    for (int j = 0; j < H; ++j) S[i][j] = 0.5L * (W(i, j) - W(i, p - j));
+    S[i][H] = 0.5L * (a(i) + a(p - i));
+    for (int j = 0; j <= H; ++j) big = std::max(big, std::fabs(S[i][j]));
+  }
+  for (int i = 0; i < H; ++i) {
+    for (int j = 0; j < H; ++j) D[i][j] = 0.5L * (W(i, j) + W(i, p - j));
+    if (mid) D[i][H] = W(i, H);
+    D[i][H + mid] = 0.5L * (a(i) - a(p - i));
+    for (int j = 0; j <= H + mid; ++j) big = std::max(big, std::fabs(D[i][j]));
+  }
+  if (!(big > 0) || !std::isfinite((double)big)) return;
+  int e = 0;
+  std::frexp(big, &e);   // big < 2^e
+  B.sc = e;
+  for (int i = 0; i < H + mid; ++i)
+    for (int j = 0; j <= H; ++j) B.S[i][j] = limbs58(std::ldexp(S[i][j], -e));
+  for (int i = 0; i < H; ++i)
+    for (int j = 0; j <= H + mid; ++j) B.D[i][j] = limbs58(std::ldexp(D[i][j], -e));
+  B.ok = 1;
+}
+
 // Composed step constants (StepConsts in adg_internal.h), built in long double from the
 // unrounded stage constants of upwind advection with a > 0.
 // Butcher form (a, b) of the 2N scheme of rk (ls_table): with k_j = L(U_{j-1}), stage s+1's
@@ -1331,6 +1376,9 @@ int reset_exponent(adg_ctx *c, InstHost &h, bool from_scan = false) {
   return ADG_OK;
 }
 
+// The instance takes k_burgers_step (inviscid Burgers, SSP-RK3).
+bool burgers_step(const Inst &I) { return I.pde == ADG_BURGERS && !I.visc && !I.ls; }
+
 // Elements per thread of the composed-step kernel. The FP64 composed step times one, two and
 // four on a copy of u0 held in the instance's v1/v2 fields (free at this point) and keeps the
 // fastest; the fixed-point step takes two for even K, which measured faster in every timing
@@ -1531,6 +1579,7 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
   }
   I.dt = h.dt;
   fold_constants(h);
+  if (burgers_step(I)) fold_burgers(h);
   if (I.euler) {
     const double so[3][3][2] = {{{0.0, 1.0}}, {{0.0, 1.0}, {0.5, 0.5}},
                                 {{0.0, 1.0}, {0.75, 0.25}, {1.0 / 3.0, 2.0 / 3.0}}};
@@ -1786,6 +1835,23 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
     CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
     return ADG_OK;
   }
+  if (!c->batch && burgers_step(c->inst[0].I)) {
+    // u -> v1 -> u ..; an odd count ends u -> v1 -> v2 -> u (a single step: a copy back)
+    const Inst &I = c->inst[0].I;
+    double *in = I.u;
+    for (int rel = 0; rel < nsteps; ++rel) {
+      double *out = in != I.u ? I.u : I.v1;
+      if (nsteps % 2 && rel == nsteps - 2) out = I.v2;
+      CK(adg::launch_burgers_step(I, in, out, nullptr, nullptr, rel, c->stream,
+                                  direct_launches(c) && rel > 0));
+      in = out;
+    }
+    if (in != I.u)
+      CK(cudaMemcpyAsync(I.u, in, (size_t)I.K * I.Np * sizeof(double), cudaMemcpyDeviceToDevice,
+                         c->stream));
+    CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
+    return ADG_OK;
+  }
   for (int rel = 0; rel < nsteps; ++rel) {
     for (int s = 0; s < kStages; ++s) {
       if (c->batch) {
@@ -1967,14 +2033,8 @@ int sweep_recompute(adg_ctx *c, InstHost &h, double *seg, int len, int rel0 = 0)
   const size_t nd = (size_t)h.I.K * h.I.Np;
   for (int t = 0; t < len; ++t) {
     double *slot = seg + (size_t)t * kStages * nd;
-    Inst I = h.I;
-    I.u = slot;
-    I.v1 = slot + nd;
-    I.v2 = slot + 2 * nd;
-    I.unext = slot + kStages * nd;
-    for (int s = 0; s < kStages; ++s) {
-      CK(adg::launch_stage(I, s, rel0 + t, c->stream));
-    }
+    CK(adg::launch_burgers_step(h.I, slot, slot + kStages * nd, slot + nd, slot + 2 * nd, rel0 + t,
+                                c->stream));
   }
   return ADG_OK;
 }

@@ -1,0 +1,90 @@
+// Local block fixed point: FP64 fields in memory, the element arithmetic of the nonlinear
+// stages in 57-bit integers.
+//
+// On this part a warp's FP64 instruction holds the SM's FP64 pipe for 16 clocks (2 lanes per
+// clock per SM), a 32 x 32 -> 64-bit integer product the heavy FMA pipe of one of the four
+// sub-partitions for 4, and shifts and adds run beside it. A stage evaluated in FP64 is bound
+// by that pipe (73-84 FP64 instructions per element at p = 4), so the stages here load FP64
+// values, bring the elements of one warp to a common scale, work in integers, and round once
+// to FP64 when the step is done.
+//
+// A warp's values are X = x 2^(57 - E), |x| < 2^E over all of its elements, so |X| < 2^57 at
+// the start of the step; every intermediate value is checked to stay below 2^58. Squares and
+// face fluxes are held in units of 2^(2E - 56): G = X^2 2^-58. An operator coefficient c is
+// C = round(c 2^(58 - sc)), |C| <= 2^58, split as in adg_fixed.cuh, and sums of products are
+// rounded once. Against FP64: a value is exact to 2^-57 of the warp's largest; the warp takes
+// this path only if every non-zero element reaches 2^-6 of that largest value (kBfSpan), so
+// an element's error per stage is at most about 2^-51 of its own largest value, as the chain of
+// FP64 roundings gives; other warps (and exponents near the ends of the FP64 range, NaN,
+// infinities, growth past the headroom within a step, Courant numbers whose coefficients
+// do not fit) take the FP64 stages.
+#pragma once
+
+#include "adg_fixed.cuh"
+
+namespace adg {
+namespace {
+
+constexpr int kBfSpan = 6;      // exponent span of a warp's elements on the integer path
+constexpr int kBfMinE = 600;    // biased exponents of the warp's largest value
+constexpr int kBfMaxE = 1400;
+constexpr int kBfTop = 58;      // every intermediate value below 2^kBfTop
+
+// x 2^(1079 - be) rounded to an integer: |x| < 2^(be - 1022) gives |X| < 2^57. Exponents
+// below be - 63 (zeros and subnormals among them: be >= kBfMinE) give 0.
+__device__ __forceinline__ long long bf_from(double x, int be) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  int d = be - e;
+  d = d > 63 ? 63 : d;
+  const unsigned long long m =
+      (unsigned long long)fx_join(lo << 5, __funnelshift_l(lo, mh, 5));   // mantissa 2^5
+  const long long M = (long long)(((m >> d) + 1) >> 1);
+  const long long s = (long long)(hi >> 31);
+  return (M ^ s) - s;
+}
+
+// y 2^sigma rounded to nearest even, for results inside the normal range (the integer path's
+// exponents keep them there) or zero.
+__device__ __forceinline__ double bf_to(long long y, int sigma) {
+  const long long s = y >> 63;
+  const unsigned long long a = (unsigned long long)((y ^ s) - s);   // < 2^62
+  const int lz = __clzll((long long)a);
+  const unsigned long long nrm = a << (lz - 1);   // leading one in bit 62: no carry out
+  const unsigned long long m = (nrm + 0x1ffull + ((nrm >> 10) & 1ull)) >> 10;   // <= 2^53
+  // the leading one of m adds one to the exponent field
+  const unsigned long long r = m + ((unsigned long long)(unsigned)(1085 + sigma - lz) << 52);
+  return a == 0 ? 0.0 : __longlong_as_double((long long)(r | ((unsigned long long)s << 63)));
+}
+
+// X^2 2^-58 (|X| < 2^58; below 2 units of error).
+__device__ __forceinline__ long long bf_square(int xh, int xl) {
+  return fx_mul(xh, xh) + (fx_mul(xh, xl) >> 28);
+}
+
+// Local Lax-Friedrichs flux 1/4 (a^2 + b^2) - 1/2 max(|a|, |b|) (b - a) of the traces a = u^-,
+// b = u^+ with squares ga, gb, in the squares' units.
+__device__ __forceinline__ long long bf_llf(long long a, long long b, long long ga, long long gb) {
+  const unsigned long long ma = (unsigned long long)(a < 0 ? -a : a);
+  const unsigned long long mb = (unsigned long long)(b < 0 ? -b : b);
+  int lh, ll, jh, jl;
+  fx_split((long long)(ma >= mb ? ma : mb), lh, ll);
+  fx_split(b - a, jh, jl);
+  const long long prod = fx_mul(lh, jh) + ((fx_mul(lh, jl) + fx_mul(ll, jh)) >> 29);
+  return (ga + gb - 2 * prod + 2) >> 2;
+}
+
+// 1/3 as limbs of round(2^58 / 3).
+constexpr long long kThird = ((1ll << 58) - 1) / 3;
+constexpr int kThirdLo = (int)(((kThird & 0x1FFFFFFF) ^ 0x10000000) - 0x10000000);
+constexpr int kThirdHi = (int)((kThird - kThirdLo) >> 29);
+
+// v 2^-d (d < 0: a left shift; the caller has checked that the result fits).
+__device__ __forceinline__ long long bf_shift(long long v, int d) {
+  return d >= 0 ? v >> d : (long long)((unsigned long long)v << (-d));
+}
+
+}  // namespace
+}  // namespace adg

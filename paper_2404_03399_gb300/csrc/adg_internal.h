@@ -106,6 +106,19 @@ struct FxSlot {
   int sigma;
 };
 
+// The Burgers operator dt L(v)_i = sum_j W_ij g_j + a_i F_L + b_i F_R (g = v^2, F the face
+// fluxes) on mirrored nodes (p - i, p - j; the node set is symmetric, so W and (a, b) change
+// sign under the mirror):
+//   (dt L_i + dt L_{p-i}) / 2 = sum_{j < Np/2} S[i][j] (g_j - g_{p-j}) + S[i][Np/2] (F_L - F_R),
+//   (dt L_i - dt L_{p-i}) / 2 = sum_{j < Np/2} D[i][j] (g_j + g_{p-j}) [+ D[i][Np/2] g_mid]
+//                               + D[i][last] (F_L + F_R),
+// each coefficient c held as C = round(c 2^(58 - sc)), |C| <= 2^58, in limbs as in StepFixed.
+struct BurgersFixed {
+  int2 S[(kMaxNp + 1) / 2][kMaxNp / 2 + 1];
+  int2 D[kMaxNp / 2][(kMaxNp + 1) / 2 + 1];
+  int sc, ok;
+};
+
 // One DG instance as the kernels see it. Nodal fields are node-major: field[i*K + e].
 struct alignas(16) Inst {
   double *u;            // u^n, updated in place by stage 3
@@ -159,6 +172,7 @@ struct alignas(16) Inst {
   double tvb_m, dx;
   double *w;
   double avg_w[kMaxNp], p1_w[kMaxNp], xi[kMaxNp];
+  BurgersFixed bf;      // inviscid Burgers, SSP-RK3 (k_burgers_step)
   double pad3_;
 };
 
@@ -207,6 +221,11 @@ struct AdjFace {
 // One stage over all elements; for an asynchronous instance the same kernel applies the
 // PE-face correction (delayed / AT flux) and writes the ring (step meta[0] + rel).
 cudaError_t launch_stage(const Inst &I, int stage, int rel, cudaStream_t s, bool pdl = false);
+// One SSP-RK3 step of inviscid Burgers uin -> uout (adg_burgers.cu), with the delayed / AT
+// flux and the ring write (its entries hold the face's flux) at PE faces; r1, r2 (both or
+// neither) receive the inputs of stages 1 and 2.
+cudaError_t launch_burgers_step(const Inst &I, const double *uin, double *uout, double *r1,
+                                double *r2, int rel, cudaStream_t s, bool pdl = false);
 // Stage s of a 2N low-storage step (I.ls): dU_s = A_s dU_{s-1} + dt L(U_{s-1}) in place in
 // I.v1 (A_1 = 0: dU_0 is not read) and U_s = U_{s-1} + B_s dU_s from uin (U_{s-1}) into uout,
 // with the delayed / AT flux and the ring write of the stage-input traces at PE faces.

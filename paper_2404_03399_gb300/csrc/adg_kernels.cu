@@ -223,7 +223,7 @@ __device__ __forceinline__ void stage_body(const I &inst, int e, int64_t n = 0,
 // it (the halo lanes' 2/32 redundant work replaces the single-lane flux and the second
 // evaluation of every PE-face value, which a warp's FP64 instruction pays in full whatever its
 // active lanes).
-template <int NP, int PDE, int STAGE, int DIR, bool FACES, class I>
+template <int NP, int STAGE, int DIR, bool FACES, class I>
 __device__ __forceinline__ void stage_body_halo(const I &inst, int warp, int64_t n) {
   const int K = inst.K;
   const int lane = threadIdx.x & 31;
@@ -257,41 +257,16 @@ __device__ __forceinline__ void stage_body_halo(const I &inst, int warp, int64_t
   const double vLm = __shfl_up_sync(full, v[NP - 1], 1);   // lanes >= 1
   const double vRp = __shfl_down_sync(full, v[0], 1);      // lanes <= 30
   double jL = 0.0, jR = 0.0;
-  if (PDE == 0) {
-    if (DIR > 0) jL = __dsub_rn(v[0], vLm);
-    else jR = __dsub_rn(v[NP - 1], vRp);
-  } else {
-    const double FL = num_flux<1>(0.0, vLm, v[0]);
-    const double FR = __shfl_down_sync(full, FL, 1);
-    jL = __dsub_rn(phys_flux<1>(0.0, v[0]), FL);
-    jR = __dsub_rn(phys_flux<1>(0.0, v[NP - 1]), FR);
-  }
-
-  double g[NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) g[i] = PDE == 0 ? v[i] : v[i] * v[i];
+  if (DIR > 0) jL = __dsub_rn(v[0], vLm);
+  else jR = __dsub_rn(v[NP - 1], vRp);
 
   double out[NP];
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
-    double acc;
-    if (PDE == 0) {
-      acc = STAGE == 0 ? C.A[i * NP] * g[0] : fma(C.A[i * NP], g[0], C.alpha * u[i]);
-    } else {
-      acc = STAGE == 0 ? v[i] : fma(C.beta, v[i], C.alpha * u[i]);
-      acc = fma(C.A[i * NP], g[0], acc);
-    }
+    double acc = STAGE == 0 ? C.A[i * NP] * v[0] : fma(C.A[i * NP], v[0], C.alpha * u[i]);
 #pragma unroll
-    for (int jj = 1; jj < NP; ++jj) acc = fma(C.A[i * NP + jj], g[jj], acc);
-    out[i] = acc;
-  }
-  if (PDE == 1 || DIR > 0) {
-#pragma unroll
-    for (int i = 0; i < NP; ++i) out[i] = fma(C.lL[i], jL, out[i]);
-  }
-  if (PDE == 1 || DIR < 0) {
-#pragma unroll
-    for (int i = 0; i < NP; ++i) out[i] = fma(C.lR[i], jR, out[i]);
+    for (int jj = 1; jj < NP; ++jj) acc = fma(C.A[i * NP + jj], v[jj], acc);
+    out[i] = DIR > 0 ? fma(C.lL[i], jL, acc) : fma(C.lR[i], jR, acc);
   }
   if (FACES) {
     // lane l (1 .. 31) forms the PE-face difference of its left face when its element owns
@@ -301,7 +276,7 @@ __device__ __forceinline__ void stage_body_halo(const I &inst, int warp, int64_t
     const int jq = eo / Kpe;
     const bool face = lane >= 1 && e <= K && eo - jq * Kpe == 0;
     double d = 0.0;
-    if (face) d = pe_face_delta<PDE, DIR>(inst, jq, n, STAGE, vLm, v[0], own);
+    if (face) d = pe_face_delta<0, DIR>(inst, jq, n, STAGE, vLm, v[0], own);
     const double dR = __shfl_down_sync(full, d, 1);
     const bool faceR = __shfl_down_sync(full, face ? 1 : 0, 1) != 0;
     if (own && face && nonzero(d)) {
@@ -323,12 +298,12 @@ __device__ __forceinline__ void stage_body_halo(const I &inst, int warp, int64_t
   }
 }
 
-template <int NP, int PDE, int STAGE, int DIR, bool FACES>
+template <int NP, int STAGE, int DIR, bool FACES>
 __global__ void __launch_bounds__(kTile) k_stage_halo(const Inst inst, int rel) {
   pdl_wait();   // the stage before (programmatic launch) has written this one's input
   pdl_trigger();
   const int64_t n = FACES ? inst.meta[0] + rel : 0;
-  stage_body_halo<NP, PDE, STAGE, DIR, FACES>(inst, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n);
+  stage_body_halo<NP, STAGE, DIR, FACES>(inst, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n);
 }
 
 template <int NP, int PDE, int STAGE, int DIR, bool FACES, bool VISC = false>
@@ -1320,21 +1295,21 @@ __global__ void __launch_bounds__(kRedThreads)
 template <int NP, int PDE, int STAGE, int DIR>
 cudaError_t launch_np_pde_stage(const Inst &I, int rel, cudaStream_t s, bool pdl) {
   const int bs = stage_block(I.K);
-  const unsigned grid = (unsigned)((I.K + bs - 1) / bs);
-  if (PDE == 1 && I.visc) {
+  if constexpr (PDE == 1) {   // viscous (inviscid Burgers takes k_burgers_step)
+    if (!I.visc) return cudaErrorInvalidValue;
+    const dim3 g((unsigned)((I.K + bs - 1) / bs));
     if (I.async)
-      return launch_maybe_pdl(k_stage<NP, PDE, STAGE, DIR, true, true>, dim3(grid), dim3(bs), s,
-                              pdl, I, rel);
-    return launch_maybe_pdl(k_stage<NP, PDE, STAGE, DIR, false, true>, dim3(grid), dim3(bs), s,
-                            pdl, I, rel);
+      return launch_maybe_pdl(k_stage<NP, PDE, STAGE, DIR, true, true>, g, dim3(bs), s, pdl, I, rel);
+    return launch_maybe_pdl(k_stage<NP, PDE, STAGE, DIR, false, true>, g, dim3(bs), s, pdl, I, rel);
+  } else {
+    // 30 elements per warp (halo lanes); one-thread-per-element stage_body is kept for the 2N
+    // low-storage, viscous and batched stages
+    const int64_t warps = (I.K + 29) / 30;
+    const dim3 g((unsigned)((warps * 32 + bs - 1) / bs));
+    if (I.async)
+      return launch_maybe_pdl(k_stage_halo<NP, STAGE, DIR, true>, g, dim3(bs), s, pdl, I, rel);
+    return launch_maybe_pdl(k_stage_halo<NP, STAGE, DIR, false>, g, dim3(bs), s, pdl, I, rel);
   }
-  // 30 elements per warp (halo lanes); one-thread-per-element stage_body is kept for the 2N
-  // low-storage, viscous and batched stages
-  const int64_t warps = (I.K + 29) / 30;
-  const dim3 g((unsigned)((warps * 32 + bs - 1) / bs));
-  if (I.async)
-    return launch_maybe_pdl(k_stage_halo<NP, PDE, STAGE, DIR, true>, g, dim3(bs), s, pdl, I, rel);
-  return launch_maybe_pdl(k_stage_halo<NP, PDE, STAGE, DIR, false>, g, dim3(bs), s, pdl, I, rel);
 }
 
 template <int NP, int PDE, int DIR>

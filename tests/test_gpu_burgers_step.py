@@ -1,0 +1,69 @@
+"""The fused SSP-RK3 step of inviscid Burgers (local block fixed point, with its FP64 path)
+against the CPU oracle: mesh sizes around the warp's 26 owned elements, every degree and mode,
+fields the integer path takes and fields it leaves to FP64."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+import paper_2404_03399_gb300 as adg  # noqa: E402
+from oracle import delays as odelays, dg  # noqa: E402
+from workloads import random_nodal  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-12   # the parity bar of the other kernels, relative to the field's maximum
+
+
+def _pair(cfg, u0, steps):
+    s = adg.Solver(cfg, torch.tensor(u0, device="cuda"))
+    s.step(steps)
+    got, dt = s.state().cpu().numpy(), s.dt
+    s.close()
+    sync = cfg.mode == "sync" or cfg.P == 1
+    tbl = None if sync else odelays.delay_table(cfg.seed, cfg.P, steps, cfg.L)
+    prob = dg.Problem(pde="burgers", K=cfg.K, p=cfg.p, P=cfg.P, dt=dt, x0=cfg.x0, x1=cfg.x1,
+                      mode="sync" if sync else "adg", q=cfg.q if cfg.mode == "at" else 1, delays=tbl)
+    return got, dg.run(prob, u0, steps).numpy()
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("K,P,mode", [(3, 1, "sync"), (26, 26, "async"), (27, 9, "at"), (53, 1, "sync"),
+                                      (31, 31, "at"), (1000, 8, "at")])
+def test_sizes_degrees_and_modes(K, P, mode, p):
+    cfg = adg.Config(pde="burgers", K=K, p=p, P=P, cfl=0.004, mode=mode, L=3, q=2, seed=4)
+    got, ref = _pair(cfg, 0.3 + random_nodal(K, p, 7), 33)
+    assert np.max(np.abs(got - ref)) < TOL * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("field", ["pulse", "tiny", "huge", "courant", "zero patch"])
+def test_fields_outside_the_integer_path(field):
+    # pulse: elements far below the warp's largest value keep their own relative accuracy;
+    # tiny and huge: exponents beyond the integer path's range; courant: operator coefficients
+    # above its headroom; zero patch: zero elements beside others
+    K, p, cfl = 512, 3, 0.01
+    x = dg.node_coordinates(K, p, 0.0, 2.0 * math.pi)
+    u0 = 0.5 + np.sin(x)
+    if field == "pulse":
+        u0 = np.exp(-40.0 * (x - math.pi) ** 2)
+    elif field in ("tiny", "huge"):
+        u0 = u0 * (1e-150 if field == "tiny" else 1e140)
+    elif field == "courant":
+        cfl = 0.3
+    elif field == "zero patch":
+        u0 = np.where(np.abs(x - math.pi) < 1.0, 0.0, u0)
+    cfg = adg.Config(pde="burgers", K=K, p=p, P=8, cfl=cfl, mode="at" if field != "courant" else "sync",
+                     L=3, q=2, seed=9)
+    got, ref = _pair(cfg, u0, 40 if field != "courant" else 4)
+    tol = TOL * np.max(np.abs(ref))
+    if field == "courant":
+        # unstable at this Courant number: one rounding of u0 already moves the oracle by more
+        # than the bar, so the run is held to eight times that, as on the decaying field
+        ulp = np.random.default_rng(0).uniform(-1.0, 1.0, u0.shape) * 2.0**-52
+        prob = dg.Problem(pde="burgers", K=K, p=p, P=1, dt=dg.dt_from_cfl("burgers", cfl, 2.0 * math.pi / K, 1.0, u0),
+                          x0=cfg.x0, x1=cfg.x1, mode="sync", q=1, delays=None)
+        tol = 8.0 * np.max(np.abs(dg.run(prob, u0 * (1.0 + ulp), 4).numpy() - ref))
+    assert np.max(np.abs(got - ref)) < tol
+    if field == "pulse":
+        big = np.max(np.abs(ref), axis=1, keepdims=True)
+        assert np.max(np.abs(got - ref) / big) < 1e-11   # every element to its own largest value
