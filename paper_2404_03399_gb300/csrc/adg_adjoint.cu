@@ -1,13 +1,13 @@
 // Discrete adjoint of the ADG / ADG-AT SSP-RK3 step (used by adg_grad).
 //
-// The forward stage, per element, is (see adg_internal.h)
-//   out = alpha u + A v + lL (f(v_0) - F_L) + lR (f(v_p) - F_R)      (Burgers adds beta v,
-// with A applied to v^2), followed at PE faces by out^e += lL d, out^{e-1} += lR d with
-// d = F_sync - F_delayed. Its transpose, for the adjoint w of the stage output, is
-//   lambda_u += alpha w,
-//   lambda_v  = A^T w (advection) or beta w + 2 v (A^T w) (Burgers),
-//   face adjoint mu_f = -(lL . w^f) - (lR . w^{f-1}) applied through the flux partial
-//   derivatives to the traces of the stage input,
+// Here advection, stage by stage; Burgers takes one kernel per step (adg_burgers.cu). The
+// forward stage, per element, is (see adg_internal.h)
+//   out = alpha u + A v + lL (v_0 - G_L) + lR (v_p - G_R),
+// followed at PE faces by out^e += lL d, out^{e-1} += lR d with d = G_sync - G_delayed. Its
+// transpose, for the adjoint w of the stage output, is
+//   lambda_u += alpha w,   lambda_v = A^T w,
+//   face adjoint mu_f = -(lL . w^f) - (lR . w^{f-1}) applied to the upwind trace of the stage
+//   input,
 // and at PE faces the delayed flux F = sum_i c_i fhat(T_{n-k-i}) sends c_i mu_f to an
 // adjoint ring indexed like the forward one; the entry of level m, stage s is turned into
 // trace adjoints when the reverse sweep reaches step m, stage s.
@@ -15,31 +15,6 @@
 
 namespace adg {
 namespace {
-
-// Partial derivatives of the local Lax-Friedrichs flux
-//   F = 1/2 (uL^2/2 + uR^2/2) - 1/2 lam (uR - uL),  lam = max(|uL|, |uR|),
-// with lam taken from uL when |uL| >= |uR| and d|u|/du = +1 for u >= 0, -1 otherwise.
-__device__ __forceinline__ void llf_partials(double uL, double uR, double &dL, double &dR) {
-  const bool fromL = abs_bits(uL) >= abs_bits(uR);
-  const double lam = fromL ? fabs(uL) : fabs(uR);
-  const double jump = uR - uL;
-  double gL = 0.0, gR = 0.0;
-  if (fromL) gL = nonneg(uL) ? 1.0 : -1.0;
-  else gR = nonneg(uR) ? 1.0 : -1.0;
-  dL = 0.5 * uL + 0.5 * lam - 0.5 * gL * jump;
-  dR = 0.5 * uR - 0.5 * lam - 0.5 * gR * jump;
-}
-
-// Partials of the face value (trace units for advection, flux for Burgers).
-template <int PDE, int DIR>
-__device__ __forceinline__ void value_partials(double tl, double tr, double &dL, double &dR) {
-  if (PDE == 0) {
-    dL = DIR > 0 ? 1.0 : 0.0;
-    dR = DIR > 0 ? 0.0 : 1.0;
-  } else {
-    llf_partials(tl, tr, dL, dR);
-  }
-}
 
 // Adjoint of one stage with halo lanes (the layout of the forward k_stage_halo): warp w takes
 // elements 30w .. 30w+29 in lanes 1 .. 30 and lanes 0 and 31 hold the elements on either side
@@ -49,7 +24,7 @@ __device__ __forceinline__ void value_partials(double tl, double tr, double &dL,
 // (which, owned, also posts the delayed levels and clears the ring entry). A warp's FP64
 // instruction costs the same pipe time whatever its active lanes, so the halo lanes' 2/32
 // redundant work is cheaper than single-lane edge and face work.
-template <int NP, int PDE, int STAGE, int DIR, bool FACES>
+template <int NP, int STAGE, int DIR, bool FACES>
 __global__ void __launch_bounds__(kTile) k_adj_stage_halo(const AdjStage A) {
   const int K = A.K;
   const int lane = threadIdx.x & 31;
@@ -68,38 +43,21 @@ __global__ void __launch_bounds__(kTile) k_adj_stage_halo(const AdjStage A) {
     sL = fma(C.lL[i], w[i], sL);
     sR = fma(C.lR[i], w[i], sR);
   }
-  double v[NP];
-  if (PDE == 1) {
-#pragma unroll
-    for (int i = 0; i < NP; ++i) v[i] = __ldg(A.v + (size_t)i * K + ec);
-  }
   double lv[NP];
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
     double acc = C.A[j] * w[0];
 #pragma unroll
     for (int i = 1; i < NP; ++i) acc = fma(C.A[i * NP + j], w[i], acc);
-    lv[j] = PDE == 0 ? acc : fma(C.beta, w[j], 2.0 * v[j] * acc);
+    lv[j] = acc;
   }
   const double sRp = __shfl_up_sync(full, sR, 1);     // sR of the element to the left
-  if (PDE == 0) {
-    if (DIR > 0) {
-      lv[0] += sL;
-      lv[NP - 1] -= __shfl_down_sync(full, sL, 1);
-    } else {
-      lv[NP - 1] += sR;
-      lv[0] -= sRp;
-    }
+  if (DIR > 0) {
+    lv[0] += sL;
+    lv[NP - 1] -= __shfl_down_sync(full, sL, 1);
   } else {
-    lv[0] = fma(v[0], sL, lv[0]);
-    lv[NP - 1] = fma(v[NP - 1], sR, lv[NP - 1]);
-    // left face of e: adjoint mu = -sL^e - sR^{e-1}, traces (v_p^{e-1}, v_0^e)
-    const double vLm = __shfl_up_sync(full, v[NP - 1], 1);
-    const double muL = -sL - sRp;
-    double dL, dR;
-    llf_partials(vLm, v[0], dL, dR);
-    lv[0] = fma(muL, dR, lv[0]);
-    lv[NP - 1] += __shfl_down_sync(full, muL * dL, 1);
+    lv[NP - 1] += sR;
+    lv[0] -= sRp;
   }
 
   if (FACES) {
@@ -109,7 +67,6 @@ __global__ void __launch_bounds__(kTile) k_adj_stage_halo(const AdjStage A) {
     // and both elements add g times the value's partial derivative to their trace node (the
     // left one through a shuffle); an owned lane also posts c_i (-nu) to the delayed levels
     // (never to level n) and clears the ring entry the previous adjoint kernel read.
-    const double tl = PDE == 1 ? __shfl_up_sync(full, v[NP - 1], 1) : 0.0;
     const int eo = e < K ? e : e - K;
     const int jq = eo / A.Kpe;
     const bool face = lane >= 1 && e <= K && eo - jq * A.Kpe == 0;
@@ -126,7 +83,8 @@ __global__ void __launch_bounds__(kTile) k_adj_stage_halo(const AdjStage A) {
       const DelayAt d = delay_at(A, jq, n);
       const double r = A.lring[((size_t)nm * kStages + STAGE) * A.P + jq];
       g = d.k == 0 ? r : nu + r;
-      value_partials<PDE, DIR>(tl, PDE == 1 ? v[0] : 0.0, pL, pR);
+      pL = DIR > 0 ? 1.0 : 0.0;   // the value is the upwind trace
+      pR = DIR > 0 ? 0.0 : 1.0;
       if (own) {
         for (int i = 0; i < d.qe; ++i) {
           const double ci = d.c[i];
@@ -164,7 +122,7 @@ __global__ void __launch_bounds__(kTile) k_adj_stage_halo(const AdjStage A) {
 //   the synchronous flux the stage kernel assumed is undone (+nu on its partials);
 //   the delayed levels receive c_i (-nu) in the adjoint ring;
 //   the ring entry of this step and stage becomes trace adjoints, then is cleared.
-template <int PDE, int DIR>
+template <int DIR>
 __global__ void __launch_bounds__(256) k_adj_faces(const AdjFace F) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= F.P) return;
@@ -186,16 +144,8 @@ __global__ void __launch_bounds__(256) k_adj_faces(const AdjFace F) {
   double *slot = F.lring + (ring_slot(n, F.R) * kStages + s) * F.P + j;
   const double r = *slot;
   *slot = 0.0;
-  double tl = 0.0, tr = 0.0;
-  if (PDE == 1) {
-    tl = F.v[(size_t)(Np - 1) * K + eL];
-    tr = F.v[e];
-  }
-  double dL, dR;
-  value_partials<PDE, DIR>(tl, tr, dL, dR);
-  const double g = nu + r;
-  F.target[(size_t)(Np - 1) * K + eL] += g * dL;
-  F.target[e] += g * dR;
+  const double g = nu + r;   // to the upwind trace
+  F.target[DIR > 0 ? (size_t)(Np - 1) * K + eL : (size_t)e] += g;
 }
 
 __global__ void k_adj_init(const double *__restrict__ u, const double *__restrict__ g, int K,
@@ -211,56 +161,47 @@ __global__ void k_adj_init(const double *__restrict__ u, const double *__restric
   }
 }
 
-template <int NP, int PDE, int STAGE, bool FACES>
+template <int NP, int STAGE, bool FACES>
 cudaError_t adj_launch(const AdjStage &A, int dir, cudaStream_t s) {
   const int bs = stage_block(A.K);
-  const unsigned grid = (unsigned)((A.K + bs - 1) / bs);
-  (void)grid;
   // 30 elements per warp (halo lanes)
   const int64_t warps = (A.K + 29) / 30;
   const unsigned g = (unsigned)((warps * 32 + bs - 1) / bs);
-  if (PDE == 1) k_adj_stage_halo<NP, 1, STAGE, 0, FACES><<<g, bs, 0, s>>>(A);
-  else if (dir > 0) k_adj_stage_halo<NP, 0, STAGE, 1, FACES><<<g, bs, 0, s>>>(A);
-  else k_adj_stage_halo<NP, 0, STAGE, -1, FACES><<<g, bs, 0, s>>>(A);
+  if (dir > 0) k_adj_stage_halo<NP, STAGE, 1, FACES><<<g, bs, 0, s>>>(A);
+  else k_adj_stage_halo<NP, STAGE, -1, FACES><<<g, bs, 0, s>>>(A);
   return cudaGetLastError();
 }
 
-template <int NP, int PDE, int STAGE>
-cudaError_t adj_np_pde_stage(const AdjStage &A, int dir, cudaStream_t s) {
-  return A.faces ? adj_launch<NP, PDE, STAGE, true>(A, dir, s) : adj_launch<NP, PDE, STAGE, false>(A, dir, s);
-}
-
-template <int NP, int PDE>
-cudaError_t adj_np_pde(const AdjStage &A, int stage, int dir, cudaStream_t s) {
-  switch (stage) {
-    case 0: return adj_np_pde_stage<NP, PDE, 0>(A, dir, s);
-    case 1: return adj_np_pde_stage<NP, PDE, 1>(A, dir, s);
-    default: return adj_np_pde_stage<NP, PDE, 2>(A, dir, s);
-  }
+template <int NP, int STAGE>
+cudaError_t adj_np_stage(const AdjStage &A, int dir, cudaStream_t s) {
+  return A.faces ? adj_launch<NP, STAGE, true>(A, dir, s) : adj_launch<NP, STAGE, false>(A, dir, s);
 }
 
 template <int NP>
-cudaError_t adj_np(const AdjStage &A, int pde, int stage, int dir, cudaStream_t s) {
-  return pde == 1 ? adj_np_pde<NP, 1>(A, stage, dir, s) : adj_np_pde<NP, 0>(A, stage, dir, s);
+cudaError_t adj_np(const AdjStage &A, int stage, int dir, cudaStream_t s) {
+  switch (stage) {
+    case 0: return adj_np_stage<NP, 0>(A, dir, s);
+    case 1: return adj_np_stage<NP, 1>(A, dir, s);
+    default: return adj_np_stage<NP, 2>(A, dir, s);
+  }
 }
 
 }  // namespace
 
-cudaError_t launch_adj_stage(const AdjStage &A, int pde, int stage, int dir, cudaStream_t s) {
+cudaError_t launch_adj_stage(const AdjStage &A, int stage, int dir, cudaStream_t s) {
   switch (A.Np) {
-    case 2: return adj_np<2>(A, pde, stage, dir, s);
-    case 3: return adj_np<3>(A, pde, stage, dir, s);
-    case 4: return adj_np<4>(A, pde, stage, dir, s);
-    case 5: return adj_np<5>(A, pde, stage, dir, s);
+    case 2: return adj_np<2>(A, stage, dir, s);
+    case 3: return adj_np<3>(A, stage, dir, s);
+    case 4: return adj_np<4>(A, stage, dir, s);
+    case 5: return adj_np<5>(A, stage, dir, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_adj_faces(const AdjFace &F, int pde, int dir, cudaStream_t s) {
+cudaError_t launch_adj_faces(const AdjFace &F, int dir, cudaStream_t s) {
   const unsigned grid = (unsigned)((F.P + 255) / 256);
-  if (pde == 1) k_adj_faces<1, 0><<<grid, 256, 0, s>>>(F);
-  else if (dir > 0) k_adj_faces<0, 1><<<grid, 256, 0, s>>>(F);
-  else k_adj_faces<0, -1><<<grid, 256, 0, s>>>(F);
+  if (dir > 0) k_adj_faces<1><<<grid, 256, 0, s>>>(F);
+  else k_adj_faces<-1><<<grid, 256, 0, s>>>(F);
   return cudaGetLastError();
 }
 

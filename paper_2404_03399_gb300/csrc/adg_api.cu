@@ -2049,11 +2049,14 @@ int sweep_reverse(adg_ctx *c, InstHost &h, const double *seg, double *lam, doubl
   double *Lv = lam + 2 * nd, *Lv2 = lam + 3 * nd;
   for (int t = len - 1; t >= 0; --t) {
     double *Lu = lam + (size_t)par * nd, *Lacc = lam + (size_t)(1 - par) * nd;
-    const double *slot = seg ? seg + (size_t)t * kStages * nd : nullptr;
+    if (seg) {   // Burgers: one kernel per step
+      CK(adg::launch_burgers_adj(I, seg + (size_t)t * kStages * nd, Lu, Lacc, lring, t, c->stream));
+      par = 1 - par;
+      continue;
+    }
     for (int s = kStages - 1; s >= 0; --s) {
       adg::AdjStage A;
       A.w = s == 2 ? Lu : (s == 1 ? Lv : Lv2);
-      A.v = slot ? slot + (size_t)s * nd : nullptr;
       A.lv = s == 2 ? Lv : (s == 1 ? Lv2 : nullptr);
       A.lacc = Lacc;
       A.K = I.K;
@@ -2070,11 +2073,10 @@ int sweep_reverse(adg_ctx *c, InstHost &h, const double *seg, double *lam, doubl
       A.R = I.R;
       A.q = I.q;
       A.faces = (I.async && I.Kpe >= 8) ? 1 : 0;
-      CK(adg::launch_adj_stage(A, I.pde, s, dir, c->stream));
+      CK(adg::launch_adj_stage(A, s, dir, c->stream));
       if (I.async && !A.faces) {
         adg::AdjFace F;
         F.w = A.w;
-        F.v = A.v;
         F.target = s == 0 ? Lacc : A.lv;
         F.lring = lring;
         F.table = I.table;
@@ -2092,7 +2094,7 @@ int sweep_reverse(adg_ctx *c, InstHost &h, const double *seg, double *lam, doubl
           F.lL[i] = I.sc[s].lL[i];
           F.lR[i] = I.sc[s].lR[i];
         }
-        CK(adg::launch_adj_faces(F, I.pde, dir, c->stream));
+        CK(adg::launch_adj_faces(F, dir, c->stream));
       }
     }
     par = 1 - par;

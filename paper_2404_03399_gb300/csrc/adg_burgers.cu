@@ -1,4 +1,5 @@
-// Inviscid Burgers, SSP-RK3: one kernel per step, the three stages in registers.
+// Inviscid Burgers, SSP-RK3: one kernel per step and one per step of its discrete adjoint,
+// the three stages in registers.
 #include "adg_bfp.cuh"
 #include "adg_device.cuh"
 
@@ -241,6 +242,302 @@ __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ In
   burgers_step_fp64<NP, FACES, REC>(I, warp, uin, uout, r1, r2, nm, sV, pe, late);
 }
 
+// What the reverse step reads: the recorded stage inputs u, v1, v2 (y, one field of nd values
+// after another), the adjoint of u^{n+1} (w), the adjoint ring; it writes the adjoint of u^n.
+struct AdjArgs {
+  const double *y;
+  const double *w;
+  double *out;
+  double *lring;
+  int rel;
+};
+
+// Partial derivatives of the local Lax-Friedrichs flux (adg_adjoint.cu), doubled and in
+// integers: lambda from a where |a| >= |b|, d|x|/dx = 1 for x >= 0.
+__device__ __forceinline__ void bf_llf_partials2(long long a, long long b, long long &dl,
+                                                 long long &dr) {
+  const long long ma = a < 0 ? -a : a, mb = b < 0 ? -b : b;
+  if (ma >= mb) {
+    dl = a >= 0 ? 3 * a - b : b - a;
+    dr = b - ma;
+  } else {
+    dl = a + mb;
+    dr = b >= 0 ? a - b : 3 * b - a;
+  }
+}
+
+// The same in FP64.
+__device__ __forceinline__ void llf_partials_fp64(double a, double b, double &dl, double &dr) {
+  const bool left = abs_bits(a) >= abs_bits(b);
+  const double lam = left ? fabs(a) : fabs(b), jump = b - a;
+  const double gl = left ? (nonneg(a) ? 1.0 : -1.0) : 0.0;
+  const double gr = left ? 0.0 : (nonneg(b) ? 1.0 : -1.0);
+  dl = 0.5 * a + 0.5 * lam - 0.5 * gl * jump;
+  dr = 0.5 * b - 0.5 * lam - 0.5 * gr * jump;
+}
+
+// A PE face in the reverse sweep: the flux adjoint mu of the stage is posted, times the AT
+// coefficients, to the delayed levels' ring entries (its owner only).
+__device__ __forceinline__ void post_levels(const Inst &I, double *lring, int j, int nm, int s,
+                                            int k, int qe, const double *c, double mu) {
+  for (int i = 0; i < qe; ++i) {
+    if (k + i < 1 || c[i] == 0.0) continue;
+    int sl = nm - k - i;
+    if (sl < 0) sl += I.R;
+    double *q = lring + ((size_t)sl * kStages + s) * I.P + j;
+    *q += c[i] * mu;
+  }
+}
+
+// The reverse step in FP64 (warps that the integer path does not take); face: pe as in
+// burgers_step_fp64, sR[stage][lane] the ring entries of this step.
+template <int NP, bool FACES>
+__device__ __noinline__ void burgers_adj_fp64(const Inst &I, const AdjArgs &A, int warp, int nm,
+                                              const double (*sR)[32], bool pe, int k, int qe,
+                                              const double *c) {
+  const int K = I.K;
+  const size_t nd = (size_t)K * NP;
+  const int lane = threadIdx.x & 31;
+  bool own;
+  const int e = warp_element(K, warp, lane, own);
+  const unsigned full = 0xffffffffu;
+  double w[NP], acc[NP];
+  load_elem<NP>(A.w, K, e, w);
+#pragma unroll
+  for (int i = 0; i < NP; ++i) acc[i] = 0.0;
+#pragma unroll
+  for (int s = kStages - 1; s >= 0; --s) {
+    const StageConsts &C = I.sc[s];
+    double v[NP], lv[NP];
+    load_elem<NP>(A.y + s * nd, K, e, v);
+    double sL = 0.0, sRt = 0.0;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      sL = fma(C.lL[i], w[i], sL);
+      sRt = fma(C.lR[i], w[i], sRt);
+    }
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      double a = C.A[j] * w[0];
+#pragma unroll
+      for (int i = 1; i < NP; ++i) a = fma(C.A[i * NP + j], w[i], a);
+      lv[j] = fma(C.beta, w[j], 2.0 * v[j] * a);
+    }
+    lv[0] = fma(v[0], sL, lv[0]);
+    lv[NP - 1] = fma(v[NP - 1], sRt, lv[NP - 1]);
+    double mu = -sL - __shfl_up_sync(full, sRt, 1);
+    double dl, dr;
+    llf_partials_fp64(__shfl_up_sync(full, v[NP - 1], 1), v[0], dl, dr);
+    if (FACES && pe) {
+      const double r = sR[s][lane];
+      if (own) post_levels(I, A.lring, e / I.Kpe, nm, s, k, qe, c, mu);
+      mu = k > 0 ? r : mu + r;
+    }
+    lv[0] = fma(mu, dr, lv[0]);
+    lv[NP - 1] += __shfl_down_sync(full, mu * dl, 1);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      if (s == 2) acc[i] = C.alpha * w[i];
+      if (s == 1) acc[i] = fma(C.alpha, w[i], acc[i]);
+      w[i] = lv[i];
+    }
+  }
+  if (own) {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) A.out[(size_t)i * K + e] = acc[i] + w[i];
+  }
+}
+
+// The adjoint of one SSP-RK3 step of inviscid Burgers, from the recorded stage inputs: the
+// layout and the integer arithmetic of k_burgers_step, with a second scale for the adjoint
+// (Ew: |w| < 2^Ew over the warp). For the adjoint w of a stage's output the adjoint of its
+// input v is beta (w + Z),
+//   Z_j = 2 v_j (W^T w)_j + (mu_L dF_L/du^+ at j = 0) + (mu_R dF_R/du^- at j = p),
+// mu the flux adjoints a . w^e + b . w^{e-1}; W^T, a and b act on sums and differences of
+// mirrored nodes with the coefficients of the forward step (transposed). A PE face posts
+// c_i mu to the delayed levels of the adjoint ring and takes the ring entry of its own step
+// and stage for (delay > 0) or beside (delay 0) mu; its owner clears the entries of step
+// n + 1, which the kernel before this one read. The gradient on 65536 elements (p = 3, 100
+// steps): 6.3 -> 3.9 ms against
+// three FP64 stage kernels of 14 us each, bound by the FP64 pipe.
+template <int NP, bool FACES>
+__global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Inst I,
+                                                     const __grid_constant__ AdjArgs A) {
+  constexpr int HP = NP / 2, MID = NP % 2;
+  __shared__ double sR_[FACES ? 4 * kStages : 1][32];
+  const int K = I.K;
+  const size_t nd = (size_t)K * NP;
+  const int lane = threadIdx.x & 31;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if ((int64_t)warp * kOwn >= K) return;
+  const unsigned full = 0xffffffffu;
+  bool own;
+  const int e = warp_element(K, warp, lane, own);
+  double wd[NP], yd[kStages][NP];
+  load_elem<NP>(A.w, K, e, wd);
+#pragma unroll
+  for (int s = 0; s < kStages; ++s) load_elem<NP>(A.y + s * nd, K, e, yd[s]);
+
+  bool pe = false;
+  int nm = 0, k = 0, qe = 0;
+  const double *c = nullptr;
+  double (*sR)[32] = sR_ + (FACES ? (threadIdx.x >> 5) * kStages : 0);
+  int rmax = 0;
+  if (FACES) {
+    const int j = e / I.Kpe;
+    const int64_t n = I.meta[0] + A.rel;
+    nm = (int)(n % I.R);
+    pe = e == j * I.Kpe;
+    if (pe) {
+      const DelayAt d = delay_at(I, j, n);
+      k = d.k;
+      qe = d.qe;
+      c = d.c;
+      const int nx = nm + 1 == I.R ? 0 : nm + 1;
+#pragma unroll
+      for (int s = 0; s < kStages; ++s) {
+        const double r = A.lring[((size_t)nm * kStages + s) * I.P + j];
+        sR[s][lane] = r;
+        rmax = max(rmax, __double2hiint(r) & 0x7fffffff);
+        if (own && I.R > 1) A.lring[((size_t)nx * kStages + s) * I.P + j] = 0.0;
+      }
+    }
+  }
+
+  // the scales: of the adjoint (every non-zero element near the warp's largest, as in the
+  // forward step), and of the stage inputs (2^E, which enter as factors of w)
+  int hw = 0, hv = 0;
+  unsigned lo = 0;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    hw = max(hw, __double2hiint(wd[i]) & 0x7fffffff);
+    lo |= (unsigned)__double2loint(wd[i]);
+#pragma unroll
+    for (int s = 0; s < kStages; ++s) hv = max(hv, __double2hiint(yd[s][i]) & 0x7fffffff);
+  }
+  const int bw = __reduce_max_sync(full, hw) >> 20, bv = __reduce_max_sync(full, hv) >> 20;
+  const int Ew = bw - 1022, E = bv - 1022;
+  const int d0 = -(I.bf.sc + E + 1) - 2;   // (2 P + P') -> units of w
+  bool bad = bw < kBfMinE || bw > kBfMaxE || bv < kBfMinE || bv > kBfMaxE || d0 < -3 || !I.bf.ok;
+  bad = bad || (hw ? (hw >> 20) < bw - kBfSpan : lo != 0);
+  // ring entries below 2^60 in units of mu
+  if (FACES) bad = bad || (rmax >> 20) > I.bf.sc + Ew + 1025;
+
+  if (!__any_sync(full, bad)) {
+    const BurgersFixed &B = I.bf;
+    const int smu = I.bf.sc + Ew - 57;   // unit of the flux adjoints
+    const int d = d0 > 60 ? 60 : d0;
+    const long long half = d > 0 ? 1ll << (d - 1) : 0;
+    long long w[NP], acc[NP];
+    double post[kStages];   // beta mu of a PE face's stages (FP64), posted once the step holds
+#pragma unroll
+    for (int i = 0; i < NP; ++i) w[i] = bf_from(wd[i], bw);
+    unsigned long long mag = 0;
+    // x / 3 for |x| < 2^60
+    auto third = [](long long x) {
+      int h, l;
+      fx_split(x, h, l);
+      FxAcc t;
+      fx_mac(t, make_int2(kThirdHi, kThirdLo), h, l);
+      return fx_round(t);
+    };
+    // x y 2^-58 for |x|, |y| < 2^60, from the limbs of both
+    auto mul = [](int xh, int xl, int yh, int yl) {
+      return fx_mul(xh, yh) + ((fx_mul(xh, yl) + fx_mul(xl, yh)) >> 29);
+    };
+#pragma unroll
+    for (int s = kStages - 1; s >= 0; --s) {
+      long long v[NP];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) v[i] = bf_from(yd[s][i], bv);
+      int th[HP ? HP : 1], tl[HP ? HP : 1], sh[HP + MID], sl[HP + MID];
+#pragma unroll
+      for (int i = 0; i < HP; ++i) {
+        fx_split(w[i] - w[NP - 1 - i], th[i], tl[i]);
+        fx_split(w[i] + w[NP - 1 - i], sh[i], sl[i]);
+      }
+      if (MID) fx_split(w[HP], sh[HP], sl[HP]);
+      // a . w = ev + od, b . w = od - ev
+      FxAcc ae, ao;
+#pragma unroll
+      for (int i = 0; i < HP + MID; ++i) fx_mac(ae, B.S[i][HP], sh[i], sl[i]);
+#pragma unroll
+      for (int i = 0; i < HP; ++i) fx_mac(ao, B.D[i][HP + MID], th[i], tl[i]);
+      const long long ev = fx_round(ae), od = fx_round(ao);
+      long long mu = ev + od + __shfl_up_sync(full, od - ev, 1);
+      long long dl, dr;
+      bf_llf_partials2(__shfl_up_sync(full, v[NP - 1], 1), v[0], dl, dr);
+      if (FACES && pe) {
+        const long long r = bf_from(sR[s][lane], B.sc + Ew + 1025) << 3;
+        mag |= fx_mag(mu) >> 4;   // below 2^62
+        const double m = bf_to(mu, smu);
+        post[s] = s == 2 ? m * (2.0 / 3.0) : (s == 1 ? 0.25 * m : m);
+        // the ring holds adjoints of the flux with beta: divided by it here
+        const long long rb = s == 2 ? r + (r >> 1) : (s == 1 ? 4 * r : r);
+        mu = k > 0 ? rb : mu + rb;
+      }
+      mag |= fx_mag(mu) >> 4;   // below 2^62
+      int mh, ml, xh, xl;
+      fx_split((mu + 4) >> 3, mh, ml);
+      fx_split(dl, xh, xl);
+      const long long pl = mul(mh, ml, xh, xl);
+      fx_split(dr, xh, xl);
+      const long long pr = mul(mh, ml, xh, xl);
+      const long long pR = __shfl_down_sync(full, pl, 1);
+#pragma unroll
+      for (int j = 0; j < HP + MID; ++j) {
+        // half the sum and half the difference of (W^T w)_j and (W^T w)_{p-j}
+        FxAcc a, b;
+#pragma unroll
+        for (int i = 0; i < HP; ++i) fx_mac(a, B.D[i][j], th[i], tl[i]);
+        const long long sum = fx_round(a);
+        long long dif = 0;
+        if (j < HP) {
+#pragma unroll
+          for (int i = 0; i < HP + MID; ++i) fx_mac(b, B.S[i][j], sh[i], sl[i]);
+          dif = fx_round(b);
+        }
+#pragma unroll
+        for (int m = 0; m < (j < HP ? 2 : 1); ++m) {
+          const int q = m ? NP - 1 - j : j;
+          int rh, rl, vh, vl;
+          fx_split(((m ? sum - dif : sum + dif) + 2) >> 2, rh, rl);
+          fx_split(v[q], vh, vl);
+          long long z = 2 * mul(rh, rl, vh, vl) + half;
+          if (q == 0) z += pr;
+          if (q == NP - 1) z += pR;
+          if (d < 0 && (fx_mag(z) >> (kBfTop + d))) mag |= 1ull << kBfTop;
+          const long long x = w[q] + bf_shift(z, d);
+          mag |= fx_mag(x);
+          if (s == 2) {
+            acc[q] = third(w[q]);
+            w[q] = third(2 * x);
+          } else if (s == 1) {
+            acc[q] += (3 * w[q] + 2) >> 2;
+            w[q] = (x + 2) >> 2;
+          } else {
+            w[q] = x + acc[q];
+            mag |= fx_mag(w[q]);
+          }
+        }
+      }
+    }
+    if (!__any_sync(full, (mag >> kBfTop) != 0)) {
+      if (own) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) A.out[(size_t)i * K + e] = bf_to(w[i], Ew - 57);
+        if (FACES && pe) {
+#pragma unroll
+          for (int s = 0; s < kStages; ++s)
+            post_levels(I, A.lring, e / I.Kpe, nm, s, k, qe, c, post[s]);
+        }
+      }
+      return;
+    }
+  }
+  burgers_adj_fp64<NP, FACES>(I, A, warp, nm, sR, pe, k, qe, c);
+}
+
 // One-warp blocks while the mesh gives fewer than 16 warps per SM (they spread evenly).
 template <int NP>
 cudaError_t burgers_np(const Inst &I, const double *uin, double *uout, double *r1, double *r2,
@@ -253,7 +550,30 @@ cudaError_t burgers_np(const Inst &I, const double *uin, double *uout, double *r
   return I.async ? go(k_burgers_step<NP, true, false>) : go(k_burgers_step<NP, false, false>);
 }
 
+template <int NP>
+cudaError_t burgers_adj_np(const Inst &I, const AdjArgs &A, cudaStream_t s) {
+  const int64_t warps = ((int64_t)I.K + kOwn - 1) / kOwn;
+  const int bs = warps < 16 * sm_count() ? 32 : 128;
+  const unsigned g = (unsigned)((warps * 32 + bs - 1) / bs);
+  if (I.async) k_burgers_adj<NP, true><<<g, bs, 0, s>>>(I, A);
+  else k_burgers_adj<NP, false><<<g, bs, 0, s>>>(I, A);
+  return cudaGetLastError();
+}
+
 }  // namespace
+
+cudaError_t launch_burgers_adj(const Inst &I, const double *y, const double *w, double *out,
+                               double *lring, int rel, cudaStream_t s) {
+  if (w == out) return cudaErrorInvalidValue;
+  const AdjArgs A{y, w, out, lring, rel};
+  switch (I.Np) {
+    case 2: return burgers_adj_np<2>(I, A, s);
+    case 3: return burgers_adj_np<3>(I, A, s);
+    case 4: return burgers_adj_np<4>(I, A, s);
+    case 5: return burgers_adj_np<5>(I, A, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
 
 cudaError_t launch_burgers_step(const Inst &I, const double *uin, double *uout, double *r1,
                                 double *r2, int rel, cudaStream_t s, bool pdl) {

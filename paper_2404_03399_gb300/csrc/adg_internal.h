@@ -181,13 +181,12 @@ static_assert(sizeof(Inst) % 16 == 0, "Inst is copied to shared memory as int4")
 // stage an Inst in shared memory.
 static_assert(sizeof(Inst) <= 8192, "Inst is passed by value as a kernel parameter");
 
-// Adjoint of one stage (adg_adjoint.cu): w is the adjoint of the stage output, v the stage
-// input (Burgers), lv receives the adjoint of the stage input (stages 1, 2); lacc collects
+// Adjoint of one stage of advection (adg_adjoint.cu): w is the adjoint of the stage output, lv
+// receives the adjoint of the stage input (stages 1, 2); lacc collects
 // the adjoint of u^n (stage 2 starts it with alpha w, stage 1 adds alpha w, stage 0 adds the
 // adjoint of its input u^n).
 struct AdjStage {
   const double *w;
-  const double *v;
   double *lv;
   double *lacc;
   int K, Np;
@@ -206,7 +205,6 @@ struct AdjStage {
 // coef, P, q, R) let the delay lookup serve both.
 struct AdjFace {
   const double *w;
-  const double *v;
   double *target;       // adjoint of the stage input (lacc for stage 0)
   double *lring;        // [R][3][P] adjoint of the face values of each stored level
   const uint8_t *table;
@@ -226,6 +224,11 @@ cudaError_t launch_stage(const Inst &I, int stage, int rel, cudaStream_t s, bool
 // neither) receive the inputs of stages 1 and 2.
 cudaError_t launch_burgers_step(const Inst &I, const double *uin, double *uout, double *r1,
                                 double *r2, int rel, cudaStream_t s, bool pdl = false);
+// Its adjoint: from the recorded stage inputs y (u, v1, v2 one after another) of step
+// meta[0] + rel and the adjoint w of its result, the adjoint of its input into out, with the
+// adjoint ring lring [R][3][P] at PE faces.
+cudaError_t launch_burgers_adj(const Inst &I, const double *y, const double *w, double *out,
+                               double *lring, int rel, cudaStream_t s);
 // Stage s of a 2N low-storage step (I.ls): dU_s = A_s dU_{s-1} + dt L(U_{s-1}) in place in
 // I.v1 (A_1 = 0: dU_0 is not read) and U_s = U_{s-1} + B_s dU_s from uin (U_{s-1}) into uout,
 // with the delayed / AT flux and the ring write of the stage-input traces at PE faces.
@@ -396,8 +399,8 @@ cudaError_t launch_reduce(int kind, const double *u, const double *g, int K, int
 int reduce_blocks(int K);
 
 // Adjoint launchers (adg_adjoint.cu); dir is the sign of the advection speed.
-cudaError_t launch_adj_stage(const AdjStage &A, int pde, int stage, int dir, cudaStream_t s);
-cudaError_t launch_adj_faces(const AdjFace &F, int pde, int dir, cudaStream_t s);
+cudaError_t launch_adj_stage(const AdjStage &A, int stage, int dir, cudaStream_t s);
+cudaError_t launch_adj_faces(const AdjFace &F, int dir, cudaStream_t s);
 cudaError_t launch_adj_init(const double *u, const double *g, int K, int Np, const double *M,
                             double scale, double *lam, cudaStream_t s);
 
