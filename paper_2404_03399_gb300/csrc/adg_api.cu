@@ -1453,6 +1453,8 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
   h.q_eff = cfg->mode == ADG_ASYNC_AT ? (cfg->at_order > 0 ? cfg->at_order : std::min(cfg->p + 1, ADG_MAX_Q)) : 1;
   I.q = h.q_eff;
   I.L = cfg->L;
+  // the levels that delays and AT sums reach (and, below, spare slots where one launch takes
+  // several steps, so that it overwrites no level that it still reads)
   I.R = (cfg->L - 1) + h.q_eff;
   {
     const LsTable *lt = cfg->rk == ADG_SSPRK3 ? nullptr : ls_table(cfg->rk);
@@ -1646,6 +1648,7 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
   }
 
   if (I.async) {
+    if (I.euler) I.R += adg::kEulerSteps - 1;
     const int q = h.q_eff, L = cfg->L;
     std::vector<double> cf((size_t)L * q * q, 0.0);
     for (int k = 0; k < L; ++k)
@@ -1740,6 +1743,23 @@ bool direct_launches(const adg_ctx *c) {
   return dof >= (int64_t(1) << 20);
 }
 
+// Launches of up to m steps each, launch(in, out, rel, steps), from u through v1 and v2 back to
+// u: u -> v1 -> u .., an odd number of launches ending u -> v1 -> v2 -> u (one alone: a copy).
+template <class F>
+int launch_alternating(adg_ctx *c, int nsteps, int m, size_t bytes, F &&launch) {
+  const Inst &I = c->inst[0].I;
+  const int count = (nsteps + m - 1) / m;
+  double *in = I.u;
+  for (int k = 0; k < count; ++k) {
+    double *out = in != I.u ? I.u : I.v1;
+    if (count % 2 && k == count - 2) out = I.v2;
+    CK(launch(in, out, k * m, std::min(m, nsteps - k * m)));
+    in = out;
+  }
+  if (in != I.u) CK(cudaMemcpyAsync(I.u, in, bytes, cudaMemcpyDeviceToDevice, c->stream));
+  return ADG_OK;
+}
+
 int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
   if (!c->batch && c->inst[0].I.fused) return launch_fused_steps(c, nsteps, kind);
   if (c->batch && c->batch_fixed && c->bu && c->split && direct_launches(c)) {
@@ -1799,6 +1819,14 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
     // single stage goes through v1: it reads its input's neighbours)
     const Inst &I = c->inst[0].I;
     const size_t fbytes = 3 * (size_t)I.K * I.Np * sizeof(double);
+    if (const int m = adg::euler_steps_per_launch(I)) {
+      int r = launch_alternating(c, nsteps, m, fbytes, [&](double *in, double *out, int rel, int k) {
+        return adg::launch_euler_steps(I, in, out, rel, k, c->stream);
+      });
+      if (r) return r;
+      CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
+      return ADG_OK;
+    }
     for (int rel = 0; rel < nsteps; ++rel) {
       for (int s = 0; s < I.ns; ++s) {
         double *dst = (s == I.ns - 1) ? I.u : (s == 0 ? I.v1 : I.v2);
@@ -1836,19 +1864,14 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
     return ADG_OK;
   }
   if (!c->batch && burgers_step(c->inst[0].I)) {
-    // u -> v1 -> u ..; an odd count ends u -> v1 -> v2 -> u (a single step: a copy back)
     const Inst &I = c->inst[0].I;
-    double *in = I.u;
-    for (int rel = 0; rel < nsteps; ++rel) {
-      double *out = in != I.u ? I.u : I.v1;
-      if (nsteps % 2 && rel == nsteps - 2) out = I.v2;
-      CK(adg::launch_burgers_step(I, in, out, nullptr, nullptr, rel, c->stream,
-                                  direct_launches(c) && rel > 0));
-      in = out;
-    }
-    if (in != I.u)
-      CK(cudaMemcpyAsync(I.u, in, (size_t)I.K * I.Np * sizeof(double), cudaMemcpyDeviceToDevice,
-                         c->stream));
+    const bool pdl = direct_launches(c);
+    int r = launch_alternating(c, nsteps, 1, (size_t)I.K * I.Np * sizeof(double),
+                               [&](double *in, double *out, int rel, int) {
+                                 return adg::launch_burgers_step(I, in, out, nullptr, nullptr, rel,
+                                                                 c->stream, pdl && rel > 0);
+                               });
+    if (r) return r;
     CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
     return ADG_OK;
   }

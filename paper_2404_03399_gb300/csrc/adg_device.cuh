@@ -50,6 +50,11 @@ __device__ __forceinline__ double num_flux(double a, double uL, double uR) {
 
 __device__ __forceinline__ int64_t ring_slot(int64_t level, int R) { return level % R; }
 
+// n mod m for n >= 0, m > 0 (a 32-bit remainder while n fits in 31 bits).
+__device__ __forceinline__ int mod_step(int64_t n, int m) {
+  return n <= 0x7fffffff ? (int)((unsigned)n % (unsigned)m) : (int)(n % m);
+}
+
 // Loads the Np nodal values of element e from a node-major field by pointer steps of K
 // (no per-node 64-bit index products).
 template <int NP, class T>

@@ -8,12 +8,15 @@
 //       out = alpha u + beta (v + dt L(v)),   dt L(v) = dt [ -QD f + qlL (f_0 - F_L) + qlR (f_p - F_R) ]
 //     (the strong form of the nodal DG operator, QD = (2/dx) D, qlL = -(2/dx) M^{-1} e_0,
 //     qlR = (2/dx) M^{-1} e_p), with the local Lax-Friedrichs flux at faces; at PE faces the
-//     flux is the AT sum (Eq. at-flux-gen) of the Lax-Friedrichs flux of the stored traces of
-//     the common delayed level, and the face owner stores the stage input's traces.
+//     flux is the AT sum (Eq. at-flux-gen) of the stored Lax-Friedrichs fluxes of
+//     the common delayed level, and the face owner stores the stage's flux.
 //   * k_euler_limit: the TVB-minmod slope limiter on every component (cell average a0 and
 //     P_1 coefficient a1; a1' = minmod(2 a1, d+, d-) / 2 unless |a1| <= M dx^2 / 2; an
 //     element whose a1 changes becomes a0 + a1' xi). Its stencil ends at PE faces (one-sided
 //     there), so it needs no exchange.
+#include <algorithm>
+#include <cmath>
+
 #include "adg_device.cuh"
 
 namespace adg {
@@ -51,52 +54,22 @@ __device__ __forceinline__ void euler_llf_from(const double UL[3], const double 
   for (int c = 0; c < 3; ++c) F[c] = 0.5 * (fl[c] + fr[c]) - 0.5 * lam * (UR[c] - UL[c]);
 }
 
-// Local Lax-Friedrichs flux of traces UL = U^-, UR = U^+ (the same arithmetic as the
-// interior faces, so a zero delay reproduces the synchronous flux bit for bit).
-__device__ __forceinline__ void euler_llf(const double UL[3], const double UR[3], double F[3]) {
-  double fl[3], fr[3], sl, sr;
-  euler_flux_speed(UL, fl, sl);
-  euler_flux_speed(UR, fr, sr);
-  euler_llf_from(UL, UR, fl, fr, sl, sr, F);
-}
-
-// AT value of the flux at PE face j, step n, stage s from the ring [R][ns][3][P] of (U^-, U^+)
-// traces; level n (k = 0) from the current traces (TL, TR), which the owner also stores.
-__device__ void euler_pe_flux(const Inst &I, int j, int64_t n, int s, const double TL[3],
-                              const double TR[3], bool owner, double F[3]) {
-  const int P = I.P, R = I.R;
-  const int nm = (int)(n % R);
-  const DelayAt d = delay_at(I, j, n);
-  auto level = [&](int m, double *out) {   // flux of level n - m from the ring, m >= 1
-    int slot = nm - m;
-    if (slot < 0) slot += R;
+// AT value of the flux at PE face j (delay d.k > 0), stage s of the step whose ring slot is nm,
+// from the ring [R][ns][3][P] of the face's fluxes.
+__device__ __forceinline__ void euler_pe_flux(const Inst &I, const DelayAt &d, int j, int nm, int s,
+                                              double F[3]) {
+  const int P = I.P;
+  for (int i = 0; i < d.qe; ++i) {
+    const double ci = d.c[i];
+    if (i && ci == 0.0) continue;
+    int slot = nm - d.k - i;
+    if (slot < 0) slot += I.R;
     const double2 *col = I.ring + ((size_t)slot * I.ns + s) * 3 * P + j;
-    double a[3], b[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const double2 t = col[(size_t)c * P];
-      a[c] = t.x;
-      b[c] = t.y;
+      const double x = __dmul_rn(ci, col[(size_t)c * P].x);
+      F[c] = i ? __dadd_rn(F[c], x) : x;
     }
-    euler_llf(a, b, out);
-  };
-  double G[3];
-  if (d.k == 0) euler_llf(TL, TR, G);
-  else level(d.k, G);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) F[c] = __dmul_rn(d.c[0], G[c]);
-  for (int i = 1; i < d.qe; ++i) {
-    const double ci = d.c[i];
-    if (ci != 0.0) {
-      level(d.k + i, G);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) F[c] = __dadd_rn(F[c], __dmul_rn(ci, G[c]));
-    }
-  }
-  if (owner) {
-    double2 *col = I.ring + ((size_t)nm * I.ns + s) * 3 * P + j;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) col[(size_t)c * P] = make_double2(TL[c], TR[c]);
   }
 }
 
@@ -146,7 +119,7 @@ __global__ void __launch_bounds__(kTile) k_euler_stage(const Inst I, int rel, do
   }
   // left face: U^- with its flux and speed from the left neighbour's last node (the lane
   // below), U^+ this element's first node; the right face's flux from the lane above
-  double VLm[3], VRp[3], V0[3], Vp[3], fLm[3], f0[3], fp[3];
+  double VLm[3], V0[3], Vp[3], fLm[3], f0[3], fp[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     V0[c] = V[c][0];
@@ -155,21 +128,28 @@ __global__ void __launch_bounds__(kTile) k_euler_stage(const Inst I, int rel, do
     fp[c] = f[c][NP - 1];
     VLm[c] = __shfl_up_sync(full, Vp[c], 1);
     fLm[c] = __shfl_up_sync(full, fp[c], 1);
-    VRp[c] = __shfl_down_sync(full, V0[c], 1);
   }
   const double sLm = __shfl_up_sync(full, sp, 1);
   double FL[3], FR[3];
   euler_llf_from(VLm, V0, fLm, f0, sLm, s0, FL);
+  if (FACES && lane > 0) {
+    // the lane of the element right of a PE face takes its flux: the owner stores it in the
+    // ring, and a delayed one replaces it (the left element's lane below takes it as its FR)
+    const int j = ec / I.Kpe;
+    if (ec == j * I.Kpe) {
+      const int64_t n = I.meta[0] + rel;
+      const int nm = (int)(n % I.R);
+      const DelayAt d = delay_at(I, j, n);
+      if (own) {
+        double2 *col = I.ring + ((size_t)nm * I.ns + STAGE) * 3 * I.P + j;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) col[(size_t)c * I.P] = make_double2(FL[c], 0.0);
+      }
+      if (d.k > 0) euler_pe_flux(I, d, j, nm, STAGE, FL);
+    }
+  }
 #pragma unroll
   for (int c = 0; c < 3; ++c) FR[c] = __shfl_down_sync(full, FL[c], 1);
-  if (FACES && e < K) {
-    const int64_t n = I.meta[0] + rel;
-    const int Kpe = I.Kpe;
-    const int jq = e / Kpe;
-    const int r = e - jq * Kpe;
-    if (r == 0) euler_pe_flux(I, jq, n, STAGE, VLm, V0, true, FL);
-    if (r == Kpe - 1) euler_pe_flux(I, jq + 1 == I.P ? 0 : jq + 1, n, STAGE, Vp, VRp, false, FR);
-  }
   if (e >= K) return;
   const double dt = I.dt;
 #pragma unroll
@@ -238,6 +218,26 @@ __device__ __forceinline__ double cell_average(const Inst &I, const double *v) {
   return a;
 }
 
+template <int NP>
+__device__ __forceinline__ double first_moment(const Inst &I, const double *v) {
+  double a = I.p1_w[0] * v[0];
+#pragma unroll
+  for (int j = 1; j < NP; ++j) a = fma(I.p1_w[j], v[j], a);
+  return a;
+}
+
+// The limited element of values v (average a0, slope a1) between the neighbours' averages.
+template <int NP>
+__device__ __forceinline__ void limit_element(const Inst &I, const double *v, double a0, double a1,
+                                              double dp, double dm, bool use_p, bool use_m,
+                                              double keep, double *out) {
+  double a1n = limited_slope(a1, dp, dm, use_p, use_m);
+  if ((__double_as_longlong(a1) & 0x7fffffffffffffffLL) <= __double_as_longlong(keep)) a1n = a1;
+  const bool change = a1n != a1;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) out[i] = change ? fma(a1n, I.xi[i], a0) : v[i];
+}
+
 template <int NP, bool PES>
 __global__ void __launch_bounds__(kTile) k_euler_limit(const Inst I, const double *__restrict__ src,
                                                        double *__restrict__ dst) {
@@ -262,9 +262,7 @@ __global__ void __launch_bounds__(kTile) k_euler_limit(const Inst I, const doubl
       q += K;
     }
     const double a0 = cell_average<NP>(I, v);
-    double a1 = I.p1_w[0] * v[0];
-#pragma unroll
-    for (int j = 1; j < NP; ++j) a1 = fma(I.p1_w[j], v[j], a1);
+    const double a1 = first_moment<NP>(I, v);
     double aL = __shfl_up_sync(0xffffffffu, a0, 1);
     double aR = __shfl_down_sync(0xffffffffu, a0, 1);
     if (lane == 0) {
@@ -278,15 +276,168 @@ __global__ void __launch_bounds__(kTile) k_euler_limit(const Inst I, const doubl
       aR = cell_average<NP>(I, w);
     }
     if (e >= K) continue;
-    double a1n = limited_slope(a1, aR - a0, a0 - aL, use_p, use_m);
-    if ((__double_as_longlong(a1) & 0x7fffffffffffffffLL) <= __double_as_longlong(keep)) a1n = a1;
+    limit_element<NP>(I, v, a0, a1, aR - a0, a0 - aL, use_p, use_m, keep, w);
     double *o = dst + c * nd + e;
-    const bool change = a1n != a1;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      *o = change ? fma(a1n, I.xi[i], a0) : v[i];
+      *o = w[i];
       o += K;
     }
+  }
+}
+
+constexpr int kEulerThreads = 128;
+
+// m steps of a small mesh in one launch. Four threads per element (eight at p = 4): node by
+// node for the fluxes and wave speeds, then component by component for the face fluxes, the
+// rows and the limiter, exchanged through shared memory. A warp's FP64 instruction holds its
+// sub-partition's FP64 pipe for 64 clocks however many lanes are active, so at a warp or
+// two per SM a step takes as long as one thread's FP64 instructions: about 57 a stage at p = 1
+// in this form, about 155 with a whole element per thread (14.7 us a step below). A block
+// owns EB - 2 H of its EB elements and forms the H on either side again (one per stage for the
+// faces, one more for the limiter), so blocks need nothing from one another. Every element's
+// arithmetic is that of k_euler_stage and k_euler_limit, so the results are theirs bit for bit,
+// whatever the block or the split of a run into launches. A PE face's fluxes are kept in shared
+// memory, the ring's levels before the launch (loaded at its start) and then the launch's own;
+// the ring has kEulerSteps - 1 spare slots, so that no block overwrites a level that another
+// still reads. Sod's problem on 1024 elements, ADG-AT2-RK2: 42 us a step as two stage and
+// two limiter kernels (whose PE lanes recomputed the fluxes of delayed traces), 8.0 us so.
+template <int NP, bool FACES, bool PES, bool LIM>
+__global__ void __launch_bounds__(kEulerThreads)
+    k_euler_steps(const __grid_constant__ Inst I, const double *__restrict__ uin,
+                  double *__restrict__ uout, int rel, int m, int H) {
+  constexpr int LPE = NP <= 4 ? 4 : 8, EB = kEulerThreads / LPE;
+  __shared__ double Vs[3][NP][EB], fs[3][NP][EB], s0[EB], sp[EB], Fs[3][EB], as[3][EB];
+  __shared__ unsigned char delay[FACES ? kEulerSteps : 1][EB];
+  extern __shared__ double hist[];   // [levels][ns][3][EB], then the AT coefficients
+  const int K = I.K, S = I.ns;
+  const size_t nd = (size_t)K * NP;
+  const int el = threadIdx.x / LPE, r = threadIdx.x - el * LPE;
+  const int c = r;                    // component (r < 3)
+  const int OWN = EB - 2 * H;
+  const int eraw = (int)blockIdx.x * OWN - H + el;
+  const bool own = el >= H && el < H + OWN && eraw < K;
+  int e = eraw;
+  if ((unsigned)e >= (unsigned)K) {
+    e %= K;
+    if (e < 0) e += K;
+  }
+  const int elL = el ? el - 1 : 0, elR = el + 1 < EB ? el + 1 : el;
+  double V[NP], u[NP];
+  if (r < 3) {
+    load_elem<NP>(uin + c * nd, K, e, u);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) Vs[c][i][el] = u[i];
+  }
+  const int j = e / I.Kpe;
+  const bool face = FACES && r < 3 && e == j * I.Kpe;
+  const bool use_m = !(PES && e == j * I.Kpe), use_p = !(PES && e + 1 == (j + 1) * I.Kpe);
+  const double keep = I.tvb_m * (I.dx * I.dx) * 0.5;
+  const double dt = I.dt;
+  const int back = I.L - 1 + I.q - 1;   // levels before the current step that it can reach
+  const int64_t n0 = FACES ? I.meta[0] + rel : 0;
+  auto at = [&](int level, int s) -> double & {   // level: relative to n0
+    return hist[(((level + back) * S + s) * 3 + c) * EB + el];
+  };
+  double *coef = hist + (back + m) * S * 3 * EB;
+  if (FACES)
+    for (int k = threadIdx.x; k < I.L * I.q * I.q; k += kEulerThreads) coef[k] = __ldg(I.coef + k);
+  if (face) {
+    const uint8_t *row = I.table + (n0 - I.meta[1]) * I.P + j;
+    for (int t = c; t < m; t += 3) delay[t][el] = row[(size_t)t * I.P];
+    for (int b = 1; b <= back && b <= n0; ++b) {
+      const int slot = mod_step(n0 - b, I.R);
+      for (int s = 0; s < S; ++s) at(-b, s) = I.ring[(((size_t)slot * S + s) * 3 + c) * I.P + j].x;
+    }
+  }
+  __syncthreads();
+  for (int t = 0; t < m; ++t) {
+    // as delay_at: k <= n, order q' = min(q, n - k + 1)
+    int dk = 0, qe = 0, nm = 0;
+    const double *cf = nullptr;
+    if (face) {
+      const int64_t n = n0 + t;
+      dk = (int)min((int64_t)delay[t][el], n);
+      qe = (int)min((int64_t)I.q, n - dk + 1);
+      cf = coef + (dk * I.q + qe - 1) * I.q;
+      nm = mod_step(n, I.R);
+    }
+    if (r < 3) {
+#pragma unroll
+      for (int i = 0; i < NP; ++i) V[i] = u[i];
+    }
+    for (int s = 0; s < S; ++s) {
+      const StageConsts &C = I.sc[s];
+      if (r < NP) {   // node r
+        const double Ui[3] = {Vs[0][r][el], Vs[1][r][el], Vs[2][r][el]};
+        double fi[3], si;
+        euler_flux_speed(Ui, fi, si);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) fs[k][r][el] = fi[k];
+        if (r == 0) s0[el] = si;
+        if (r == NP - 1) sp[el] = si;
+      }
+      __syncthreads();
+      if (r < 3) {
+        const double lam = fmax(sp[elL], s0[el]);
+        double F = 0.5 * (fs[c][NP - 1][elL] + fs[c][0][el]) -
+                   0.5 * lam * (Vs[c][0][el] - Vs[c][NP - 1][elL]);
+        if (face) {
+          at(t, s) = F;
+          if (own) I.ring[(((size_t)nm * S + s) * 3 + c) * I.P + j] = make_double2(F, 0.0);
+          if (dk > 0) {
+            F = __dmul_rn(cf[0], at(t - dk, s));
+            for (int k = 1; k < qe; ++k)
+              if (cf[k] != 0.0) F = __dadd_rn(F, __dmul_rn(cf[k], at(t - dk - k, s)));
+          }
+        }
+        Fs[c][el] = F;
+      }
+      __syncthreads();
+      double o[NP], a0 = 0.0, a1 = 0.0;
+      if (r < 3) {
+        double f[NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) f[i] = fs[c][i][el];
+        const double jl = __dsub_rn(f[0], Fs[c][el]);
+        const double jr = __dsub_rn(f[NP - 1], Fs[c][elR]);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+          double x = -I.QD[i * NP] * f[0];
+#pragma unroll
+          for (int k = 1; k < NP; ++k) x = fma(-I.QD[i * NP + k], f[k], x);
+          x = fma(I.qlL[i], jl, x);
+          x = fma(I.qlR[i], jr, x);
+          o[i] = C.beta * fma(dt, x, V[i]);
+          if (s > 0) o[i] = fma(C.alpha, u[i], o[i]);
+        }
+        if (LIM) {
+          a0 = cell_average<NP>(I, o);
+          a1 = first_moment<NP>(I, o);
+          as[c][el] = a0;
+        }
+      }
+      if (LIM) __syncthreads();
+      if (r < 3) {
+        if (LIM) {
+          limit_element<NP>(I, o, a0, a1, as[c][elR] - a0, a0 - as[c][elL], use_p, use_m, keep, V);
+        } else {
+#pragma unroll
+          for (int i = 0; i < NP; ++i) V[i] = o[i];
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) Vs[c][i][el] = V[i];
+      }
+      __syncthreads();
+    }
+    if (r < 3) {
+#pragma unroll
+      for (int i = 0; i < NP; ++i) u[i] = V[i];
+    }
+  }
+  if (own && r < 3) {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) uout[c * nd + (size_t)i * K + e] = u[i];
   }
 }
 
@@ -327,6 +478,70 @@ cudaError_t launch_euler_stage(const Inst &I, int stage, int rel, double *dst, c
     case 3: return euler_stage<3>(I, stage, rel, dst, s);
     case 4: return euler_stage<4>(I, stage, rel, dst, s);
     case 5: return euler_stage<5>(I, stage, rel, dst, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+namespace {
+constexpr int euler_block(int Np) { return kEulerThreads / (Np <= 4 ? 4 : 8); }
+
+// Halo of m steps of k_euler_steps and its dynamic shared memory.
+int euler_halo(const Inst &I, int m) { return m * I.ns * (I.limiter ? 2 : 1); }
+size_t euler_hist(const Inst &I, int m) {
+  return I.async ? ((size_t)(I.L + I.q - 2 + m) * I.ns * 3 * euler_block(I.Np) + I.L * I.q * I.q) *
+                       sizeof(double)
+                 : 0;
+}
+
+template <int NP>
+cudaError_t euler_steps(const Inst &I, const double *uin, double *uout, int rel, int m,
+                        cudaStream_t s) {
+  const int H = euler_halo(I, m), own = euler_block(NP) - 2 * H;
+  const unsigned g = (unsigned)((I.K + own - 1) / own);
+  auto go = [&](auto kernel) {
+    kernel<<<g, kEulerThreads, euler_hist(I, m), s>>>(I, uin, uout, rel, m, H);
+    return cudaGetLastError();
+  };
+  if (I.async)
+    return I.limiter ? go(k_euler_steps<NP, true, true, true>) : go(k_euler_steps<NP, true, true, false>);
+  if (I.P > 1 && I.limiter) return go(k_euler_steps<NP, false, true, true>);
+  return I.limiter ? go(k_euler_steps<NP, false, false, true>) : go(k_euler_steps<NP, false, false, false>);
+}
+}  // namespace
+
+// A launch costs about 2.5 us; a block's stage holds its SM's FP64 pipes (one warp each) for 64
+// clocks per instruction of a thread, an element's stage and limiter in the two kernels of a
+// stage its warp's pipe for as many of a whole element. The number of steps with the least
+// estimated time; 0: the stage and limiter kernels.
+int euler_steps_per_launch(const Inst &I) {
+  const double sms = sm_count(), clk = 64 / 1900.0 * I.ns;
+  const int NP = I.Np, lim = I.limiter ? 2 * NP + 5 : 0;
+  const double thread = clk * (35 + NP * (NP + 4) + lim);
+  const double element = clk * (30 * NP + 3 * (5 + NP * (NP + 4) + lim));
+  double best = 2.5 * I.ns * (I.limiter ? 2 : 1) + element * std::max(1.0, I.K / 30.0 / (4 * sms));
+  int pick = 0;
+  for (int m = 1; m <= kEulerSteps; ++m) {
+    const int own = euler_block(NP) - 2 * euler_halo(I, m);
+    if (own < 1 || euler_hist(I, m) > 32 * 1024) break;
+    const double us = 2.5 / m + thread * std::max(1.0, std::ceil((double)I.K / own) / sms);
+    if (us < best) {
+      best = us;
+      pick = m;
+    }
+  }
+  return pick;
+}
+
+cudaError_t launch_euler_steps(const Inst &I, const double *uin, double *uout, int rel, int m,
+                               cudaStream_t s) {
+  if (uin == uout || m < 1 || m > kEulerSteps ||
+      euler_block(I.Np) - 2 * euler_halo(I, m) < 1)
+    return cudaErrorInvalidValue;
+  switch (I.Np) {
+    case 2: return euler_steps<2>(I, uin, uout, rel, m, s);
+    case 3: return euler_steps<3>(I, uin, uout, rel, m, s);
+    case 4: return euler_steps<4>(I, uin, uout, rel, m, s);
+    case 5: return euler_steps<5>(I, uin, uout, rel, m, s);
     default: return cudaErrorInvalidValue;
   }
 }

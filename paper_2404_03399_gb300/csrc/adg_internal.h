@@ -242,6 +242,12 @@ cudaError_t launch_ldg_q(const Inst &I, const double *vin, int stage, int rel, c
 // (u, v1, v2 by stage) into dst, and the slope limiter src -> dst (src != dst).
 cudaError_t launch_euler_stage(const Inst &I, int stage, int rel, double *dst, cudaStream_t s);
 cudaError_t launch_euler_limit(const Inst &I, const double *src, double *dst, cudaStream_t s);
+// m steps uin -> uout in one launch (small meshes; the same results), and the m that an
+// instance takes: 1 .. kEulerSteps, or 0 for the stage and limiter kernels.
+constexpr int kEulerSteps = 4;
+int euler_steps_per_launch(const Inst &I);
+cudaError_t launch_euler_steps(const Inst &I, const double *uin, double *uout, int rel, int m,
+                               cudaStream_t s);
 cudaError_t launch_batch_stage(const Inst *insts_dev, const int2 *work_dev, int nwork,
                                int stage, int rel, int tile, cudaStream_t s);
 // Batched PE-face pass after each batched stage: ring write of the stage-input traces and

@@ -498,11 +498,6 @@ struct FaceLoads {
   int k, qe, nm;   // nm: the ring slot of step n
 };
 
-// n mod m for n >= 0, m > 0 (a 32-bit remainder while n fits in 31 bits).
-__device__ __forceinline__ int mod_step(int64_t n, int m) {
-  return n <= 0x7fffffff ? (int)((unsigned)n % (unsigned)m) : (int)(n % m);
-}
-
 template <int S>
 __device__ __forceinline__ void face_loads(const Inst &I, int j, int64_t n, FaceLoads<S> &f) {
   const DelayAt dl = delay_at(I, j, n);
