@@ -1649,6 +1649,7 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
 
   if (I.async) {
     if (I.euler) I.R += adg::kEulerSteps - 1;
+    if (I.pde == ADG_ADVECTION && !I.fused && !I.ls) I.R += adg::kAdvSteps - 1;
     const int q = h.q_eff, L = cfg->L;
     std::vector<double> cf((size_t)L * q * q, 0.0);
     for (int k = 0; k < L; ++k)
@@ -1870,6 +1871,16 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
                                [&](double *in, double *out, int rel, int) {
                                  return adg::launch_burgers_step(I, in, out, nullptr, nullptr, rel,
                                                                  c->stream, pdl && rel > 0);
+                               });
+    if (r) return r;
+    CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
+    return ADG_OK;
+  }
+  if (const int m = !c->batch && c->inst[0].I.pde == ADG_ADVECTION ? adg::adv_steps_per_launch(c->inst[0].I) : 0) {
+    const Inst &I = c->inst[0].I;
+    int r = launch_alternating(c, nsteps, m, (size_t)I.K * I.Np * sizeof(double),
+                               [&](double *in, double *out, int rel, int k) {
+                                 return adg::launch_adv_steps(I, in, out, rel, k, c->stream);
                                });
     if (r) return r;
     CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));

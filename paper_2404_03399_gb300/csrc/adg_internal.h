@@ -219,6 +219,13 @@ struct AdjFace {
 // One stage over all elements; for an asynchronous instance the same kernel applies the
 // PE-face correction (delayed / AT flux) and writes the ring (step meta[0] + rel).
 cudaError_t launch_stage(const Inst &I, int stage, int rel, cudaStream_t s, bool pdl = false);
+// m staged SSP-RK3 steps of advection uin -> uout in one launch (adg_steps.cu; small meshes, the
+// same results as launch_stage), and the m that an instance takes: 1 .. kAdvSteps, or 0 for
+// the stage kernels.
+constexpr int kAdvSteps = 8;
+int adv_steps_per_launch(const Inst &I);
+cudaError_t launch_adv_steps(const Inst &I, const double *uin, double *uout, int rel, int m,
+                             cudaStream_t s);
 // One SSP-RK3 step of inviscid Burgers uin -> uout (adg_burgers.cu), with the delayed / AT
 // flux and the ring write (its entries hold the face's flux) at PE faces; r1, r2 (both or
 // neither) receive the inputs of stages 1 and 2.
