@@ -349,8 +349,7 @@ struct InstHost {
   double *coef = nullptr;
   double *w = nullptr, *M = nullptr;
   int stages = 3;            // stages per step of the RK scheme (the ring may keep more slots)
-  double *qbuf = nullptr;    // viscous Burgers: q = u_x of the stage input
-  double *ringq = nullptr;   // ... and the PE faces' q^+ traces
+  double *ringq = nullptr;   // viscous Burgers: the PE faces' -2 nu q^+
   adg::FxSlot *fx = nullptr; // scale slots of the fixed-point composed step
   double *fd = nullptr;      // ... and its PE faces' stage differences [2][P][3]
   bool fixed_ok = false;     // the composed coefficients fit the fixed-point bounds
@@ -478,7 +477,7 @@ void fold_constants(InstHost &h) {
   }
 }
 
-// c 2^58 rounded, in limbs ch 2^29 + cl with balanced cl (|c| <= 1).
+// c 2^58 rounded, in limbs ch 2^29 + cl with balanced cl (|c| < 2).
 int2 limbs58(ld c) {
   const long long C = llrintl(c * 288230376151711744.0L);
   long long lo = C & 0x1FFFFFFF;
@@ -486,7 +485,8 @@ int2 limbs58(ld c) {
   return make_int2((int)((C - lo) >> 29), (int)lo);
 }
 
-// The Burgers operator on mirrored nodes (BurgersFixed) for the integer step.
+// The Burgers operator on mirrored nodes, the 2N coefficients and the viscosity (BurgersFixed)
+// for the integer step.
 void fold_burgers(InstHost &h) {
   const Ops &o = h.ops;
   const int Np = o.Np, p = Np - 1, H = Np / 2, mid = Np % 2;
@@ -520,7 +520,15 @@ void fold_burgers(InstHost &h) {
     for (int j = 0; j <= H; ++j) B.S[i][j] = limbs58(std::ldexp(S[i][j], -e));
   for (int i = 0; i < H; ++i)
     for (int j = 0; j <= H + mid; ++j) B.D[i][j] = limbs58(std::ldexp(D[i][j], -e));
-  B.ok = 1;
+  for (int s = 0; s < adg::kMaxStages; ++s) {
+    B.lsA[s] = limbs58(h.I.lsA[s]);
+    B.lsB[s] = limbs58(h.I.lsB[s]);
+  }
+  if (h.I.visc) {
+    const ld vn = std::frexp(2.0L * (ld)h.I.nu / (ld)h.dt, &B.sn);
+    B.vn = limbs58(vn);
+  }
+  B.ok = std::abs(B.sc) < 300 && std::abs(B.sn) < 300;   // far from the ends of FP64's range
 }
 
 // Composed step constants (StepConsts in adg_internal.h), built in long double from the
@@ -1376,9 +1384,6 @@ int reset_exponent(adg_ctx *c, InstHost &h, bool from_scan = false) {
   return ADG_OK;
 }
 
-// The instance takes k_burgers_step (inviscid Burgers, SSP-RK3).
-bool burgers_step(const Inst &I) { return I.pde == ADG_BURGERS && !I.visc && !I.ls; }
-
 // Elements per thread of the composed-step kernel. The FP64 composed step times one, two and
 // four on a copy of u0 held in the instance's v1/v2 fields (free at this point) and keeps the
 // fastest; the fixed-point step takes two for even K, which measured faster in every timing
@@ -1502,10 +1507,6 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
   }
 
   const size_t nd = (size_t)K * Np;
-  if (I.visc) {
-    CK(cudaMalloc(&h.qbuf, nd * sizeof(double)));
-    I.qbuf = h.qbuf;
-  }
   // u | v1 | v2 (| w: Euler's raw stage output under the limiter), ncomp components each
   const int ncomp = I.euler ? 3 : 1;
   const size_t fnd = ncomp * nd;
@@ -1581,7 +1582,7 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
   }
   I.dt = h.dt;
   fold_constants(h);
-  if (burgers_step(I)) fold_burgers(h);
+  if (I.pde == ADG_BURGERS) fold_burgers(h);
   if (I.euler) {
     const double so[3][3][2] = {{{0.0, 1.0}}, {{0.0, 1.0}, {0.5, 0.5}},
                                 {{0.0, 1.0}, {0.75, 0.25}, {1.0 / 3.0, 2.0 / 3.0}}};
@@ -1845,26 +1846,7 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
     CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
     return ADG_OK;
   }
-  if (!c->batch && c->inst[0].I.ls) {
-    // 2N low-storage step: U_0 = u, dU in v1, U_s alternately in v2 and u (each stage reads
-    // its input's neighbours, so it writes the other field); an odd stage count ends in v2
-    const Inst &I = c->inst[0].I;
-    for (int rel = 0; rel < nsteps; ++rel) {
-      const double *in = I.u;
-      for (int s = 0; s < I.ns; ++s) {
-        double *out = (s % 2 == 0) ? I.v2 : I.u;
-        if (I.visc) CK(adg::launch_ldg_q(I, in, s, rel, c->stream));
-        CK(adg::launch_lsrk_stage(I, s, rel, in, out, c->stream));
-        in = out;
-      }
-      if (I.ns % 2)
-        CK(cudaMemcpyAsync(I.u, I.v2, (size_t)I.K * I.Np * sizeof(double),
-                           cudaMemcpyDeviceToDevice, c->stream));
-    }
-    CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
-    return ADG_OK;
-  }
-  if (!c->batch && burgers_step(c->inst[0].I)) {
+  if (!c->batch && c->inst[0].I.pde == ADG_BURGERS) {
     const Inst &I = c->inst[0].I;
     const bool pdl = direct_launches(c);
     int r = launch_alternating(c, nsteps, 1, (size_t)I.K * I.Np * sizeof(double),
@@ -1873,6 +1855,24 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
                                                                  c->stream, pdl && rel > 0);
                                });
     if (r) return r;
+    CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
+    return ADG_OK;
+  }
+  if (!c->batch && c->inst[0].I.ls) {
+    // 2N low-storage step: U_0 = u, dU in v1, U_s alternately in v2 and u (each stage reads
+    // its input's neighbours, so it writes the other field); an odd stage count ends in v2
+    const Inst &I = c->inst[0].I;
+    for (int rel = 0; rel < nsteps; ++rel) {
+      const double *in = I.u;
+      for (int s = 0; s < I.ns; ++s) {
+        double *out = (s % 2 == 0) ? I.v2 : I.u;
+        CK(adg::launch_lsrk_stage(I, s, rel, in, out, c->stream));
+        in = out;
+      }
+      if (I.ns % 2)
+        CK(cudaMemcpyAsync(I.u, I.v2, (size_t)I.K * I.Np * sizeof(double),
+                           cudaMemcpyDeviceToDevice, c->stream));
+    }
     CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
     return ADG_OK;
   }
@@ -1894,13 +1894,10 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
           CK(adg::launch_batch_faces(c->insts_dev, c->fwork_dev, c->nfwork, s, rel, c->stream));
       } else {
         const Inst &I = c->inst[0].I;
-        if (I.visc) CK(adg::launch_ldg_q(I, s == 0 ? I.u : (s == 1 ? I.v1 : I.v2), s, rel, c->stream));
         // a programmatic dependent of the stage before it on runs launched without graphs
-        // (the first of the chunk follows other work; the viscous stage follows its q pass).
-        // Inside the graphs of small runs programmatic launches measured slower (the adjoint
-        // workload's forward 78 -> 95 ms), on the 2^20-element Burgers mesh 1.6% faster.
-        CK(adg::launch_stage(I, s, rel, c->stream,
-                             direct_launches(c) && !I.visc && (rel > 0 || s > 0)));
+        // (the first of the chunk follows other work; inside the graphs of small runs
+        // programmatic launches measured slower)
+        CK(adg::launch_stage(I, s, rel, c->stream, direct_launches(c) && (rel > 0 || s > 0)));
       }
     }
   }
@@ -2410,7 +2407,6 @@ void adg_destroy(adg_ctx *c) {
     cudaFree(h.M);
     cudaFree(h.fx);
     cudaFree(h.fd);
-    cudaFree(h.qbuf);
     cudaFree(h.ringq);
   }
   cudaFree(c->meta);

@@ -1,20 +1,21 @@
-// Inviscid Burgers, SSP-RK3: one kernel per step and one per step of its discrete adjoint,
-// the three stages in registers.
+// Burgers: one kernel per step (every RK scheme, inviscid or viscous) and one per step of the
+// discrete adjoint (inviscid, SSP-RK3), the stages in registers.
 #include "adg_bfp.cuh"
 #include "adg_device.cuh"
 
 namespace adg {
 namespace {
 
-constexpr int kHalo = 3;   // elements a step's stages read on either side (one per stage)
-
-// A warp's 32 consecutive elements: the first and last kHalo are the neighbours' (periodic),
-// formed again so that warps need nothing from one another. own: written by this warp.
+constexpr int kHalo = kStages;   // elements an SSP-RK3 step's stages read on either side
 constexpr int kOwn = 32 - 2 * kHalo;
 
-__device__ __forceinline__ int warp_element(int K, int warp, int lane, bool &own) {
-  int e = warp * kOwn - kHalo + lane;
-  own = lane >= kHalo && lane < kHalo + kOwn && e < K;
+// A warp's 32 consecutive elements: the first H and the last HR are the neighbours' (periodic),
+// formed again so that warps need nothing from one another: one on either side per stage (and
+// one more on the right for a delayed uhat at the last element's right face, viscous Burgers).
+// own: written by this warp.
+__device__ __forceinline__ int warp_element(int K, int warp, int lane, int H, int HR, bool &own) {
+  int e = warp * (32 - H - HR) - H + lane;
+  own = lane >= H && lane < 32 - HR && e < K;
   if ((unsigned)e >= (unsigned)K) {
     e %= K;
     if (e < 0) e += K;
@@ -22,114 +23,212 @@ __device__ __forceinline__ int warp_element(int K, int warp, int lane, bool &own
   return e;
 }
 
-// The delayed / AT flux of PE face j at stage s of step n (k = d.k > 0) from the ring, whose
-// entries hold the face's flux of each level.
-__device__ __forceinline__ double ring_flux(const Inst &I, const DelayAt &d, int j, int nm, int s) {
+// Face quantities of a stage with a delayed / AT value at PE faces: the flux, and for viscous
+// Burgers uhat = u^- and qhat = q^+ (kept as y = -2 nu q^+).
+template <bool VISC>
+constexpr int kFaceVals = VISC ? 3 : 1;
+
+// Value `which` of ring level n - m (slot sl): flux and u^- in I.ring, y in I.ringq.
+__device__ __forceinline__ double ring_value(const Inst &I, int which, int sl, int s, int j) {
+  const size_t at = ((size_t)sl * I.ns + s) * I.P + j;
+  return which == 0 ? I.ring[at].x : (which == 1 ? I.ring[at].y : I.ringq[at]);
+}
+
+// The delayed / AT value of PE face j at stage s (d.k > 0) from the ring.
+__device__ __forceinline__ double ring_sum(const Inst &I, const DelayAt &d, int which, int j, int nm,
+                                           int s) {
   double V = 0.0;
   for (int i = 0; i < d.qe; ++i) {
     int sl = nm - d.k - i;
     if (sl < 0) sl += I.R;
-    const double x = __dmul_rn(d.c[i], I.ring[((size_t)sl * kStages + s) * I.P + j].x);
+    const double x = __dmul_rn(d.c[i], ring_value(I, which, sl, s, j));
     V = i ? __dadd_rn(V, x) : x;
   }
   return V;
 }
 
-// The step in FP64 (warps that the integer path does not take): the stages of the staged
-// kernels, with the delayed fluxes sV[stage][lane] at PE faces (pe: the element's left face is
-// one; late: its flux is a delayed one).
-template <int NP, bool FACES, bool REC>
-__device__ __noinline__ void burgers_step_fp64(const Inst &I, int warp, const double *uin,
-                                               double *uout, double *r1, double *r2, int nm,
+// Fields of a step and what it writes besides.
+struct StepArgs {
+  const double *uin;
+  double *uout;
+  double *r1, *r2;   // REC: the inputs of stages 1 and 2
+  int rel, H, HR;
+};
+
+// The step in FP64 (warps that the integer path does not take): stage by stage in the staged
+// kernels' arithmetic, with the delayed values sV[value * ns + stage][lane] at PE faces (pe:
+// the element's left face is one; late: its values are delayed ones).
+template <int NP, bool FACES, bool REC, bool VISC, bool LS>
+__device__ __noinline__ void burgers_step_fp64(const Inst &I, const StepArgs &A, int warp, int nm,
                                                const double (*sV)[32], bool pe, bool late) {
-  const int K = I.K;
+  const int K = I.K, S = LS ? I.ns : kStages;
   const int lane = threadIdx.x & 31;
   bool own;
-  const int e = warp_element(K, warp, lane, own);
+  const int e = warp_element(K, warp, lane, A.H, A.HR, own);
   const unsigned full = 0xffffffffu;
-  double u[NP], v[NP];
-  load_elem<NP>(uin, K, e, u);
+  double u[NP], v[NP];   // u: u^n, or dU of a 2N scheme
+  load_elem<NP>(A.uin, K, e, v);
 #pragma unroll
-  for (int i = 0; i < NP; ++i) v[i] = u[i];
-#pragma unroll
-  for (int s = 0; s < kStages; ++s) {
-    const StageConsts &C = I.sc[s];
-    double FL = num_flux<1>(0.0, __shfl_up_sync(full, v[NP - 1], 1), v[0]);
+  for (int i = 0; i < NP; ++i) u[i] = LS ? 0.0 : v[i];
+  for (int s = 0; s < S; ++s) {
+    const StageConsts &C = I.sc[LS ? 0 : s];
+    const double vl = __shfl_up_sync(full, v[NP - 1], 1);
+    double FL = num_flux<1>(0.0, vl, v[0]);
+    const size_t at = FACES && pe ? ((size_t)nm * I.ns + s) * I.P + e / I.Kpe : 0;
     if (FACES && pe) {
-      if (own) I.ring[((size_t)nm * kStages + s) * I.P + e / I.Kpe] = make_double2(FL, 0.0);
+      if (own) I.ring[at] = make_double2(FL, vl);
       if (late) FL = sV[s][lane];
+    }
+    double q[NP], jqL = 0.0, jqR = 0.0;
+    if (VISC) {
+      const double uL = FACES && late ? sV[S + s][lane] : vl;
+      const double uN = __shfl_down_sync(full, uL, 1);
+      const double uR = FACES && lane < 31 ? uN : v[NP - 1];   // v_p but at delayed faces
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        double acc = I.QD[i * NP] * v[0];
+#pragma unroll
+        for (int k = 1; k < NP; ++k) acc = fma(I.QD[i * NP + k], v[k], acc);
+        acc = fma(I.qlL[i], uL - v[0], acc);
+        q[i] = fma(I.qlR[i], uR - v[NP - 1], acc);
+      }
+      double qL = q[0];
+      if (FACES && pe) {
+        if (own) I.ringq[at] = -2.0 * I.nu * q[0];
+        if (late) qL = sV[2 * S + s][lane] / (-2.0 * I.nu);
+      }
+      jqL = qL - q[0];
+      jqR = __shfl_down_sync(full, qL, 1) - q[NP - 1];
     }
     const double FR = __shfl_down_sync(full, FL, 1);
     const double jL = __dsub_rn(phys_flux<1>(0.0, v[0]), FL);
     const double jR = __dsub_rn(phys_flux<1>(0.0, v[NP - 1]), FR);
-    double g[NP];
+    double g[NP], out[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) g[i] = v[i] * v[i];
-    double *o = s == 2 ? uout : (REC ? (s == 0 ? r1 : r2) : nullptr);
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      double acc = s == 0 ? v[i] : fma(C.beta, v[i], C.alpha * u[i]);
+      double acc = LS ? I.lsA[s] * u[i] : (s == 0 ? v[i] : fma(C.beta, v[i], C.alpha * u[i]));
 #pragma unroll
       for (int k = 0; k < NP; ++k) acc = fma(C.A[i * NP + k], g[k], acc);
-      v[i] = fma(C.lR[i], jR, fma(C.lL[i], jL, acc));
+      acc = fma(C.lR[i], jR, fma(C.lL[i], jL, acc));
+      if (VISC) {
+        double vq = C.A[i * NP] * q[0];
+#pragma unroll
+        for (int k = 1; k < NP; ++k) vq = fma(C.A[i * NP + k], q[k], vq);
+        acc = fma(I.nu, fma(C.lL[i], jqL, fma(C.lR[i], jqR, -2.0 * vq)), acc);
+      }
+      out[i] = acc;
+    }
+    double *o = s == S - 1 ? A.uout : (REC ? (s == 0 ? A.r1 : A.r2) : nullptr);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      if (LS) {
+        u[i] = out[i];
+        v[i] = fma(I.lsB[s], out[i], v[i]);
+      } else {
+        v[i] = out[i];
+      }
       if (o && own) o[(size_t)i * K + e] = v[i];
     }
   }
 }
 
-// One SSP-RK3 step of inviscid Burgers. Warp w owns 26 elements and forms three more on
-// either side, so the three stages run in registers with shuffles for the face values and no
-// barrier, and u is read and written once per step (three launches and eight field passes
-// before). The stage operator
-//   dt L(v)_i = sum_j W_ij v_j^2 + a_i F_L + b_i F_R
+// The operator on mirrored nodes (BurgersFixed): sums of the rows i and p - i, odd[i] + even[i]
+// and odd[i] - even[i], of node values g (|g| < 2^59) and face values FL, FR (|.| < 2^59),
+// with `half` added to each (a rounding constant of the shift that follows).
+template <int NP>
+__device__ __forceinline__ void burgers_operator(const BurgersFixed &B, const long long *g,
+                                                 long long FL, long long FR, long long half,
+                                                 long long *out) {
+  constexpr int HP = NP / 2, MID = NP % 2;   // mirrored pairs, middle node
+  int dh[HP + 1], dl[HP + 1], sh[HP + MID + 1], sl[HP + MID + 1];
+#pragma unroll
+  for (int j = 0; j < HP; ++j) {
+    fx_split(g[j] - g[NP - 1 - j], dh[j], dl[j]);
+    fx_split(g[j] + g[NP - 1 - j], sh[j], sl[j]);
+  }
+  if (MID) fx_split(g[HP], sh[HP], sl[HP]);
+  fx_split(FL - FR, dh[HP], dl[HP]);
+  fx_split(FL + FR, sh[HP + MID], sl[HP + MID]);
+#pragma unroll
+  for (int i = 0; i < HP + MID; ++i) {
+    FxAcc a;
+    a.a = half;
+#pragma unroll
+    for (int j = 0; j <= HP; ++j) fx_mac(a, B.S[i][j], dh[j], dl[j]);
+    const long long odd = fx_round(a);
+    if (i < HP) {
+      FxAcc b;
+#pragma unroll
+      for (int j = 0; j <= HP + MID; ++j) fx_mac(b, B.D[i][j], sh[j], sl[j]);
+      const long long even = fx_round(b);
+      out[i] = odd + even;
+      out[NP - 1 - i] = odd - even;
+    } else {
+      out[i] = odd;
+    }
+  }
+}
+
+// One step of Burgers (SSP-RK3, or with LS a 2N low-storage scheme; with VISC the viscous term
+// of the local DG method). Warp w owns 32 - H - HR elements and forms H = ns more on the left
+// and HR on the right (warp_element), so the stages run in registers with shuffles for the face values and no barrier, and u is
+// read and written once per step. The operator
+//   dt L(v)_i = sum_j W_ij g_j + a_i F_L + b_i F_R,   g = v^2
 // (W = c2/2 (D + M^-1 e_0 e_0^T - M^-1 e_p e_p^T), a = -c2 M^-1 e_0, b = c2 M^-1 e_p) maps the
-// even part of (v^2, faces) to the odd part and back, since the nodes are symmetric, so it is
+// even part of (g, faces) to the odd part and back, since the nodes are symmetric, so it is
 // applied to sums and differences of mirrored nodes: 17 products instead of 35 at p = 4
 // (BurgersFixed). REC also writes the stage inputs v1, v2 (recorded sweeps of the gradient).
-// Bound by instruction issue (integer). K = 2^20, p = 4, ADG-AT2: 0.50 ms a step as three FP64
-// stage kernels (80% of the FP64 pipe), 0.078 ms so; K = 10125, p = 2: 14.5 -> 5.3 us, where
-// the launch and the dependent loads of the delays and ring levels are what is left. Two
-// elements per thread (58 of 64 owned, 128 registers) took 0.089 ms and 7.0 us.
-template <int NP, bool FACES, bool REC>
+// VISC: with (g, F) = (2 v, uhat) the same operator gives Z = -dt q of the local DG method
+// (uhat = u^-), and (g, F) = (v^2 - 2 nu q, F - nu qhat) (qhat = q^+) the whole dt L; Z is
+// brought to 58 bits by its largest value over the warp, since smooth fields leave it far
+// below its bound.
+// Bound by instruction issue (integer). K = 2^20, p = 4, ADG-AT2, SSP-RK3: 0.50 ms a step as
+// three FP64 stage kernels (80% of the FP64 pipe, eight field passes), 0.078 ms so; K = 10125,
+// p = 2: 14.5 -> 5.3 us, where the launch and the dependent loads of the delays and ring levels
+// are what is left. Two elements per thread (58 of 64 owned, 128 registers) took 0.089 ms and
+// 7.0 us.
+template <int NP, bool FACES, bool REC, bool VISC, bool LS>
 __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ Inst I,
-                                                      const double *__restrict__ uin,
-                                                      double *__restrict__ uout,
-                                                      double *__restrict__ r1,
-                                                      double *__restrict__ r2, int rel) {
-  constexpr int HP = NP / 2, MID = NP % 2;   // mirrored pairs, middle node
-  __shared__ double sV_[FACES ? 4 * kStages : 1][32];
+                                                      const __grid_constant__ StepArgs A) {
+  constexpr int NV = kFaceVals<VISC>, MS = LS ? kMaxStages : kStages;
+  __shared__ double sV_[FACES ? 4 * NV * MS : 1][32];
   pdl_wait();
   pdl_trigger();
-  const int K = I.K;
+  const int K = I.K, S = LS ? I.ns : kStages;
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if ((int64_t)warp * kOwn >= K) return;
+  if ((int64_t)warp * (32 - A.H - A.HR) >= K) return;
   const unsigned full = 0xffffffffu;
   bool own;
-  const int e = warp_element(K, warp, lane, own);
+  const int e = warp_element(K, warp, lane, A.H, A.HR, own);
   double ud[NP];
-  load_elem<NP>(uin, K, e, ud);
+  load_elem<NP>(A.uin, K, e, ud);
 
-  // a PE face on the left of this lane's element, and its delayed fluxes
+  // a PE face on the left of this lane's element, and its delayed values
   bool pe = false, late = false;
   int nm = 0;
-  double (*sV)[32] = sV_ + (FACES ? (threadIdx.x >> 5) * kStages : 0);
-  int vmax = 0;   // largest high word of a delayed flux
+  double (*sV)[32] = sV_ + (FACES ? (threadIdx.x >> 5) * NV * MS : 0);
+  int fmax = 0, umax = 0;   // largest high words of the delayed fluxes and traces
   if (FACES) {
     const int j = e / I.Kpe;
-    const int64_t n = I.meta[0] + rel;
-    nm = (int)(n % I.R);
+    const int64_t n = I.meta[0] + A.rel;
+    nm = mod_step(n, I.R);
     pe = e == j * I.Kpe;
     if (pe) {
       const DelayAt d = delay_at(I, j, n);
       late = d.k > 0;
       if (late) {
+        for (int s = 0; s < S; ++s)
 #pragma unroll
-        for (int s = 0; s < kStages; ++s) {
-          const double V = ring_flux(I, d, j, nm, s);
-          sV[s][lane] = V;
-          vmax = max(vmax, __double2hiint(V) & 0x7fffffff);
-        }
+          for (int w = 0; w < NV; ++w) {
+            const double V = ring_sum(I, d, w, j, nm, s);
+            sV[w * S + s][lane] = V;
+            const int h = __double2hiint(V) & 0x7fffffff;
+            if (w == 0) fmax = max(fmax, h);
+            if (w == 1) umax = max(umax, h);
+          }
       }
     }
   }
@@ -144,25 +243,24 @@ __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ In
   }
   const int be = __reduce_max_sync(full, hi) >> 20;
   const int E = be - 1022;              // |u| < 2^E
-  const int d0 = -(I.bf.sc + E + 1);    // operator sums -> value units
-  bool bad = be < kBfMinE || be > kBfMaxE || d0 < -2 || !I.bf.ok;
+  const BurgersFixed &B = I.bf;
+  const int d0 = -(B.sc + E + 1);       // operator sums -> value units (inviscid)
+  bool bad = be < kBfMinE || be > kBfMaxE || d0 < -2 || !B.ok;
   bad = bad || (hi ? (hi >> 20) < be - kBfSpan : lo != 0);
-  if (FACES) bad = bad || (vmax >> 20) > 2 * E + 1023;   // a delayed flux of 2^(2E + 1) or more
+  // a delayed flux of 2^(2E + 1) or more, a delayed trace of 2^(E + 1) or more
+  if (FACES) bad = bad || (fmax >> 20) > 2 * E + 1023;
+  if (FACES && VISC) bad = bad || (umax >> 20) > be + 1;
 
   if (!__any_sync(full, bad)) {
-    const BurgersFixed &B = I.bf;
     const int sg = 2 * E - 56;   // unit of the squares and fluxes
-    long long u[NP], v[NP];
+    long long u[NP], v[NP];      // u: u^n, or dU of a 2N scheme
 #pragma unroll
-    for (int i = 0; i < NP; ++i) v[i] = u[i] = bf_from(ud[i], be);
+    for (int i = 0; i < NP; ++i) {
+      v[i] = bf_from(ud[i], be);
+      u[i] = LS ? 0 : v[i];
+    }
     unsigned long long mag = 0;
-#pragma unroll
-    for (int s = 0; s < kStages; ++s) {
-      // shift of the operator's sums: stage 1 takes a quarter of them, stage 2 (inside the
-      // sum divided by 3) twice
-      int d = s == 0 ? d0 : (s == 1 ? d0 + 2 : d0 - 1);
-      d = d > 60 ? 60 : d;
-      const long long half = d > 0 ? 1ll << (d - 1) : 0;
+    auto stage = [&](int s) {
       long long G[NP];
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
@@ -173,73 +271,122 @@ __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ In
       const long long vl = __shfl_up_sync(full, v[NP - 1], 1);
       const long long gl = __shfl_up_sync(full, G[NP - 1], 1);
       long long FL = bf_llf(vl, v[0], gl, G[0]);
+      const size_t at = FACES && pe ? ((size_t)nm * I.ns + s) * I.P + e / I.Kpe : 0;
       if (FACES && pe) {
-        if (own)
-          I.ring[((size_t)nm * kStages + s) * I.P + e / I.Kpe] = make_double2(bf_to(FL, sg), 0.0);
+        if (own) I.ring[at] = make_double2(bf_to(FL, sg), VISC ? bf_to(vl, E - 57) : 0.0);
         if (late) FL = bf_from(sV[s][lane], 2 * E + 1023);
       }
-      const long long FR = __shfl_down_sync(full, FL, 1);
-      // sums and differences of mirrored nodes, and of the faces
-      int dh[HP + 1], dl[HP + 1], sh[HP + MID + 1], sl[HP + MID + 1];
+      int d = d0;
+      if (VISC) {
+        long long uL = vl;
+        if (FACES && late) uL = bf_from(sV[S + s][lane], be + 1) << 1;
+        const long long uN = __shfl_down_sync(full, uL, 1);
+        const long long uR = FACES && lane < 31 ? uN : v[NP - 1];   // v_p but at delayed faces
+        long long g2[NP], Z[NP];
 #pragma unroll
-      for (int j = 0; j < HP; ++j) {
-        fx_split(G[j] - G[NP - 1 - j], dh[j], dl[j]);
-        fx_split(G[j] + G[NP - 1 - j], sh[j], sl[j]);
-      }
-      if (MID) fx_split(G[HP], sh[HP], sl[HP]);
-      fx_split(FL - FR, dh[HP], dl[HP]);
-      fx_split(FL + FR, sh[HP + MID], sl[HP + MID]);
+        for (int i = 0; i < NP; ++i) g2[i] = 2 * v[i];
+        burgers_operator<NP>(B, g2, uL, uR, 0, Z);
+        // Z 2^nz below 2^58 over the warp
+        unsigned zh = 0;
 #pragma unroll
-      for (int i = 0; i < HP + MID; ++i) {
-        FxAcc a;
-        a.a = half;
+        for (int i = 0; i < NP; ++i) zh = max(zh, (unsigned)(fx_mag(Z[i]) >> 32));
+        zh = __reduce_max_sync(full, zh);
+        const int nz = __clz((int)zh) - 6;   // bit length of |Z| at most 64 - clz(zh)
+        // y = -2 nu q = (2 nu / dt) Z: limbs of (2 nu / dt) 2^-sn, in units of 2^uq
+        const int uq = B.sc + E - 57 - nz + B.sn;
+        const int uphi = max(uq, sg), sq = min(uphi - uq, 60), sf = min(uphi - sg, 60);
+        const long long hq = sq > 0 ? 1ll << (sq - 1) : 0, hf = sf > 0 ? 1ll << (sf - 1) : 0;
+        long long y0 = 0;
 #pragma unroll
-        for (int j = 0; j <= HP; ++j) fx_mac(a, B.S[i][j], dh[j], dl[j]);
-        const long long odd = fx_round(a);
-        long long even = 0;
-        if (i < HP) {
-          FxAcc b;
-#pragma unroll
-          for (int j = 0; j <= HP + MID; ++j) fx_mac(b, B.D[i][j], sh[j], sl[j]);
-          even = fx_round(b);
+        for (int i = 0; i < NP; ++i) {
+          int zh2, zl2;
+          fx_split(bf_shift(Z[i], -nz), zh2, zl2);
+          FxAcc c;
+          fx_mac(c, B.vn, zh2, zl2);
+          const long long y = (fx_round(c) + hq) >> sq;
+          G[i] = ((G[i] + hf) >> sf) + y;
+          if (i == 0) y0 = y;
         }
-#pragma unroll
-        for (int m = 0; m < (i < HP ? 2 : 1); ++m) {
-          const int k = m ? NP - 1 - i : i;
-          const long long r = m ? odd - even : odd + even;
-          if (d < 0 && (fx_mag(r) >> (kBfTop + d))) mag |= 1ull << kBfTop;
-          const long long x = bf_shift(r, d);
-          if (s == 0) {
-            v[k] += x;
-          } else if (s == 1) {
-            v[k] = ((3 * u[k] + v[k] + 2) >> 2) + x;
-          } else {
-            const long long T = u[k] + 2 * v[k] + x;
-            mag |= fx_mag(T) >> 2;   // below 2^60: its high limb fits 32 bits
-            int th, tl;
-            fx_split(T, th, tl);
-            FxAcc c;
-            fx_mac(c, make_int2(kThirdHi, kThirdLo), th, tl);
-            v[k] = fx_round(c);
+        FL = (FL + hf) >> sf;
+        if (FACES && pe) {
+          if (own) I.ringq[at] = bf_to(y0, uphi);
+          if (late) {
+            const double y = sV[2 * S + s][lane];
+            // |y| < 2^(uphi + 58)
+            if (((__double2hiint(y) & 0x7fffffff) >> 20) > uphi + 1080) mag |= 1ull << kBfTop;
+            else y0 = bf_from(y, uphi + 1080) << 1;
           }
-          mag |= fx_mag(v[k]);
         }
+        FL += (y0 + 1) >> 1;
+        d = -(B.sc + uphi - E + 57);
+        if (d < -2) {
+          mag |= 1ull << kBfTop;
+          d = -2;
+        }
+      }
+      const long long FR = __shfl_down_sync(full, FL, 1);
+      // shift of the operator's sums: in SSP-RK3 stage 1 takes a quarter of them, stage 2
+      // (inside the sum divided by 3) twice
+      if (!LS) d = s == 0 ? d : (s == 1 ? d + 2 : d - 1);
+      d = d > 60 ? 60 : d;
+      long long r[NP];
+      burgers_operator<NP>(B, G, FL, FR, d > 0 ? 1ll << (d - 1) : 0, r);
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        if (d < 0 && (fx_mag(r[k]) >> (kBfTop + d))) mag |= 1ull << kBfTop;
+        const long long x = bf_shift(r[k], d);
+        if (LS) {
+          if (s > 0) {
+            int h, l;
+            fx_split(u[k], h, l);
+            FxAcc c;
+            fx_mac(c, B.lsA[s], h, l);
+            u[k] = fx_round(c) + x;
+          } else {
+            u[k] = x;
+          }
+          mag |= fx_mag(u[k]);
+          int h, l;
+          fx_split(u[k], h, l);
+          FxAcc c;
+          fx_mac(c, B.lsB[s], h, l);
+          v[k] += fx_round(c);
+        } else if (s == 0) {
+          v[k] += x;
+        } else if (s == 1) {
+          v[k] = ((3 * u[k] + v[k] + 2) >> 2) + x;
+        } else {
+          const long long T = u[k] + 2 * v[k] + x;
+          mag |= fx_mag(T) >> 2;   // below 2^60: its high limb fits 32 bits
+          int th, tl;
+          fx_split(T, th, tl);
+          FxAcc c;
+          fx_mac(c, make_int2(kThirdHi, kThirdLo), th, tl);
+          v[k] = fx_round(c);
+        }
+        mag |= fx_mag(v[k]);
       }
       if (REC && s < 2 && own) {
-        double *o = s == 0 ? r1 : r2;
+        double *o = s == 0 ? A.r1 : A.r2;
 #pragma unroll
         for (int i = 0; i < NP; ++i) o[(size_t)i * K + e] = bf_to(v[i], E - 57);
       }
+    };
+    if (LS) {
+      for (int s = 0; s < S; ++s) stage(s);
+    } else {
+#pragma unroll
+      for (int s = 0; s < kStages; ++s) stage(s);
     }
     if (!__any_sync(full, (mag >> kBfTop) != 0)) {
       if (own) {
 #pragma unroll
-        for (int i = 0; i < NP; ++i) uout[(size_t)i * K + e] = bf_to(v[i], E - 57);
+        for (int i = 0; i < NP; ++i) A.uout[(size_t)i * K + e] = bf_to(v[i], E - 57);
       }
       return;
     }
   }
-  burgers_step_fp64<NP, FACES, REC>(I, warp, uin, uout, r1, r2, nm, sV, pe, late);
+  burgers_step_fp64<NP, FACES, REC, VISC, LS>(I, A, warp, nm, sV, pe, late);
 }
 
 // What the reverse step reads: the recorded stage inputs u, v1, v2 (y, one field of nd values
@@ -299,7 +446,7 @@ __device__ __noinline__ void burgers_adj_fp64(const Inst &I, const AdjArgs &A, i
   const size_t nd = (size_t)K * NP;
   const int lane = threadIdx.x & 31;
   bool own;
-  const int e = warp_element(K, warp, lane, own);
+  const int e = warp_element(K, warp, lane, kHalo, kHalo, own);
   const unsigned full = 0xffffffffu;
   double w[NP], acc[NP];
   load_elem<NP>(A.w, K, e, w);
@@ -372,7 +519,7 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
   if ((int64_t)warp * kOwn >= K) return;
   const unsigned full = 0xffffffffu;
   bool own;
-  const int e = warp_element(K, warp, lane, own);
+  const int e = warp_element(K, warp, lane, kHalo, kHalo, own);
   double wd[NP], yd[kStages][NP];
   load_elem<NP>(A.w, K, e, wd);
 #pragma unroll
@@ -539,21 +686,27 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
 }
 
 // One-warp blocks while the mesh gives fewer than 16 warps per SM (they spread evenly).
-template <int NP>
-cudaError_t burgers_np(const Inst &I, const double *uin, double *uout, double *r1, double *r2,
-                       int rel, cudaStream_t s, bool pdl) {
-  const int64_t warps = ((int64_t)I.K + kOwn - 1) / kOwn;
-  const int bs = warps < 16 * sm_count() ? 32 : 128;
+int burgers_block(int64_t warps) { return warps < 16 * sm_count() ? 32 : 128; }
+
+template <int NP, bool FACES>
+cudaError_t burgers_np(const Inst &I, const StepArgs &A, cudaStream_t s, bool pdl) {
+  const int own = 32 - A.H - A.HR;
+  const int64_t warps = ((int64_t)I.K + own - 1) / own;
+  const int bs = burgers_block(warps);
   const dim3 g((unsigned)((warps * 32 + bs - 1) / bs)), b(bs);
-  auto go = [&](auto kernel) { return launch_maybe_pdl(kernel, g, b, s, pdl, I, uin, uout, r1, r2, rel); };
-  if (r1) return I.async ? go(k_burgers_step<NP, true, true>) : go(k_burgers_step<NP, false, true>);
-  return I.async ? go(k_burgers_step<NP, true, false>) : go(k_burgers_step<NP, false, false>);
+  auto go = [&](auto kernel) { return launch_maybe_pdl(kernel, g, b, s, pdl, I, A); };
+  if (A.r1) return go(k_burgers_step<NP, FACES, true, false, false>);
+  if (I.ls)
+    return I.visc ? go(k_burgers_step<NP, FACES, false, true, true>)
+                  : go(k_burgers_step<NP, FACES, false, false, true>);
+  return I.visc ? go(k_burgers_step<NP, FACES, false, true, false>)
+                : go(k_burgers_step<NP, FACES, false, false, false>);
 }
 
 template <int NP>
 cudaError_t burgers_adj_np(const Inst &I, const AdjArgs &A, cudaStream_t s) {
   const int64_t warps = ((int64_t)I.K + kOwn - 1) / kOwn;
-  const int bs = warps < 16 * sm_count() ? 32 : 128;
+  const int bs = burgers_block(warps);
   const unsigned g = (unsigned)((warps * 32 + bs - 1) / bs);
   if (I.async) k_burgers_adj<NP, true><<<g, bs, 0, s>>>(I, A);
   else k_burgers_adj<NP, false><<<g, bs, 0, s>>>(I, A);
@@ -577,12 +730,13 @@ cudaError_t launch_burgers_adj(const Inst &I, const double *y, const double *w, 
 
 cudaError_t launch_burgers_step(const Inst &I, const double *uin, double *uout, double *r1,
                                 double *r2, int rel, cudaStream_t s, bool pdl) {
-  if (uin == uout) return cudaErrorInvalidValue;
+  if (uin == uout || (r1 && (I.ls || I.visc))) return cudaErrorInvalidValue;
+  const StepArgs A{uin, uout, r1, r2, rel, I.ns, I.ns + (I.visc ? 1 : 0)};
   switch (I.Np) {
-    case 2: return burgers_np<2>(I, uin, uout, r1, r2, rel, s, pdl);
-    case 3: return burgers_np<3>(I, uin, uout, r1, r2, rel, s, pdl);
-    case 4: return burgers_np<4>(I, uin, uout, r1, r2, rel, s, pdl);
-    case 5: return burgers_np<5>(I, uin, uout, r1, r2, rel, s, pdl);
+    case 2: return I.async ? burgers_np<2, true>(I, A, s, pdl) : burgers_np<2, false>(I, A, s, pdl);
+    case 3: return I.async ? burgers_np<3, true>(I, A, s, pdl) : burgers_np<3, false>(I, A, s, pdl);
+    case 4: return I.async ? burgers_np<4, true>(I, A, s, pdl) : burgers_np<4, false>(I, A, s, pdl);
+    case 5: return I.async ? burgers_np<5, true>(I, A, s, pdl) : burgers_np<5, false>(I, A, s, pdl);
     default: return cudaErrorInvalidValue;
   }
 }

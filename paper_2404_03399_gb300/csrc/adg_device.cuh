@@ -96,20 +96,13 @@ __device__ __forceinline__ DelayAt delay_at(const I &inst, int j, int64_t n) {
 // Value at PE face j for step n, stage s (Eqs. asyncEulerDGconserved and at-flux-gen):
 // delay k = min(D[n][j], n), order q' = min(q, n-k+1),
 //   V = sum_{i<q'} c_i(k; q') v(T_{n-k-i, s, j}),
-// where T are the traces (u^-, u^+) of the stage-s input of step n-k-i and v is the
-// numerical flux (Burgers) or, for linear advection, the upwind trace (the flux is a V,
-// the same AT flux with the factor a taken out of the sum). Level n (k = 0) uses the
-// current traces (tl, tr); the owner (the element right of the face) stores T_{n,s,j}.
-template <int PDE, int DIR, class I>
-__device__ __forceinline__ double face_value(const I &inst, double uL, double uR) {
-  if (PDE == 0) return DIR > 0 ? uL : uR;
-  return num_flux<1>(0.0, uL, uR);
-}
-
+// where T are the traces (u^-, u^+) of the stage-s input of step n-k-i and v the upwind trace
+// (the flux is a V, the AT flux with the factor a taken out of the sum). Level n (k = 0)
+// uses the current traces (tl, tr); the owner (the element right of the face) stores T_{n,s,j}.
 // Ring levels prefetched by pe_value (rings with more levels fall back to dependent loads).
 constexpr int kPrefetchR = 12;
 
-template <int PDE, int DIR, class I>
+template <int DIR, class I>
 __device__ __forceinline__ double pe_value(const I &inst, int j, int64_t n, int s, double tl,
                                         double tr, bool owner) {
   const int P = inst.P;
@@ -144,45 +137,13 @@ __device__ __forceinline__ double pe_value(const I &inst, int j, int64_t n, int 
   const int k = d.k;
   const int qe = d.qe;
   const double *c = d.c;
-  double V;
-  if (k == 0) {
-    V = __dmul_rn(c[0], face_value<PDE, DIR>(inst, tl, tr));
-  } else {
-    const double2 t0 = fetch(k);
-    V = __dmul_rn(c[0], face_value<PDE, DIR>(inst, t0.x, t0.y));
-  }
+  auto upwind = [](double2 t) { return DIR > 0 ? t.x : t.y; };
+  double V = __dmul_rn(c[0], k == 0 ? (DIR > 0 ? tl : tr) : upwind(fetch(k)));
   for (int i = 1; i < qe; ++i) {
     const double ci = c[i];
-    if (ci != 0.0) {
-      const double2 ti = fetch(k + i);
-      V = __dadd_rn(V, __dmul_rn(ci, face_value<PDE, DIR>(inst, ti.x, ti.y)));
-    }
+    if (ci != 0.0) V = __dadd_rn(V, __dmul_rn(ci, upwind(fetch(k + i))));
   }
   if (owner) col[(size_t)nm * inst.ns * P] = make_double2(tl, tr);
-  return V;
-}
-
-// The AT value of q^+ at PE face j for step n, stage s (viscous Burgers, alternating flux
-// qhat = q^+): the same sum as pe_value over the stored q^+ traces of levels n-k-i; level n
-// (k = 0) uses the current q^+ (qcur). The ring write happens in the q pass (k_ldg_q).
-template <class I>
-__device__ __forceinline__ double pe_value_q(const I &inst, int j, int64_t n, int s, double qcur) {
-  const int P = inst.P;
-  const int R = inst.R;
-  const double *col = inst.ringq + (size_t)s * P + j;
-  const int nm = (int)(n % R);
-  const DelayAt d = delay_at(inst, j, n);
-  const int k = d.k;
-  auto fetch = [&](int m) -> double {   // q^+ of level n - m, 1 <= m < R
-    int slot = nm - m;
-    if (slot < 0) slot += R;
-    return col[(size_t)slot * inst.ns * P];
-  };
-  double V = __dmul_rn(d.c[0], k == 0 ? qcur : fetch(k));
-  for (int i = 1; i < d.qe; ++i) {
-    const double ci = d.c[i];
-    if (ci != 0.0) V = __dadd_rn(V, __dmul_rn(ci, fetch(k + i)));
-  }
   return V;
 }
 

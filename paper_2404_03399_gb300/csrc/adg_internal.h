@@ -117,6 +117,10 @@ struct BurgersFixed {
   int2 S[(kMaxNp + 1) / 2][kMaxNp / 2 + 1];
   int2 D[kMaxNp / 2][(kMaxNp + 1) / 2 + 1];
   int sc, ok;
+  // the 2N coefficients (|c| < 2: limbs of round(c 2^58)), and 2 nu / dt = vn 2^sn (vn <= 1)
+  int2 lsA[kMaxStages], lsB[kMaxStages];
+  int2 vn;
+  int sn, pad_;
 };
 
 // One DG instance as the kernels see it. Nodal fields are node-major: field[i*K + e].
@@ -158,10 +162,9 @@ struct alignas(16) Inst {
   int ls;               // 1: a 2N low-storage scheme (k_lsrk_stage, coefficients lsA, lsB)
   int visc;             // 1: viscous Burgers by the local DG method (k_ldg_q, then the stage)
   double lsA[kMaxStages], lsB[kMaxStages];
-  // viscous Burgers: nu, q = u_x of the stage input (node-major like the fields), the PE
-  // faces' q^+ traces [R][ns][P], and q = QD v + qlL (uhat_L - v_0) + qlR (uhat_R - v_p)
+  // viscous Burgers: nu, the PE faces' -2 nu q^+ [R][ns][P], and
+  // q = QD v + qlL (uhat_L - v_0) + qlR (uhat_R - v_p)
   double nu;
-  double *qbuf;
   double *ringq;
   double dt;            // the step (viscous Burgers and Euler kernels)
   double QD[kMaxNp * kMaxNp], qlL[kMaxNp], qlR[kMaxNp];
@@ -172,7 +175,7 @@ struct alignas(16) Inst {
   double tvb_m, dx;
   double *w;
   double avg_w[kMaxNp], p1_w[kMaxNp], xi[kMaxNp];
-  BurgersFixed bf;      // inviscid Burgers, SSP-RK3 (k_burgers_step)
+  BurgersFixed bf;      // Burgers (k_burgers_step)
   double pad3_;
 };
 
@@ -226,9 +229,9 @@ constexpr int kAdvSteps = 8;
 int adv_steps_per_launch(const Inst &I);
 cudaError_t launch_adv_steps(const Inst &I, const double *uin, double *uout, int rel, int m,
                              cudaStream_t s);
-// One SSP-RK3 step of inviscid Burgers uin -> uout (adg_burgers.cu), with the delayed / AT
-// flux and the ring write (its entries hold the face's flux) at PE faces; r1, r2 (both or
-// neither) receive the inputs of stages 1 and 2.
+// One step of Burgers uin -> uout (adg_burgers.cu), with the delayed / AT flux and the ring
+// write (entries of flux and u^-, and -2 nu q^+ in ringq) at PE faces; r1, r2 (both or neither;
+// inviscid SSP-RK3) receive the inputs of stages 1 and 2.
 cudaError_t launch_burgers_step(const Inst &I, const double *uin, double *uout, double *r1,
                                 double *r2, int rel, cudaStream_t s, bool pdl = false);
 // Its adjoint: from the recorded stage inputs y (u, v1, v2 one after another) of step
@@ -241,10 +244,6 @@ cudaError_t launch_burgers_adj(const Inst &I, const double *y, const double *w, 
 // with the delayed / AT flux and the ring write of the stage-input traces at PE faces.
 cudaError_t launch_lsrk_stage(const Inst &I, int s, int rel, const double *uin, double *uout,
                               cudaStream_t st);
-// Viscous Burgers (I.visc): q = u_x of stage `stage`'s input vin by the local DG method into
-// I.qbuf, with the AT value of uhat at PE faces and the owners' ring writes ((u^-, u^+) into
-// I.ring, q^+ into I.ringq); launched before that stage's kernel.
-cudaError_t launch_ldg_q(const Inst &I, const double *vin, int stage, int rel, cudaStream_t s);
 // Euler (I.euler, adg_euler.cu): stage `stage` of SSP-RK in Shu and Osher's form from its input
 // (u, v1, v2 by stage) into dst, and the slope limiter src -> dst (src != dst).
 cudaError_t launch_euler_stage(const Inst &I, int stage, int rel, double *dst, cudaStream_t s);

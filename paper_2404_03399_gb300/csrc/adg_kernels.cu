@@ -1,4 +1,4 @@
-// FP64 CUDA kernels of the ADG / ADG-AT SSP-RK3 step for sm_103a.
+// FP64 CUDA kernels of the ADG / ADG-AT SSP-RK3 step of advection for sm_103a.
 //
 // One thread per element, node-major layout (field[i*K + e]) so that every load and
 // store of a nodal plane is a coalesced 256-byte warp access. Face traces of the
@@ -18,11 +18,11 @@ namespace {
 // Vs - V at PE face j, stage `stage`, step n, from the face's traces (tl, tr): the
 // synchronous face value minus the delayed / AT value; the owner writes the traces into the
 // ring slot of step n.
-template <int PDE, int DIR, class I>
+template <int DIR, class I>
 __device__ __forceinline__ double pe_face_delta(const I &inst, int j, int64_t n, int stage,
                                                 double tl, double tr, bool owner) {
-  const double Vs = face_value<PDE, DIR>(inst, tl, tr);
-  const double V = pe_value<PDE, DIR>(inst, j, n, stage, tl, tr, owner);
+  const double Vs = DIR > 0 ? tl : tr;
+  const double V = pe_value<DIR>(inst, j, n, stage, tl, tr, owner);
   return __dsub_rn(Vs, V);
 }
 
@@ -35,18 +35,17 @@ struct LsArgs {
   double As, Bs;
 };
 
-// One SSP-RK3 stage for element e (all 32 lanes of the warp take part; lanes past the
-// end duplicate element K-1 and store nothing). With LS, stage ls.s of a 2N low-storage step
-// instead: the same right-hand side dt L(U) from the constants sc[0] (no identity and no
-// factor beta), dU_s = A_s dU_{s-1} + dt L(U_{s-1}) in place in v1 and U_s = U_{s-1} + B_s dU_s. DIR is the upwind side for advection
-// (+1: a > 0, -1: a < 0) and 0 for Burgers. With FACES, the PE-face correction of the
+// One SSP-RK3 stage of advection for element e (all 32 lanes of the warp take part; lanes past
+// the end duplicate element K-1 and store nothing). With LS, stage ls.s of a 2N low-storage
+// step instead: the same right-hand side dt L(U) from the constants sc[0] (no identity and no
+// factor beta), dU_s = A_s dU_{s-1} + dt L(U_{s-1}) in place in v1 and U_s = U_{s-1} + B_s dU_s.
+// DIR is the upwind side (+1: a > 0, -1: a < 0). With FACES, the PE-face correction of the
 // delayed / AT flux is applied here too (step n): the element right of PE face j
 // (e = j Kpe) owns the face, writes its ring entry and adds lL (Vs - V); the element left
 // of it (e = j Kpe - 1) forms the same value with the same arithmetic and adds lR (Vs - V).
 // The synchronous output is rounded first, so the result is bit-identical to a stage
 // followed by a separate face pass.
-template <int NP, int PDE, int STAGE, int DIR, bool FACES, bool LS = false, bool VISC = false,
-          class I>
+template <int NP, int STAGE, int DIR, bool FACES, bool LS = false, class I>
 __device__ __forceinline__ void stage_body(const I &inst, int e, int64_t n = 0,
                                            const LsArgs &ls = LsArgs{}) {
   const int K = inst.K;
@@ -59,14 +58,7 @@ __device__ __forceinline__ void stage_body(const I &inst, int e, int64_t n = 0,
   const int rstage = LS ? ls.s : STAGE;
 
   double v[NP];
-  {
-    const double *q = vin + ec;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      v[i] = __ldg(q);
-      q += K;
-    }
-  }
+  load_elem<NP>(vin, K, ec, v);
   double u[NP];   // the alpha operand: u^n, or dU_{s-1} of a 2N stage
   if (STAGE > 0) {
     if (LS && ls.first) {
@@ -86,113 +78,45 @@ __device__ __forceinline__ void stage_body(const I &inst, int e, int64_t n = 0,
   const bool edge = (lane == 31) || (ec + 1 >= K);
   const int fR = ec + 1 >= K ? 0 : ec + 1;
   double vLm = 0.0, vRp = 0.0;
-  if (PDE == 1 || DIR > 0) {
+  if (DIR > 0) {
     vLm = __shfl_up_sync(full, v[NP - 1], 1);
     if (lane == 0) vLm = __ldg(vin + (NP - 1) * K + (ec == 0 ? K - 1 : ec - 1));
-  }
-  if (PDE == 1 || DIR < 0) {
+  } else {
     vRp = __shfl_down_sync(full, v[0], 1);
     if (edge) vRp = __ldg(vin + fR);
   }
-  // Every face takes its synchronous flux here; at PE faces the face pass that follows
-  // the stage replaces it by the delayed / AT flux (a correction of the two elements).
-  double jL = 0.0, jR = 0.0;
-  if (PDE == 0) {
-    // Face values in trace units (the flux is a times the value).
-    if (DIR > 0) jL = __dsub_rn(v[0], vLm);
-    else jR = __dsub_rn(v[NP - 1], vRp);
-  } else {
-    const double FL = num_flux<1>(0.0, vLm, v[0]);
-    double FR = __shfl_down_sync(full, FL, 1);
-    if (edge) FR = num_flux<1>(0.0, v[NP - 1], vRp);
-    jL = __dsub_rn(phys_flux<1>(0.0, v[0]), FL);
-    jR = __dsub_rn(phys_flux<1>(0.0, v[NP - 1]), FR);
-  }
-
-  double g[NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) g[i] = PDE == 0 ? v[i] : v[i] * v[i];
+  // Every face takes its synchronous value here (in trace units: the flux is a times it); at PE
+  // faces the correction below replaces it by the delayed / AT one.
+  const double jump = DIR > 0 ? __dsub_rn(v[0], vLm) : __dsub_rn(v[NP - 1], vRp);
 
   double out[NP];
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
-    double acc;
-    if (PDE == 0) {
-      acc = STAGE == 0 ? C.A[i * NP] * g[0] : fma(C.A[i * NP], g[0], alpha * u[i]);
-    } else {
-      if (LS) acc = alpha * u[i];   // no v term: dt L(U) has none
-      else acc = STAGE == 0 ? v[i] : fma(C.beta, v[i], C.alpha * u[i]);
-      acc = fma(C.A[i * NP], g[0], acc);
-    }
+    double acc = STAGE == 0 ? C.A[i * NP] * v[0] : fma(C.A[i * NP], v[0], alpha * u[i]);
 #pragma unroll
-    for (int jj = 1; jj < NP; ++jj) acc = fma(C.A[i * NP + jj], g[jj], acc);
-    out[i] = acc;
-  }
-  if (PDE == 1 || DIR > 0) {
-#pragma unroll
-    for (int i = 0; i < NP; ++i) out[i] = fma(C.lL[i], jL, out[i]);
-  }
-  if (PDE == 1 || DIR < 0) {
-#pragma unroll
-    for (int i = 0; i < NP; ++i) out[i] = fma(C.lR[i], jR, out[i]);
+    for (int jj = 1; jj < NP; ++jj) acc = fma(C.A[i * NP + jj], v[jj], acc);
+    out[i] = fma(DIR > 0 ? C.lL[i] : C.lR[i], jump, acc);
   }
   if (FACES && e < K) {
     const int Kpe = inst.Kpe;
     const int jq = e / Kpe;
     const int r = e - jq * Kpe;
     if (r == 0) {   // left face is PE face jq; this element owns it
-      const double tl = (PDE == 1 || DIR > 0) ? vLm
-                        : __ldg(vin + (NP - 1) * K + (e == 0 ? K - 1 : e - 1));
-      const double d = pe_face_delta<PDE, DIR>(inst, jq, n, rstage, tl, v[0], true);
+      const double tl = DIR > 0 ? vLm : __ldg(vin + (NP - 1) * K + (e == 0 ? K - 1 : e - 1));
+      const double d = pe_face_delta<DIR>(inst, jq, n, rstage, tl, v[0], true);
       if (nonzero(d)) {
 #pragma unroll
         for (int i = 0; i < NP; ++i) out[i] = fma(C.lL[i], d, out[i]);
       }
     }
     if (r == Kpe - 1) {   // right face is PE face jq + 1 (face 0 for the last element)
-      const double tr = (PDE == 1 || DIR < 0) ? vRp : __ldg(vin + (e + 1 == K ? 0 : e + 1));
+      const double tr = DIR < 0 ? vRp : __ldg(vin + (e + 1 == K ? 0 : e + 1));
       const int jr = jq + 1 == inst.P ? 0 : jq + 1;
-      const double d = pe_face_delta<PDE, DIR>(inst, jr, n, rstage, v[NP - 1], tr, false);
+      const double d = pe_face_delta<DIR>(inst, jr, n, rstage, v[NP - 1], tr, false);
       if (nonzero(d)) {
 #pragma unroll
         for (int i = 0; i < NP; ++i) out[i] = fma(C.lR[i], d, out[i]);
       }
-    }
-  }
-  if (VISC && PDE == 1) {
-    // Viscous term nu q_x of the local DG method, alternating flux qhat = q^+ (q from the q
-    // pass, k_ldg_q), in the stage's folded constants (C.A = b c2 D / 2, C.lL, C.lR):
-    //   nu ( -2 C.A q + C.lR (qhat_R - q_p) + C.lL (qhat_L - q_0) ),
-    // with qhat_L = q_0 and qhat_R = q^{e+1}_0 at interior faces and the AT value of the stored
-    // q^+ traces at PE faces (both elements of the face alike).
-    double q[NP];
-    {
-      const double *qq = inst.qbuf + ec;
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        q[i] = *qq;
-        qq += K;
-      }
-    }
-    double qRp = __shfl_down_sync(full, q[0], 1);
-    if (edge) qRp = inst.qbuf[fR];
-    double jqL = 0.0, jqR = __dsub_rn(qRp, q[NP - 1]);
-    if (FACES && e < K) {
-      const int Kpe = inst.Kpe;
-      const int jq = e / Kpe;
-      const int r = e - jq * Kpe;
-      if (r == 0) jqL = __dsub_rn(pe_value_q(inst, jq, n, rstage, q[0]), q[0]);
-      if (r == Kpe - 1) {
-        const int jr = jq + 1 == inst.P ? 0 : jq + 1;
-        jqR = __dsub_rn(pe_value_q(inst, jr, n, rstage, qRp), q[NP - 1]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      double vq = C.A[i * NP] * q[0];
-#pragma unroll
-      for (int jj = 1; jj < NP; ++jj) vq = fma(C.A[i * NP + jj], q[jj], vq);
-      out[i] = fma(inst.nu, fma(C.lL[i], jqL, fma(C.lR[i], jqR, -2.0 * vq)), out[i]);
     }
   }
   if (e < K) {
@@ -276,7 +200,7 @@ __device__ __forceinline__ void stage_body_halo(const I &inst, int warp, int64_t
     const int jq = eo / Kpe;
     const bool face = lane >= 1 && e <= K && eo - jq * Kpe == 0;
     double d = 0.0;
-    if (face) d = pe_face_delta<0, DIR>(inst, jq, n, STAGE, vLm, v[0], own);
+    if (face) d = pe_face_delta<DIR>(inst, jq, n, STAGE, vLm, v[0], own);
     const double dR = __shfl_down_sync(full, d, 1);
     const bool faceR = __shfl_down_sync(full, face ? 1 : 0, 1) != 0;
     if (own && face && nonzero(d)) {
@@ -306,86 +230,11 @@ __global__ void __launch_bounds__(kTile) k_stage_halo(const Inst inst, int rel) 
   stage_body_halo<NP, STAGE, DIR, FACES>(inst, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n);
 }
 
-template <int NP, int PDE, int STAGE, int DIR, bool FACES, bool VISC = false>
-__global__ void __launch_bounds__(kTile) k_stage(const Inst inst, int rel) {
-  pdl_wait();
-  pdl_trigger();
-  const int64_t n = FACES ? inst.meta[0] + rel : 0;
-  stage_body<NP, PDE, STAGE, DIR, FACES, false, VISC>(inst, blockIdx.x * blockDim.x + threadIdx.x,
-                                                      n);
-}
-
 // Stage ls.s of a 2N low-storage step (Williamson's form; I.ls).
-template <int NP, int PDE, int DIR, bool FACES, bool VISC = false>
+template <int NP, int DIR, bool FACES>
 __global__ void __launch_bounds__(kTile) k_lsrk_stage(const Inst inst, int rel, const LsArgs ls) {
   const int64_t n = FACES ? inst.meta[0] + rel : 0;
-  stage_body<NP, PDE, 1, DIR, FACES, true, VISC>(inst, blockIdx.x * blockDim.x + threadIdx.x, n,
-                                                 ls);
-}
-
-// The q pass of viscous Burgers by the local DG method (Eq. burgers, Section 6): q = u_x of
-// the stage input v with the alternating flux uhat = u^- (the left element's right trace),
-//   q^e = (2/dx) [ D v^e + M^{-1} e_p (uhat_R - v^e_p) - M^{-1} e_0 (uhat_L - v^e_0) ]
-//       = QD v^e + qlR (uhat_R - v^e_p) + qlL (uhat_L - v^e_0),
-// uhat_L = v^{e-1}_p and uhat_R = v^e_p at interior faces (the right term vanishes). At a PE
-// face both elements take uhat as the AT sum of the stored u^- traces (pe_value of the upwind
-// kind); its owner stores the stage input's traces (u^-, u^+) and its q^+ = q^e_0 for the
-// later steps.
-template <int NP, bool FACES>
-__global__ void __launch_bounds__(kTile) k_ldg_q(const Inst inst, const double *__restrict__ vin,
-                                                 int stage, int rel) {
-  const int K = inst.K;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const int ec = e < K ? e : K - 1;
-  double v[NP];
-  {
-    const double *q = vin + ec;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      v[i] = __ldg(q);
-      q += K;
-    }
-  }
-  double vLm = __shfl_up_sync(0xffffffffu, v[NP - 1], 1);
-  if (lane == 0) vLm = __ldg(vin + (NP - 1) * K + (ec == 0 ? K - 1 : ec - 1));
-  double dL = __dsub_rn(vLm, v[0]), dR = 0.0;
-  int jown = -1;
-  if (FACES && e < K) {
-    const int64_t n = inst.meta[0] + rel;
-    const int Kpe = inst.Kpe;
-    const int jq = e / Kpe;
-    const int r = e - jq * Kpe;
-    if (r == 0) {
-      dL = __dsub_rn(pe_value<0, 1>(inst, jq, n, stage, vLm, v[0], true), v[0]);
-      jown = jq;
-    }
-    if (r == Kpe - 1) {
-      const double tr = __ldg(vin + (e + 1 == K ? 0 : e + 1));
-      const int jr = jq + 1 == inst.P ? 0 : jq + 1;
-      dR = __dsub_rn(pe_value<0, 1>(inst, jr, n, stage, v[NP - 1], tr, false), v[NP - 1]);
-    }
-  }
-  if (e >= K) return;
-  double q[NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    double acc = inst.QD[i * NP] * v[0];
-#pragma unroll
-    for (int j = 1; j < NP; ++j) acc = fma(inst.QD[i * NP + j], v[j], acc);
-    acc = fma(inst.qlL[i], dL, acc);
-    q[i] = fma(inst.qlR[i], dR, acc);
-  }
-  double *o = inst.qbuf + e;
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    *o = q[i];
-    o += K;
-  }
-  if (FACES && jown >= 0) {
-    const int64_t n = inst.meta[0] + rel;
-    inst.ringq[((size_t)(n % inst.R) * inst.ns + stage) * inst.P + jown] = q[0];
-  }
+  stage_body<NP, 1, DIR, FACES, true>(inst, blockIdx.x * blockDim.x + threadIdx.x, n, ls);
 }
 
 // Composed SSP-RK3 step of upwind advection (a > 0), all faces synchronous (StepConsts):
@@ -1060,14 +909,14 @@ __global__ void k_batch_copy_back(const Inst *__restrict__ insts, const int2 *__
 // out^e += lL (Vs - V), out^{e-1} += lR (Vs - V) (the flux enters the stage linearly through
 // the lift terms). With Kpe == 1 an element borders two PE faces; then thread j owns
 // element j and applies the corrections of both its faces.
-template <int PDE, int DIR, class I>
+template <int DIR, class I>
 __device__ __forceinline__ double face_delta(const I &inst, const double *vin, int j, int64_t n,
                                              int stage, bool owner) {
   const int K = inst.K;
   const int e = j * inst.Kpe;
   const double tl = vin[(size_t)(inst.Np - 1) * K + (e == 0 ? K - 1 : e - 1)];
   const double tr = vin[e];
-  return pe_face_delta<PDE, DIR>(inst, j, n, stage, tl, tr, owner);
+  return pe_face_delta<DIR>(inst, j, n, stage, tl, tr, owner);
 }
 
 template <class I>
@@ -1078,7 +927,7 @@ __device__ __forceinline__ void apply_delta(const I &inst, double *out, int e, c
   for (int i = 0; i < inst.Np; ++i) out[(size_t)i * K + e] = fma(lift[i], d, out[(size_t)i * K + e]);
 }
 
-template <int PDE, int DIR, class I>
+template <int DIR, class I>
 __device__ __forceinline__ void face_body(const I &inst, int stage, int j, int64_t n) {
   const double *vin = stage == 0 ? inst.u : (stage == 1 ? inst.v1 : inst.v2);
   double *out = stage == 0 ? inst.v1 : (stage == 1 ? inst.v2 : inst.unext);
@@ -1096,7 +945,7 @@ __device__ __forceinline__ void face_body(const I &inst, int stage, int j, int64
         ol[i] = out[(size_t)i * K + eL];
       }
     }
-    const double d = face_delta<PDE, DIR>(inst, vin, j, n, stage, true);
+    const double d = face_delta<DIR>(inst, vin, j, n, stage, true);
     if (nonzero(d)) {
 #pragma unroll
       for (int i = 0; i < kMaxNp; ++i) {
@@ -1109,8 +958,8 @@ __device__ __forceinline__ void face_body(const I &inst, int stage, int j, int64
   } else {
     // element j borders faces j (left) and j+1 (right); the right face's value is formed
     // again here with the same arithmetic as by its owner, so both agree bit for bit.
-    const double dL = face_delta<PDE, DIR>(inst, vin, j, n, stage, true);
-    const double dR = face_delta<PDE, DIR>(inst, vin, j + 1 == inst.P ? 0 : j + 1, n, stage, false);
+    const double dL = face_delta<DIR>(inst, vin, j, n, stage, true);
+    const double dR = face_delta<DIR>(inst, vin, j + 1 == inst.P ? 0 : j + 1, n, stage, false);
     double *o = out;
     if (nonzero(dL) || nonzero(dR)) {
       for (int i = 0; i < inst.Np; ++i) {
@@ -1131,19 +980,14 @@ __global__ void __launch_bounds__(256) k_batch_faces(const Inst *__restrict__ in
   const int j = w.y + threadIdx.x;
   if (j >= I.P) return;
   const int64_t n = I.meta[0] + rel;
-  if (I.pde == 1) face_body<1, 0>(I, stage, j, n);
-  else if (I.a >= 0.0) face_body<0, 1>(I, stage, j, n);
-  else face_body<0, -1>(I, stage, j, n);
+  if (I.a >= 0.0) face_body<1>(I, stage, j, n);
+  else face_body<-1>(I, stage, j, n);
 }
 
 template <int STAGE, int NP>
-__device__ __forceinline__ void batch_dispatch_pde(const Inst &I, int e) {
-  if (I.pde == 0) {
-    if (I.a >= 0.0) stage_body<NP, 0, STAGE, 1, false>(I, e);
-    else stage_body<NP, 0, STAGE, -1, false>(I, e);
-  } else {
-    stage_body<NP, 1, STAGE, 0, false>(I, e);
-  }
+__device__ __forceinline__ void batch_dispatch(const Inst &I, int e) {
+  if (I.a >= 0.0) stage_body<NP, STAGE, 1, false>(I, e);
+  else stage_body<NP, STAGE, -1, false>(I, e);
 }
 
 // Batched stage: block b handles work item (instance, first element); the instance's
@@ -1163,10 +1007,10 @@ __global__ void __launch_bounds__(kTile) k_batch_stage(const Inst *__restrict__ 
   const Inst &I = *reinterpret_cast<const Inst *>(smem);
   const int e = w.y + threadIdx.x;
   switch (I.Np) {
-    case 2: batch_dispatch_pde<STAGE, 2>(I, e); break;
-    case 3: batch_dispatch_pde<STAGE, 3>(I, e); break;
-    case 4: batch_dispatch_pde<STAGE, 4>(I, e); break;
-    default: batch_dispatch_pde<STAGE, 5>(I, e); break;
+    case 2: batch_dispatch<STAGE, 2>(I, e); break;
+    case 3: batch_dispatch<STAGE, 3>(I, e); break;
+    case 4: batch_dispatch<STAGE, 4>(I, e); break;
+    default: batch_dispatch<STAGE, 5>(I, e); break;
   }
 }
 
@@ -1287,40 +1131,31 @@ __global__ void __launch_bounds__(kRedThreads)
   if (threadIdx.x == 0) out[0] = (kind == 0 || kind == 3) ? sh[0] * scale : sh[0];
 }
 
-template <int NP, int PDE, int STAGE, int DIR>
-cudaError_t launch_np_pde_stage(const Inst &I, int rel, cudaStream_t s, bool pdl) {
+template <int NP, int STAGE, int DIR>
+cudaError_t launch_np_stage(const Inst &I, int rel, cudaStream_t s, bool pdl) {
   const int bs = stage_block(I.K);
-  if constexpr (PDE == 1) {   // viscous (inviscid Burgers takes k_burgers_step)
-    if (!I.visc) return cudaErrorInvalidValue;
-    const dim3 g((unsigned)((I.K + bs - 1) / bs));
-    if (I.async)
-      return launch_maybe_pdl(k_stage<NP, PDE, STAGE, DIR, true, true>, g, dim3(bs), s, pdl, I, rel);
-    return launch_maybe_pdl(k_stage<NP, PDE, STAGE, DIR, false, true>, g, dim3(bs), s, pdl, I, rel);
-  } else {
-    // 30 elements per warp (halo lanes); one-thread-per-element stage_body is kept for the 2N
-    // low-storage, viscous and batched stages
-    const int64_t warps = (I.K + 29) / 30;
-    const dim3 g((unsigned)((warps * 32 + bs - 1) / bs));
-    if (I.async)
-      return launch_maybe_pdl(k_stage_halo<NP, STAGE, DIR, true>, g, dim3(bs), s, pdl, I, rel);
-    return launch_maybe_pdl(k_stage_halo<NP, STAGE, DIR, false>, g, dim3(bs), s, pdl, I, rel);
-  }
+  // 30 elements per warp (halo lanes); one-thread-per-element stage_body is kept for the 2N
+  // low-storage and batched stages
+  const int64_t warps = (I.K + 29) / 30;
+  const dim3 g((unsigned)((warps * 32 + bs - 1) / bs));
+  if (I.async)
+    return launch_maybe_pdl(k_stage_halo<NP, STAGE, DIR, true>, g, dim3(bs), s, pdl, I, rel);
+  return launch_maybe_pdl(k_stage_halo<NP, STAGE, DIR, false>, g, dim3(bs), s, pdl, I, rel);
 }
 
-template <int NP, int PDE, int DIR>
-cudaError_t launch_np_pde(const Inst &I, int stage, int rel, cudaStream_t s, bool pdl) {
+template <int NP, int DIR>
+cudaError_t launch_np_dir(const Inst &I, int stage, int rel, cudaStream_t s, bool pdl) {
   switch (stage) {
-    case 0: return launch_np_pde_stage<NP, PDE, 0, DIR>(I, rel, s, pdl);
-    case 1: return launch_np_pde_stage<NP, PDE, 1, DIR>(I, rel, s, pdl);
-    default: return launch_np_pde_stage<NP, PDE, 2, DIR>(I, rel, s, pdl);
+    case 0: return launch_np_stage<NP, 0, DIR>(I, rel, s, pdl);
+    case 1: return launch_np_stage<NP, 1, DIR>(I, rel, s, pdl);
+    default: return launch_np_stage<NP, 2, DIR>(I, rel, s, pdl);
   }
 }
 
 template <int NP>
 cudaError_t launch_np(const Inst &I, int stage, int rel, cudaStream_t s, bool pdl) {
-  if (I.pde == 1) return launch_np_pde<NP, 1, 0>(I, stage, rel, s, pdl);
-  return I.a >= 0.0 ? launch_np_pde<NP, 0, 1>(I, stage, rel, s, pdl)
-                    : launch_np_pde<NP, 0, -1>(I, stage, rel, s, pdl);
+  return I.a >= 0.0 ? launch_np_dir<NP, 1>(I, stage, rel, s, pdl)
+                    : launch_np_dir<NP, -1>(I, stage, rel, s, pdl);
 }
 
 }  // namespace
@@ -1337,48 +1172,21 @@ cudaError_t launch_stage(const Inst &I, int stage, int rel, cudaStream_t s, bool
 
 namespace {
 
-template <int NP, int PDE, int DIR>
-cudaError_t lsrk_np_pde(const Inst &I, int rel, const LsArgs &ls, cudaStream_t s) {
+template <int NP, int DIR>
+cudaError_t lsrk_np_dir(const Inst &I, int rel, const LsArgs &ls, cudaStream_t s) {
   const int bs = stage_block(I.K);
   const unsigned grid = (unsigned)((I.K + bs - 1) / bs);
-  if (PDE == 1 && I.visc) {
-    if (I.async) k_lsrk_stage<NP, PDE, DIR, true, true><<<grid, bs, 0, s>>>(I, rel, ls);
-    else k_lsrk_stage<NP, PDE, DIR, false, true><<<grid, bs, 0, s>>>(I, rel, ls);
-  } else if (I.async) {
-    k_lsrk_stage<NP, PDE, DIR, true><<<grid, bs, 0, s>>>(I, rel, ls);
-  } else {
-    k_lsrk_stage<NP, PDE, DIR, false><<<grid, bs, 0, s>>>(I, rel, ls);
-  }
-  return cudaGetLastError();
-}
-
-template <int NP>
-cudaError_t ldg_q_np(const Inst &I, const double *vin, int stage, int rel, cudaStream_t s) {
-  const int bs = stage_block(I.K);
-  const unsigned grid = (unsigned)((I.K + bs - 1) / bs);
-  if (I.async) k_ldg_q<NP, true><<<grid, bs, 0, s>>>(I, vin, stage, rel);
-  else k_ldg_q<NP, false><<<grid, bs, 0, s>>>(I, vin, stage, rel);
+  if (I.async) k_lsrk_stage<NP, DIR, true><<<grid, bs, 0, s>>>(I, rel, ls);
+  else k_lsrk_stage<NP, DIR, false><<<grid, bs, 0, s>>>(I, rel, ls);
   return cudaGetLastError();
 }
 
 template <int NP>
 cudaError_t lsrk_np(const Inst &I, int rel, const LsArgs &ls, cudaStream_t s) {
-  if (I.pde == 1) return lsrk_np_pde<NP, 1, 0>(I, rel, ls, s);
-  return I.a >= 0.0 ? lsrk_np_pde<NP, 0, 1>(I, rel, ls, s) : lsrk_np_pde<NP, 0, -1>(I, rel, ls, s);
+  return I.a >= 0.0 ? lsrk_np_dir<NP, 1>(I, rel, ls, s) : lsrk_np_dir<NP, -1>(I, rel, ls, s);
 }
 
 }  // namespace
-
-cudaError_t launch_ldg_q(const Inst &I, const double *vin, int stage, int rel, cudaStream_t s) {
-  if (!I.visc || !I.qbuf || stage < 0 || stage >= I.ns) return cudaErrorInvalidValue;
-  switch (I.Np) {
-    case 2: return ldg_q_np<2>(I, vin, stage, rel, s);
-    case 3: return ldg_q_np<3>(I, vin, stage, rel, s);
-    case 4: return ldg_q_np<4>(I, vin, stage, rel, s);
-    case 5: return ldg_q_np<5>(I, vin, stage, rel, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
 
 cudaError_t launch_lsrk_stage(const Inst &I, int s, int rel, const double *uin, double *uout,
                               cudaStream_t st) {

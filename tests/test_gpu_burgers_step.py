@@ -67,3 +67,21 @@ def test_fields_outside_the_integer_path(field):
     if field == "pulse":
         big = np.max(np.abs(ref), axis=1, keepdims=True)
         assert np.max(np.abs(got - ref) / big) < 1e-11   # every element to its own largest value
+
+
+@pytest.mark.parametrize("rk", ["rk1", "rk2", "lsrk3", "lsrk4", "ssprk3"])
+@pytest.mark.parametrize("nu", [0.0, 0.1])
+@pytest.mark.parametrize("K,P,p", [(21, 1, 3), (27, 27, 1), (50, 10, 2), (400, 8, 4)])
+def test_schemes_and_viscosity(rk, nu, K, P, p):
+    dx = 2.0 * math.pi / K
+    cfg = adg.Config(pde="burgers", K=K, p=p, P=P, dt=0.002 * dx * dx if nu else 0.002 * dx, nu=nu, rk=rk,
+                     mode="at" if P > 1 else "sync", L=3, q=2, seed=12)
+    u0 = 0.4 + np.sin(dg.node_coordinates(K, p, 0.0, 2.0 * math.pi)) + 0.02 * random_nodal(K, p, 2)
+    s = adg.Solver(cfg, torch.tensor(u0, device="cuda"))
+    s.step(21)
+    got, dt = s.state().cpu().numpy(), s.dt
+    s.close()
+    prob = dg.Problem(pde="burgers", K=K, p=p, P=P, dt=dt, x0=cfg.x0, x1=cfg.x1, nu=nu, rk=rk, q=2,
+                      mode="adg" if P > 1 else "sync", delays=odelays.delay_table(12, P, 21, 3))
+    ref = dg.run(prob, u0, 21).numpy()
+    assert np.max(np.abs(got - ref)) < TOL * np.max(np.abs(ref))
