@@ -39,8 +39,8 @@ def _stale(obj: str, deps) -> bool:
 
 def build(verbose: bool = False, force: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(CSRC, "adg_internal.h"), os.path.join(CSRC, "adg_device.cuh"),
-               os.path.join(CSRC, "adg_fixed.cuh"), os.path.join(CSRC, "adg_bfp.cuh"), os.path.join(INCLUDE, "adg.h")]
+    headers = [os.path.join(CSRC, f) for f in sorted(os.listdir(CSRC)) if f.endswith((".h", ".cuh"))]
+    headers.append(os.path.join(INCLUDE, "adg.h"))
     objs, procs = [], []
     for src in SOURCES:
         path = os.path.join(CSRC, src)

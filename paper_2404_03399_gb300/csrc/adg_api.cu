@@ -1303,6 +1303,13 @@ void fold_step_constants(InstHost &h, bool allow_basis) {
     }
   ok = ok && rsums;
   h.I.face_fx = ok ? 1 : 0;
+  h.I.rho_fx = 1;
+  std::memset(h.I.rhof, 0, sizeof(h.I.rhof));
+  for (int s = 1; s < S; ++s)
+    for (int t = 0; t < s; ++t) {
+      if (!(std::fabs(rhol[s][t]) < 2.0L)) h.I.rho_fx = 0;
+      else h.I.rhof[s][t] = limbs58(rhol[s][t]);
+    }
 }
 
 int reduce(adg_ctx *c, InstHost &h, int kind, const double *g, double scale, double *host_out,
@@ -1656,8 +1663,16 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
     for (int k = 0; k < L; ++k)
       for (int qe = 1; qe <= q; ++qe)
         for (int i = 0; i < qe; ++i) cf[((size_t)k * q + (qe - 1)) * q + i] = at_coef(k, qe, i);
+    // the coefficients and, after them, the same as integers (two to a double's place)
+    const size_t nc = cf.size();
+    cf.resize(nc + (nc + 1) / 2, 0.0);
+    for (size_t i = 0; i < nc; ++i) {
+      const int v = (int)std::llround(cf[i]);
+      std::memcpy(reinterpret_cast<char *>(cf.data() + nc) + i * sizeof(int), &v, sizeof(int));
+    }
     CK(cudaMalloc(&h.coef, cf.size() * sizeof(double)));
     I.coef = h.coef;
+    I.coefi = reinterpret_cast<const int *>(h.coef + nc);
     if (dt_from_data)
       CK(cudaMemcpyAsync(h.coef, cf.data(), cf.size() * sizeof(double), cudaMemcpyHostToDevice,
                          c->stream));
@@ -2664,13 +2679,22 @@ int adg_batch_init(const adg_config *cfgs, const double *const *u0_devs, int32_t
       if (hi[i].async)
         for (int j0 = 0; j0 < hi[i].P; j0 += 256) fwork.push_back(make_int2(i, j0));
     }
+    // the faces of each part by degree, padded (face -1) to whole warps of the fix-up (eight
+    // faces of one degree)
     int nflat_part[kBatchParts] = {};
-    for (int hh = 0; hh < kBatchParts; ++hh)
-      for (int i = 0; i < n; ++i)
-        if (half[i] == hh && hi[i].async) {
-          for (int j = 0; j < hi[i].P; ++j) fflat.push_back(make_int2(i, j));
-          nflat_part[hh] += hi[i].P;
-        }
+    for (int hh = 0; hh < kBatchParts; ++hh) {
+      const size_t start = fflat.size();
+      for (int Np = 2; Np <= adg::kMaxNp; ++Np) {
+        int last = 0;
+        for (int i = 0; i < n; ++i)
+          if (half[i] == hh && hi[i].async && hi[i].Np == Np) {
+            for (int j = 0; j < hi[i].P; ++j) fflat.push_back(make_int2(i, j));
+            last = i;
+          }
+        while (fflat.size() % 8) fflat.push_back(make_int2(last, -1));
+      }
+      nflat_part[hh] = (int)(fflat.size() - start);
+    }
     // every instance of a degree with the same fixed-point coefficients: pass them per degree,
     // with one record per work item of ept tiles (ept elements per thread)
     if (!r && all_fixed) {

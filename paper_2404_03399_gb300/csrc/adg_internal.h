@@ -132,6 +132,7 @@ struct alignas(16) Inst {
   const uint8_t *table; // [table_rows][P] delays
   const int64_t *meta;  // meta[0] = step index of rel 0; meta[1] = first table row's step
   const double *coef;   // AT coefficients [L][q][q]: coef[(k*q + (q'-1))*q + i]
+  const int *coefi;     // the same as integers
   double a;
   int K, Np, P, Kpe, R, L, q, pde, async, table_rows;
   int fused;            // 0: staged; composed stencil + PE-face fix-up in 1: FP64 (StepConsts),
@@ -147,6 +148,8 @@ struct alignas(16) Inst {
   // face_fx is set (every |R| < 2)
   int2 Rf[kMaxCS][kMaxCS + 1][kMaxNp];
   int face_fx;
+  int rho_fx;           // every |rho| < 2: rhof holds st.rho in limbs
+  int2 rhof[kMaxCS][kMaxCS];
   // fused == 2 (where the basis is accepted): the int64 state holds w = Tbi u, the coordinates of u in a
   // basis (columns of Tb) in which every composed-step matrix G is block diagonal (2 x 2
   // blocks (2m, 2m+1), a 1 x 1 block last for odd Np) with block rows 2m equal to

@@ -7,6 +7,7 @@
 // at PE faces, the delayed / AT flux (Eqs. asyncEulerDGconserved, at-flux-gen) with the
 // ring-buffer write of the stage-input traces are fused into one kernel per stage.
 #include "adg_device.cuh"
+#include "adg_faces.cuh"
 #include "adg_fixed.cuh"
 
 #include <cstdio>
@@ -337,179 +338,7 @@ __global__ void __launch_bounds__(kTile) k_step_fused(const Inst inst, const dou
   fused_body<NP, EPT>(inst, uin, uout, blockIdx.x * (kTile * EPT), sh);
 }
 
-// What the PE-face correction of face j at step n reads besides the field: its delay k and
-// order q' (delay_at), the AT coefficients, and the upwind traces of levels n-k-i (i < q')
-// for the S stages from the ring [slot][stage][P] (zero when k = 0).
-template <int S>
-struct FaceLoads {
-  double Rv[S][kMaxQ];
-  double c[kMaxQ];
-  int k, qe, nm;   // nm: the ring slot of step n
-};
-
-template <int S>
-__device__ __forceinline__ void face_loads(const Inst &I, int j, int64_t n, FaceLoads<S> &f) {
-  const DelayAt dl = delay_at(I, j, n);
-  const int P = I.P, R = I.R;
-  const int nm = mod_step(n, R);
-  f.nm = nm;
-  const double2 *col = I.ring + j;
-  f.k = dl.k;
-  f.qe = dl.qe;
-#pragma unroll
-  for (int i = 0; i < kMaxQ; ++i) {
-    int sl = nm - (dl.k + i);
-    if (sl < 0) sl += R;
-    const bool use = dl.k > 0 && i < dl.qe;
-    f.c[i] = i < dl.qe ? dl.c[i] : 0.0;
-    const double2 *lv = col + (size_t)sl * (S * P);
-#pragma unroll
-    for (int st = 0; st < S; ++st) f.Rv[st][i] = use ? lv[st * P].x : 0.0;
-  }
-}
-
-// The synchronous traces of element e-1's stage inputs at a PE face (e the face's element):
-// T[0] = p^{e-1}, the right trace of u^{e-1}, and the channel scalars T[s] = Y_s^{e-1}_p =
-// r_s . u^{e-1} + sum_{t<s} k_st Y_t^{e-2}_p, from elements e-S .. e-1 (w = 0 .. S-1).
-template <int S>
-struct FaceTraces {
-  double T[S];
-};
-
-// The channel scalars Y_s^m_p of elements m = e-S+1 .. e-1 in FP64, from the elements
-// e-S .. e-1 (U[w], w = 0 .. S-1): element e-S+w forms Y_1 .. Y_w from its values and the
-// scalars of the element before it.
-template <int NP, int S>
-__device__ __forceinline__ FaceTraces<S> face_traces(const Inst &I, const double (*U)[NP]) {
-  const StepConsts &C = I.st;
-  double Yp[S];   // the channel scalars of the element one to the left (Yp[0] = its trace)
-  Yp[0] = U[0][NP - 1];
-#pragma unroll
-  for (int w = 1; w < S; ++w) {
-    const int ns = w;   // channels 1 .. w of element e-S+w
-    double Y[S];
-    Y[0] = U[w][NP - 1];
-#pragma unroll
-    for (int s = 1; s <= ns; ++s) {
-      double a = C.r[s][0] * U[w][0];
-#pragma unroll
-      for (int i = 1; i < NP; ++i) a = fma(C.r[s][i], U[w][i], a);
-#pragma unroll
-      for (int t = 0; t < s; ++t) a = fma(C.k[s][t], Yp[t], a);
-      Y[s] = a;
-    }
-#pragma unroll
-    for (int s = 0; s <= ns; ++s) Yp[s] = Y[s];
-  }
-  FaceTraces<S> t;
-#pragma unroll
-  for (int s = 0; s < S; ++s) t.T[s] = Yp[s];
-  return t;
-}
-
-// The right trace of an int64 element: its last value, or for block-basis coordinates the
-// sum of the first coordinate of each block, w_0 + w_2 (exact).
-template <int NP>
-__device__ __forceinline__ long long fx_trace(const Inst &I, const long long *X) {
-  if (!I.basis) return X[NP - 1];
-  return NP > 2 ? X[0] + X[2] : X[0];
-}
-
-// From int64 values X at scale 2^sig: the same sums in the composed step's two-limb integer
-// arithmetic (StepFixed coefficients) at a scale chosen from these S elements alone
-// (|X'| < 2^(56 - fxh), so the result does not depend on any other face), then rounded to
-// FP64. Off the FP64 pipe but for S conversions.
-template <int NP, int S>
-__device__ __forceinline__ FaceTraces<S> face_traces_fixed(const Inst &I, const long long (*X)[NP],
-                                                           int sig) {
-  const StepFixed &F = I.sf;
-  unsigned long long m = 0;
-#pragma unroll
-  for (int w = 0; w < S; ++w)
-#pragma unroll
-    for (int i = 0; i < NP; ++i) m |= fx_mag(X[w][i]);
-  const int L = m ? 64 - __clzll((long long)m) : 0;   // |X| < 2^(L+1)
-  const int top = 55 - I.fxh;
-  const int sh = L > top ? L - top : 0;
-  long long Yp[S];
-  {
-    long long Xs[NP];
-#pragma unroll
-    for (int i = 0; i < NP; ++i) Xs[i] = fx_rescale(X[0][i], sh);
-    Yp[0] = fx_trace<NP>(I, Xs);
-  }
-#pragma unroll
-  for (int w = 1; w < S; ++w) {
-    const int ns = w;   // channels 1 .. w of element e-S+w
-    int xh[NP], xl[NP];
-#pragma unroll
-    for (int i = 0; i < NP; ++i) fx_split(fx_rescale(X[w][i], sh), xh[i], xl[i]);
-    int ph[S], pl[S];
-#pragma unroll
-    for (int t = 0; t < S - 1; ++t)
-      if (t < ns) fx_split(Yp[t], ph[t], pl[t]);
-    long long Y[S];
-    {
-      long long Xs[NP];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) Xs[i] = fx_rescale(X[w][i], sh);
-      Y[0] = fx_trace<NP>(I, Xs);
-    }
-#pragma unroll
-    for (int s = 1; s <= ns; ++s) {
-      FxAcc acc;
-#pragma unroll
-      for (int i = 0; i < NP; ++i) fx_mac(acc, F.r[s][i], xh[i], xl[i]);
-#pragma unroll
-      for (int t = 0; t < s; ++t) fx_mac(acc, F.k[s][t], ph[t], pl[t]);
-      Y[s] = fx_round(acc);
-    }
-#pragma unroll
-    for (int s = 0; s <= ns; ++s) Yp[s] = Y[s];
-  }
-  FaceTraces<S> t;
-  t.T[0] = pow2_scale((double)fx_trace<NP>(I, X[S - 1]), sig);
-#pragma unroll
-  for (int s = 1; s < S; ++s) t.T[s] = pow2_scale((double)Yp[s], sig + sh);
-  return t;
-}
-
-// The stage differences d_s = T_s - V_s at PE face j, step n, from the synchronous traces and
-// the face's loads, and the ring write of T_s (the PE-face correction below).
-template <int S>
-__device__ __forceinline__ void face_diffs(const Inst &I, int j, const FaceLoads<S> &f,
-                                           const FaceTraces<S> &tr, double *d) {
-  const int P = I.P;
-  const StepConsts &C = I.st;
-  double2 *col = I.ring + j;
-  const int k = f.k, qe = f.qe;
-  double V[S];
-#pragma unroll
-  for (int st = 0; st < S; ++st) {
-    double v = __dmul_rn(f.c[0], f.Rv[st][0]);
-#pragma unroll
-    for (int i = 1; i < kMaxQ; ++i) {
-      if (i < qe) {
-        const double ci = f.c[i];
-        if (ci != 0.0) v = __dadd_rn(v, __dmul_rn(ci, f.Rv[st][i]));
-      }
-    }
-    V[st] = v;
-  }
-  // T_s: the traces plus the responses to the earlier stages' corrections; with zero delay
-  // V_s = T_s (the current traces), so d_s = 0
-  double2 *lv = col + (size_t)f.nm * (S * P);
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    double T = tr.T[s];
-#pragma unroll
-    for (int t = 0; t < s; ++t) T = fma(C.rho[s][t], d[t], T);
-    d[s] = k > 0 ? __dsub_rn(T, V[s]) : 0.0;
-    lv[s * P] = make_double2(T, 0.0);
-  }
-}
-
-// PE-face correction of a three-stage composed step (upwind advection, a > 0; StepConsts):
+// PE-face correction of a three-stage composed step in FP64 (upwind advection, a > 0; StepConsts):
 // thread j forms, for PE face j (e = j Kpe), the synchronous right traces of element e-1's
 // stage inputs (p, q1 = v1_p, q2 = v2_p, from elements e-3 .. e-1 with the composed step's
 // coefficients), then stage by stage T_s (those traces plus the responses to the earlier
@@ -519,29 +348,24 @@ __device__ __forceinline__ void face_diffs(const Inst &I, int j, const FaceLoads
 // for a > 0; the other slot holds 0), and adds sum_s R_s d_s to the composed (synchronous)
 // result of elements e-1 .. e+2. Every load (delay, ring levels of all three stages, inputs,
 // outputs) is issued before any of them is used. A zero delay gives d_s = 0 exactly and leaves
-// the composed result as it is. Windows of different faces are disjoint when Kpe >= 8. fmt:
-// the fixed-point step's formats (bit 0: uin, bit 1: uout int64 at the step's scale). The
-// AT sums and the stage-by-stage traces are FP64; with an int64 input the synchronous traces,
-// and with an int64 output the correction itself, are formed in the step's integer limbs (as in
-// k_face_step, so batched and single runs agree bit for bit).
-template <int NP, bool FOUT>
-__device__ __forceinline__ void fixup_body(const Inst &I, int j, const void *__restrict__ uin,
-                                           void *__restrict__ uout, int rel, bool fin) {
+// the composed result as it is. Windows of different faces are disjoint when Kpe >= 8.
+template <int NP>
+__device__ __forceinline__ void fixup_body(const Inst &I, int j, const double *__restrict__ uin,
+                                           double *__restrict__ uout, int rel) {
   const int K = I.K;
   const int e = j * I.Kpe;
   const int64_t n = I.meta[0] + rel;
-  const bool fout = FOUT;
   const StepConsts &S = I.st;
   // Loads that do not depend on the step kernel before this one (its input u^n, the delay, AT
   // coefficients and earlier ring levels) come before waiting for it (programmatic launch).
-  long long Xr[3][NP];   // raw 64-bit values of e-3 .. e-1: int64, or the bits of FP64
+  double U[3][NP];   // e-3 .. e-1
   for (int w = 0; w < 3; ++w) {
     int m = e - 3 + w;
     if (m < 0) m += K;
-    const long long *q = static_cast<const long long *>(uin) + m;
+    const double *q = uin + m;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      Xr[w][i] = *q;
+      U[w][i] = *q;
       q += K;
     }
   }
@@ -549,300 +373,249 @@ __device__ __forceinline__ void fixup_body(const Inst &I, int j, const void *__r
   face_loads<3>(I, j, n, fl);
   pdl_wait();
   pdl_trigger();
-  FxScale sc{0, 0, 0, false};
-  int sig_in = 0;
-  if (I.fused == 2) {
-    sc = fx_scale(I.fx, n, fin, I.fxh, I.fxe);
-    sig_in = I.fx[sc.slot].sigma;
-  }
   // the composed result of e-1 .. e+2 (w = 0 .. 3)
   int mw[4];
+  double Y[4][NP];
   for (int w = 0; w < 4; ++w) {
     int m = e - 1 + w;
     if (m < 0) m += K;
     if (m >= K) m -= K;
     mw[w] = m;
+    const double *q = uout + m;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      Y[w][i] = *q;
+      q += K;
+    }
   }
-  long long Xq[4][NP];
-  double Yd[4][NP];
+  const FaceTraces<3> tr = face_traces<NP, 3>(I, U);
+  double d[3];
+  face_diffs<3>(I, j, fl, tr, d);
+  if (!(nonzero(d[0]) || nonzero(d[1]) || nonzero(d[2]))) return;
   for (int w = 0; w < 4; ++w) {
-    if (fout) {
-      const long long *q = static_cast<const long long *>(uout) + mw[w];
+    double *q = uout + mw[w];
 #pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        Xq[w][i] = *q;
-        q += K;
-      }
-    } else {
-      const double *q = static_cast<const double *>(uout) + mw[w];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        Yd[w][i] = *q;
-        q += K;
-      }
+    for (int i = 0; i < NP; ++i) {
+      const double c = fma(S.R[2][w][i], d[2], fma(S.R[1][w][i], d[1], S.R[0][w][i] * d[0]));
+      *q = __dadd_rn(Y[w][i], c);
+      q += K;
     }
-  }
-  FaceTraces<3> tr;
-  if (fin) {
-    tr = face_traces_fixed<NP, 3>(I, Xr, sig_in);
-  } else {
-    double U[3][NP];
-#pragma unroll
-    for (int w = 0; w < 3; ++w)
-#pragma unroll
-      for (int i = 0; i < NP; ++i) U[w][i] = __longlong_as_double(Xr[w][i]);
-    tr = face_traces<NP, 3>(I, U);
-  }
-  double dd[3];
-  face_diffs<3>(I, j, fl, tr, dd);
-  const double d0 = dd[0], d1 = dd[1], d2 = dd[2];
-  // with a NaN or infinity in u^n the fixed-point step has already written NaN (or carries
-  // the mark); nothing is added
-  if (!(nonzero(d0) || nonzero(d1) || nonzero(d2)) || sc.bad) return;
-  int emax = 0;
-  unsigned long long mag = 0;
-  if (fout && I.face_fx) {
-    // the fixed-point step's int64 output: the integer correction of k_face_step
-    const double sf = pow2_scale(1.0, -sc.sigma);
-    const long long D0 = llrint(d0 * sf), D1 = llrint(d1 * sf), D2 = llrint(d2 * sf);
-    const long long lim = 1ll << 57;
-    if (D0 > -lim && D0 < lim && D1 > -lim && D1 < lim && D2 > -lim && D2 < lim) {
-      int h0, l0, h1, l1, h2, l2;
-      fx_split(D0, h0, l0);
-      fx_split(D1, h1, l1);
-      fx_split(D2, h2, l2);
-      for (int w = 0; w < 4; ++w) {
-        long long *q = static_cast<long long *>(uout) + mw[w];
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-          FxAcc acc;
-          fx_mac(acc, I.Rf[0][w][i], h0, l0);
-          fx_mac(acc, I.Rf[1][w][i], h1, l1);
-          fx_mac(acc, I.Rf[2][w][i], h2, l2);
-          const long long X = Xq[w][i] + fx_round(acc);
-          *q = X;
-          q += K;
-          mag |= fx_mag(X);
-        }
-      }
-      or_slot(&I.fx[fx_next(sc.slot)].mag, mag);
-      return;
-    }
-  }
-  for (int w = 0; w < 4; ++w) {   // elements e-1 .. e+2
-    if (fout) {
-      // FP64 sum (block-basis coordinates: the nodal correction times Tbi)
-      double c[NP];
-#pragma unroll
-      for (int i = 0; i < NP; ++i)
-        c[i] = fma(S.R[2][w][i], d2, fma(S.R[1][w][i], d1, S.R[0][w][i] * d0));
-      if (I.basis) {
-        double cb[NP];
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-          cb[i] = I.Tbi[i * NP] * c[0];
-#pragma unroll
-          for (int k = 1; k < NP; ++k) cb[i] = fma(I.Tbi[i * NP + k], c[k], cb[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < NP; ++i) c[i] = cb[i];
-      }
-      long long *q = static_cast<long long *>(uout) + mw[w];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        const long long X = Xq[w][i] + llrint(pow2_scale(c[i], -sc.sigma));
-        *q = X;
-        q += K;
-        mag |= fx_mag(X);
-      }
-    } else {
-      double *q = static_cast<double *>(uout) + mw[w];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        const double c = fma(S.R[2][w][i], d2, fma(S.R[1][w][i], d1, S.R[0][w][i] * d0));
-        const double y = __dadd_rn(Yd[w][i], c);
-        *q = y;
-        q += K;
-        const int be = biased_exponent(y);
-        emax = be > emax ? be : emax;
-      }
-    }
-  }
-  // the fixed-point composed step takes the scale of u^{n+1} from every value written
-  if (I.fused == 2) {
-    FxSlot &nx = I.fx[fx_next(sc.slot)];
-    if (fout) or_slot(&nx.mag, mag);
-    else raise_slot(&nx.E, emax);
   }
 }
 
+template <int NP>
+__global__ void __launch_bounds__(64) k_step_fixup(const Inst I, const double *__restrict__ uin,
+                                                   double *__restrict__ uout, int rel) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < I.P) fixup_body<NP>(I, j, uin, uout, rel);
+}
+
+// Lane r's ring traces of a face: stage r of levels n - k - i, i < q' (0 beyond, or without a
+// delay).
+template <int S>
+__device__ __forceinline__ void face_ring(const Inst &I, int j, bool on, int r, const FaceDelay &dl,
+                                          int nm, double *Rv) {
+#pragma unroll
+  for (int i = 0; i < kMaxQ; ++i) {
+    int sl = nm - (dl.k + i);
+    if (sl < 0) sl += I.R;
+    Rv[i] = on && dl.k > 0 && i < dl.qe ? I.ring[((size_t)sl * S + r) * I.P + j].x : 0.0;
+  }
+}
+
+constexpr int kFaceThreads = 128;
+
 // PE-face work of the fixed-point step between two steps, on the field u that is the output
 // of step n-1 and the input of step n (n = meta[0] + rel), for PE face j (e = j Kpe), with S
-// the composed step's stages. A block of (S+1) warps takes 32 faces, warp w element e-1+w of
-// their correction windows (so the FP64 work of the differences runs in full warps):
-//   kFaceApply: adds step n-1's correction sum_s R_s[w] d_s (its differences in I.fd, buffer
-//               (n-1) & 1) to element e-1+w of u at step n-1's working scale, with the scale
-//               bookkeeping of the values written (slot n % 3);
-//   kFaceDiff:  warp 0 then forms step n's differences d_s from elements e-S .. e-1 of u
-//               (e-1 as corrected) and the ring (face_diffs), writes the ring slot of step n
-//               and I.fd buffer n & 1.
+// the composed step's stages and a group of kFaceLanes<S> lanes per face:
+//   kFaceApply: lane r <= S adds step n-1's correction sum_s R_s[r] d_s (its differences in
+//               I.fd, buffer (n-1) & 1) to element e-1+r of u at step n-1's working scale,
+//               with the scale bookkeeping of the values written (slot n % 3);
+//   kFaceDiff:  the group then forms step n's differences d_s from elements e-S .. e-1 of u
+//               (e-1 as corrected) and the ring, writes the ring slot of step n and I.fd
+//               buffer n & 1.
 // fu: u is int64 (at the scale of slot n % 3), else FP64; fin_prev: step n-1 read int64. Every
 // load is issued before any value is used; the windows of different faces (e-S .. e+S-1) are
 // disjoint when Kpe >= 2S.
 template <int NP, int S>
-__global__ void __launch_bounds__(32 * (S + 1)) k_face_step(const Inst I, void *__restrict__ u,
-                                                          int rel, int fu, int fin_prev,
-                                                          int mode) {
-  const int j = blockIdx.x * 32 + (threadIdx.x & 31), w = threadIdx.x >> 5;
-  if (j >= I.P) return;
-  const int K = I.K, P = I.P;
+__global__ void __launch_bounds__(kFaceThreads) k_face_step(const Inst I, void *__restrict__ u,
+                                                            int rel, int fu, int fin_prev,
+                                                            int mode) {
+  const int jt = (blockIdx.x * kFaceThreads + threadIdx.x) / kFaceLanes<S>;
+  const bool act = jt < I.P;
+  const int j = act ? jt : I.P - 1;
+  const FaceGroup g = face_group<S>();
+  const int K = I.K, P = I.P, r = g.r;
   const int e = j * I.Kpe;
   const int64_t n = I.meta[0] + rel;
-  const bool diff = (mode & kFaceDiff) && w == 0;
+  const bool on = act && r < S, win = act && r <= S;
   long long *uq = static_cast<long long *>(u);
-  int m = e - 1 + w;   // this thread's element; warp 0 also reads e-S .. e-2
-  if (m < 0) m += K;
-  if (m >= K) m -= K;
+  int mw = e - 1 + r, mt = e - S + r;   // this lane's element of the window, of the traces
+  if (mw < 0) mw += K;
+  if (mw >= K) mw -= K;
+  if (mt < 0) mt += K;
   // The delay, AT coefficients and ring levels of steps before n do not depend on the step
   // kernel before this one: loaded before waiting for it (programmatic launch).
-  FaceLoads<S> fl;
-  if (diff) face_loads<S>(I, j, n, fl);
+  FaceDelay dl{};
+  double Rv[kMaxQ];
+  const int nm = mod_step(n, I.R);
+  if (mode & kFaceDiff) {
+    dl = face_delay(I, I.table[(n - I.meta[1]) * P + j], n);
+    face_ring<S>(I, j, on, r, dl, nm, Rv);
+  }
+  const int *c = I.coefi + (dl.k * I.q + dl.qe - 1) * I.q;
+  long long V = 0;
+  int be = 0;
+  if (mode & kFaceDiff) face_ahead<S>(I, g, Rv, c, dl.k > 0 ? dl.qe : 0, V, be);
   pdl_wait();
   pdl_trigger();
-  long long V[S][NP];   // raw 64-bit values (int64, or the bits of FP64): e-S .. e-2, own
-  {
-    const long long *q = uq + m;
+  // raw 64-bit values (int64, or the bits of FP64)
+  long long W[NP], X[NP];
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      V[S - 1][i] = *q;
-      q += K;
-    }
-  }
-  if (diff) {
+  for (int i = 0; i < NP; ++i) W[i] = win ? uq[(size_t)i * K + mw] : 0;
 #pragma unroll
-    for (int b = 0; b < S - 1; ++b) {
-      int mb = e - S + b;
-      if (mb < 0) mb += K;
-      const long long *q = uq + mb;
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        V[b][i] = *q;
-        q += K;
-      }
-    }
-  }
+  for (int i = 0; i < NP; ++i) X[i] = (mode & kFaceDiff) && on && r < S - 1 ? uq[(size_t)i * K + mt] : 0;
   if (mode & kFaceApply) {
-    const double *dd = I.fd + (size_t)((n - 1) & 1) * S * P + S * (size_t)j;
+    const double *fd = I.fd + (size_t)((n - 1) & 1) * S * P + S * (size_t)j;
     double d[S];
-    bool any = false;
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      d[s] = dd[s];
-      any = any || nonzero(d[s]);
-    }
+    for (int s = 0; s < S; ++s) d[s] = fd[s];
+    double dr = 0.0;
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      if (r == s) dr = d[s];
     const FxScale sc = fx_scale(I.fx, n - 1, fin_prev != 0, I.fxh, I.fxe);
-    if (any && !sc.bad) {
-      bool done = false;
-      if (fu && I.face_fx) {
-        // D_s = round(d_s 2^-sigma) and sum_s R_s D_s in the step's two-limb arithmetic
-        const double sf = pow2_scale(1.0, -sc.sigma);
-        const long long lim = 1ll << 57;
-        long long D[S];
-        bool inr = true;
+    int dh[S], dlo[S];
+    const int how = face_limbs<S>(I, g, on, dr, sc.sigma, dh, dlo);
+    if (how && !sc.bad && win) {
+      long long add[NP];
+      if (fu && how == 1) {
+        face_correction<NP, S>(I, r, dh, dlo, add);
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-          D[s] = llrint(d[s] * sf);
-          inr = inr && D[s] > -lim && D[s] < lim;
-        }
-        if (inr) {
-          int hh[S], ll[S];
+        for (int i = 0; i < NP; ++i) W[i] += add[i];
+      } else if (fu) {
+        face_correction_fp64<NP, S>(I, r, d, sc.sigma, add);
 #pragma unroll
-          for (int s = 0; s < S; ++s) fx_split(D[s], hh[s], ll[s]);
-#pragma unroll
-          for (int i = 0; i < NP; ++i) {
-            FxAcc acc;
-#pragma unroll
-            for (int s = 0; s < S; ++s) fx_mac(acc, I.Rf[s][w][i], hh[s], ll[s]);
-            V[S - 1][i] += fx_round(acc);
-          }
-          done = true;
-        }
-      }
-      if (!done) {
-        // FP64: an FP64 output, or a difference beyond the integer range (block-basis
-        // coordinates: the nodal correction times Tbi)
-        const StepConsts &C = I.st;
-        double c[NP];
+        for (int i = 0; i < NP; ++i) W[i] += add[i];
+      } else {
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
-          c[i] = C.R[0][w][i] * d[0];
+          double x = I.st.R[0][r][i] * d[0];
 #pragma unroll
-          for (int s = 1; s < S; ++s) c[i] = fma(C.R[s][w][i], d[s], c[i]);
-        }
-        if (fu && I.basis) {
-          double cb[NP];
-#pragma unroll
-          for (int i = 0; i < NP; ++i) {
-            cb[i] = I.Tbi[i * NP] * c[0];
-#pragma unroll
-            for (int k = 1; k < NP; ++k) cb[i] = fma(I.Tbi[i * NP + k], c[k], cb[i]);
-          }
-#pragma unroll
-          for (int i = 0; i < NP; ++i) c[i] = cb[i];
-        }
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-          if (fu) V[S - 1][i] += llrint(pow2_scale(c[i], -sc.sigma));
-          else V[S - 1][i] = __double_as_longlong(__dadd_rn(__longlong_as_double(V[S - 1][i]), c[i]));
+          for (int s = 1; s < S; ++s) x = fma(I.st.R[s][r][i], d[s], x);
+          W[i] = __double_as_longlong(__dadd_rn(__longlong_as_double(W[i]), x));
         }
       }
       int emax = 0;
       unsigned long long mag = 0;
-      long long *q = uq + m;
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
-        const long long X = V[S - 1][i];
-        *q = X;
-        q += K;
-        if (fu) {
-          mag |= fx_mag(X);
-        } else {
-          const int be = biased_exponent(__longlong_as_double(X));
-          emax = be > emax ? be : emax;
-        }
+        uq[(size_t)i * K + mw] = W[i];
+        if (fu) mag |= fx_mag(W[i]);
+        else emax = max(emax, biased_exponent(__longlong_as_double(W[i])));
       }
       FxSlot &nx = I.fx[fx_next(sc.slot)];
       if (fu) or_slot(&nx.mag, mag);
       else raise_slot(&nx.E, emax);
     }
   }
-  if (diff) {
-    FaceTraces<S> tr;
-    if (fu) {
-      tr = face_traces_fixed<NP, S>(I, V, I.fx[(int)(n % 3)].sigma);
-    } else {
-      double U[S][NP];
+  if (mode & kFaceDiff) {
 #pragma unroll
-      for (int b = 0; b < S; ++b)
-#pragma unroll
-        for (int i = 0; i < NP; ++i) U[b][i] = __longlong_as_double(V[b][i]);
-      tr = face_traces<NP, S>(I, U);
+    for (int i = 0; i < NP; ++i) {   // element e-1, as corrected by the group's first lane
+      const long long x = __shfl_sync(kFullWarp, W[i], g.base);
+      if (r == S - 1) X[i] = x;
     }
-    double d[S];
-    face_diffs<S>(I, j, fl, tr, d);
-    double *o = I.fd + (size_t)(n & 1) * S * P + S * (size_t)j;
+    const double T0 = fu ? face_trace_fixed<NP, S>(I, g, on, X, I.fx[mod_step(n, 3)].sigma)
+                         : face_trace_fp64<NP, S>(I, g, on, X);
+    double T, d;
+    face_differences<S>(I, g, on && dl.k > 0, T0, V, be, c, dl.qe,
+                        [&](int i, int s) {
+                          double x = 0.0;
 #pragma unroll
-    for (int s = 0; s < S; ++s) o[s] = d[s];
+                          for (int q = 0; q < kMaxQ; ++q)
+                            if (q == i) x = Rv[q];
+                          return __shfl_sync(kFullWarp, x, g.base + s);
+                        },
+                        T, d);
+    if (on) {
+      I.ring[((size_t)nm * S + r) * P + j] = make_double2(T, 0.0);
+      I.fd[(size_t)(n & 1) * S * P + S * (size_t)j + r] = d;
+    }
   }
 }
 
+// The PE-face correction of one batched fixed-point step (int64 output) by a group of lanes:
+// the differences of step n from its input and the ring, and their correction of its output;
+// the values of k_face_step, so that batched and single runs agree bit for bit.
 template <int NP>
-__global__ void __launch_bounds__(64) k_step_fixup(const Inst I, const void *__restrict__ uin,
-                                                   void *__restrict__ uout, int rel, int fmt) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= I.P) return;
-  if (fmt & kFmtOutFixed) fixup_body<NP, true>(I, j, uin, uout, rel, (fmt & kFmtInFixed) != 0);
-  else fixup_body<NP, false>(I, j, uin, uout, rel, (fmt & kFmtInFixed) != 0);
+__device__ __forceinline__ void fixup_fixed(const Inst &I, int j, bool act,
+                                            const void *__restrict__ uin, void *__restrict__ uout,
+                                            int rel, bool fin) {
+  constexpr int S = kStages;
+  const FaceGroup g = face_group<S>();
+  const int K = I.K, r = g.r;
+  const int e = j * I.Kpe;
+  const int64_t n = I.meta[0] + rel;
+  const bool on = act && r < S;
+  int mw = e - 1 + r, mt = e - S + r;
+  if (mw < 0) mw += K;
+  if (mw >= K) mw -= K;
+  if (mt < 0) mt += K;
+  // as in k_face_step; the step's input does not depend on the step kernel before this one
+  long long X[NP];
+#pragma unroll
+  for (int i = 0; i < NP; ++i) X[i] = on ? static_cast<const long long *>(uin)[(size_t)i * K + mt] : 0;
+  const FaceDelay dl = face_delay(I, I.table[(n - I.meta[1]) * I.P + j], n);
+  const int nm = mod_step(n, I.R);
+  double Rv[kMaxQ];
+  face_ring<S>(I, j, on, r, dl, nm, Rv);
+  const int *c = I.coefi + (dl.k * I.q + dl.qe - 1) * I.q;
+  long long V = 0;
+  int be = 0;
+  face_ahead<S>(I, g, Rv, c, dl.k > 0 ? dl.qe : 0, V, be);
+  // the input's scale and its slot were complete before the step kernel ran
+  const FxScale sc = fx_scale(I.fx, n, fin, I.fxh, I.fxe);
+  const double T0 = fin ? face_trace_fixed<NP, S>(I, g, on, X, I.fx[sc.slot].sigma)
+                        : face_trace_fp64<NP, S>(I, g, on, X);
+  double T, dr;
+  face_differences<S>(I, g, on && dl.k > 0, T0, V, be, c, dl.qe,
+                      [&](int i, int s) {
+                        double x = 0.0;
+#pragma unroll
+                        for (int q = 0; q < kMaxQ; ++q)
+                          if (q == i) x = Rv[q];
+                        return __shfl_sync(kFullWarp, x, g.base + s);
+                      },
+                      T, dr);
+  int dh[S], dlo[S];
+  const int how = face_limbs<S>(I, g, on, dr, sc.sigma, dh, dlo);
+  long long add[NP];
+  if (how == 2) {
+    double d[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) d[s] = __shfl_sync(kFullWarp, dr, g.base + s);
+    face_correction_fp64<NP, S>(I, r, d, sc.sigma, add);
+  } else {
+    face_correction<NP, S>(I, r, dh, dlo, add);
+  }
+  pdl_wait();
+  pdl_trigger();
+  if (on) I.ring[((size_t)nm * S + r) * I.P + j] = make_double2(T, 0.0);
+  // with a NaN or infinity in u^n the step carries the mark; nothing is added
+  const bool write = act && how && !sc.bad;
+  unsigned long long mag = 0;
+  if (write) {
+    long long *q = static_cast<long long *>(uout) + mw;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const long long y = q[(size_t)i * K] + add[i];
+      q[(size_t)i * K] = y;
+      mag |= fx_mag(y);
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < kFaceLanes<S>; o *= 2) mag |= __shfl_xor_sync(kFullWarp, mag, o);
+  if (write && r == 0) or_slot(&I.fx[fx_next(sc.slot)].mag, mag);
 }
 
 // Batched composed steps: block b takes work item (instance, first element); `parity`
@@ -870,26 +643,45 @@ __global__ void __launch_bounds__(kTile) k_batch_fused(const Inst *__restrict__ 
   }
 }
 
-// The PE-face corrections of a batched composed step, one thread per PE face of any instance:
-// fflat lists (instance, face) for every PE face of every instance, so the threads of a block
-// are all busy however few faces an instance has.
-// FOUT: the step wrote int64 (fixed point), else FP64 (the FP64 composed step).
-template <bool FOUT>
+// The PE-face corrections of a batched composed step over fflat, the (instance, face) of every PE
+// face of every instance, ordered and padded (face -1) so that each eight entries have one
+// degree: FP64, one thread per face.
 __global__ void __launch_bounds__(64) k_batch_fixup(const Inst *__restrict__ insts,
                                                     const int2 *__restrict__ fflat, int nflat,
-                                                    int src, int dst, bool fin, int rel) {
+                                                    int src, int rel) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nflat) return;
   const int2 w = fflat[t];
+  if (w.y < 0) return;
   const Inst &I = insts[w.x];
-  const int j = w.y;
+  const double *uin = src == 0 ? I.u : I.v1;
+  double *uout = src == 0 ? I.v1 : I.u;
+  switch (I.Np) {
+    case 2: fixup_body<2>(I, w.y, uin, uout, rel); break;
+    case 3: fixup_body<3>(I, w.y, uin, uout, rel); break;
+    case 4: fixup_body<4>(I, w.y, uin, uout, rel); break;
+    default: fixup_body<5>(I, w.y, uin, uout, rel); break;
+  }
+}
+
+// Fixed point: a group of four lanes per face, a warp's eight faces of one degree.
+__global__ void __launch_bounds__(kFaceThreads) k_batch_fixup_fixed(const Inst *__restrict__ insts,
+                                                                    const int2 *__restrict__ fflat,
+                                                                    int nflat, int src, int dst,
+                                                                    bool fin, int rel) {
+  const int t = (blockIdx.x * kFaceThreads + threadIdx.x) / kFaceLanes<kStages>;
+  if (t >= nflat) return;   // whole warps: nflat is a multiple of eight
+  int2 w = fflat[t];
+  const bool act = w.y >= 0;
+  w.y = act ? w.y : 0;
+  const Inst &I = insts[w.x];
   const void *uin = src == 0 ? (const void *)I.u : (src == 1 ? (const void *)I.v1 : (const void *)I.v2);
   void *uout = dst == 0 ? (void *)I.u : (dst == 1 ? (void *)I.v1 : (void *)I.v2);
   switch (I.Np) {
-    case 2: fixup_body<2, FOUT>(I, j, uin, uout, rel, fin); break;
-    case 3: fixup_body<3, FOUT>(I, j, uin, uout, rel, fin); break;
-    case 4: fixup_body<4, FOUT>(I, j, uin, uout, rel, fin); break;
-    default: fixup_body<5, FOUT>(I, j, uin, uout, rel, fin); break;
+    case 2: fixup_fixed<2>(I, w.y, act, uin, uout, rel, fin); break;
+    case 3: fixup_fixed<3>(I, w.y, act, uin, uout, rel, fin); break;
+    case 4: fixup_fixed<4>(I, w.y, act, uin, uout, rel, fin); break;
+    default: fixup_fixed<5>(I, w.y, act, uin, uout, rel, fin); break;
   }
 }
 
@@ -1242,8 +1034,9 @@ cudaError_t fused_np(const Inst &I, const void *uin, void *uout, int rel, cudaSt
     else
       k_step_fused<NP, 1><<<(unsigned)((I.K + kTile - 1) / kTile), kTile, 0, s>>>(I, ui, uo);
   }
-  if (I.async && with_fixup)
-    k_step_fixup<NP><<<(unsigned)((I.P + 63) / 64), 64, 0, s>>>(I, uin, uout, rel, fmt);
+  if (I.fused == 1 && I.async && with_fixup)
+    k_step_fixup<NP><<<(unsigned)((I.P + 63) / 64), 64, 0, s>>>(
+        I, static_cast<const double *>(uin), static_cast<double *>(uout), rel);
   return cudaGetLastError();
 }
 }  // namespace
@@ -1251,7 +1044,8 @@ cudaError_t fused_np(const Inst &I, const void *uin, void *uout, int rel, cudaSt
 template <int S>
 cudaError_t face_step_s(const Inst &I, void *u, int rel, int fu, int fin_prev, int mode,
                         cudaStream_t s, bool pdl) {
-  const dim3 g((unsigned)((I.P + 31) / 32)), b(32 * (S + 1));   // 32 faces per block
+  const unsigned per = kFaceThreads / kFaceLanes<S>;   // faces of a block
+  const dim3 g((unsigned)((I.P + per - 1) / per)), b(kFaceThreads);
   switch (I.Np) {
     case 2: return launch_maybe_pdl(k_face_step<2, S>, g, b, s, pdl, I, u, rel, fu, fin_prev, mode);
     case 3: return launch_maybe_pdl(k_face_step<3, S>, g, b, s, pdl, I, u, rel, fu, fin_prev, mode);
@@ -1336,12 +1130,10 @@ cudaError_t launch_batch_fused_step(const Inst *insts_dev, const int2 *work_dev,
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (nfwork > 0) {
-    // a programmatic dependent of the step kernel: its input, delay and ring loads overlap it
-    const dim3 g((unsigned)((nfwork + 63) / 64)), b(64);
+    // a programmatic dependent of the step kernel: all but the correction itself overlaps it
     const bool fin = (fmt & kFmtInFixed) != 0;
     // the fix-up is the short, latency-bound link between a part's steps: its blocks take
-    // SM resources ahead of the other parts' queued step blocks (64 threads a block: 32
-    // measured 0.3329 against 0.3324 ms per batched step)
+    // SM resources ahead of the other parts' queued step blocks
     static int prio = [] {
       int least = 0, greatest = 0;
       if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess) {
@@ -1350,12 +1142,14 @@ cudaError_t launch_batch_fused_step(const Inst *insts_dev, const int2 *work_dev,
       }
       return greatest;
     }();
+    const int per = kFaceThreads / kFaceLanes<kStages>;
     if (fmt & kFmtOutFixed)
-      e = launch_pdl_priority(k_batch_fixup<true>, g, b, s, true, prio, insts_dev, fwork_dev,
-                              nfwork, src, dst, fin, rel);
+      e = launch_pdl_priority(k_batch_fixup_fixed, dim3((unsigned)((nfwork + per - 1) / per)),
+                              dim3(kFaceThreads), s, true, prio, insts_dev, fwork_dev, nfwork, src, dst,
+                              fin, rel);
     else
-      e = launch_pdl_priority(k_batch_fixup<false>, g, b, s, true, prio, insts_dev, fwork_dev,
-                              nfwork, src, dst, fin, rel);
+      e = launch_pdl_priority(k_batch_fixup, dim3((unsigned)((nfwork + 63) / 64)), dim3(64), s, true,
+                              prio, insts_dev, fwork_dev, nfwork, src, rel);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
