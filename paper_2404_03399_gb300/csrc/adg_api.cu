@@ -352,6 +352,7 @@ struct InstHost {
   double *ringq = nullptr;   // viscous Burgers: the PE faces' -2 nu q^+
   adg::FxSlot *fx = nullptr; // scale slots of the fixed-point composed step
   double *fd = nullptr;      // ... and its PE faces' stage differences [2][P][3]
+  void *run = nullptr;       // ... and the run kernel's exchange slots and flags
   bool fixed_ok = false;     // the composed coefficients fit the fixed-point bounds
   std::vector<uint8_t> host_rows;
 };
@@ -402,6 +403,8 @@ struct adg_ctx {
   int G = 32;                      // steps per graph (128 measured slower: 78.5 against
                                    // 77.2 ms for 2000 steps of the adjoint workload)
   int64_t n = 0;
+  // set by a kernel whose bounded wait ran out (mapped host memory, read after a synchronisation)
+  int *timeout() const { return reinterpret_cast<int *>(pinned + 7); }
 };
 
 namespace {
@@ -1312,6 +1315,21 @@ void fold_step_constants(InstHost &h, bool allow_basis) {
     }
 }
 
+int ensure_pinned(adg_ctx *c) {
+  if (c->pinned) return ADG_OK;
+  CK(cudaMallocHost(&c->pinned, 8 * sizeof(double)));
+  *c->timeout() = 0;
+  return ADG_OK;
+}
+
+// Waits for the context's stream; a bounded device wait that ran out shows here.
+int sync_stream(adg_ctx *c) {
+  CK(cudaStreamSynchronize(c->stream));
+  if (c->pinned && *static_cast<volatile int *>(c->timeout()))
+    return fail(c, ADG_ETIMEOUT, "a run kernel's wait for its other blocks ran out");
+  return ADG_OK;
+}
+
 int reduce(adg_ctx *c, InstHost &h, int kind, const double *g, double scale, double *host_out,
            const double *field = nullptr) {
   if (!c->partials) {
@@ -1320,13 +1338,15 @@ int reduce(adg_ctx *c, InstHost &h, int kind, const double *g, double scale, dou
     CK(cudaMalloc(&c->partials, 1025 * sizeof(double)));
     c->red_out = c->partials + 1024;
   }
-  if (!c->pinned) CK(cudaMallocHost(&c->pinned, 8 * sizeof(double)));
+  int r0 = ensure_pinned(c);
+  if (r0) return r0;
   const int nb = adg::reduce_blocks(h.I.K);
   const double *wm = kind == 3 ? h.M : h.w;
   CK(adg::launch_reduce(kind, field ? field : h.I.u, g, h.I.K, h.I.Np, wm, scale, c->partials, nb,
                         c->red_out, c->stream));
   CK(cudaMemcpyAsync(c->pinned, c->red_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  r0 = sync_stream(c);
+  if (r0) return r0;
   *host_out = c->pinned[0];
   return ADG_OK;
 }
@@ -1562,7 +1582,8 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
     if (!coef.empty())
       CK(cudaMemcpyAsync(h.coef, coef.data(), coef.size() * sizeof(double),
                          cudaMemcpyHostToDevice, c->stream));
-    if (!c->pinned) CK(cudaMallocHost(&c->pinned, 8 * sizeof(double)));
+    int r0 = ensure_pinned(c);
+    if (r0) return r0;
     int *emax = reinterpret_cast<int *>(c->pinned);
     CK(cudaMemcpyAsync(emax, c->scan, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -1651,6 +1672,9 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
       if (!c->batch) {
         int r2 = autotune_fused(c, h);
         if (r2) return r2;
+        // the run kernel, unless the caller forced the step kernel's elements per thread
+        const size_t bytes = cfg->ept ? 0 : adg::fixed_run_bytes(I);
+        if (bytes) CK(cudaMalloc(&h.run, bytes));
       }
     }
   }
@@ -1706,6 +1730,7 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
 constexpr int kChunkFP64 = 3;
 // Steps per directly launched chunk (at most half the delay-table window of 512 rows).
 constexpr int kDirectChunk = 256;
+static_assert(kDirectChunk <= adg::kRunSteps, "a chunk is one run kernel launch");
 
 int fixed_end(int from, int64_t m) {
   if (m == 0) return from;
@@ -1925,6 +1950,20 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
 // v1 / v2 in int64) and alternates v1 and v2.
 int launch_fused_steps(adg_ctx *c, int nsteps, int kind) {
   const Inst &I = c->inst[0].I;
+  if (c->inst[0].run && nsteps > 1) {
+    // the run kernel, int64 -> int64 (a step from FP64 first)
+    void *const f[3] = {I.u, I.v1, I.v2};
+    int from = kind == kChunkFP64 ? 0 : kind, rel = 0;
+    if (from == 0) {
+      CK(adg::launch_fused_step(I, I.u, I.v1, 0, c->stream, true, adg::kFmtOutFixed));
+      from = rel = 1;
+    }
+    const int end = fixed_end(kind == kChunkFP64 ? 0 : kind, nsteps);
+    CK(adg::launch_fixed_run(I, adg::fixed_run(c->inst[0].run, c->timeout()), f[from], f[end], rel,
+                             nsteps - rel, c->stream));
+    CK(adg::launch_advance(c->meta, 2, 1, nsteps, c->stream));
+    return ADG_OK;
+  }
   if (I.fused == 2) {
     // With PE faces, one face kernel before the chunk's first step forms its differences,
     // one between consecutive steps adds the earlier step's correction and forms the next
@@ -2422,6 +2461,7 @@ void adg_destroy(adg_ctx *c) {
     cudaFree(h.M);
     cudaFree(h.fx);
     cudaFree(h.fd);
+    cudaFree(h.run);
     cudaFree(h.ringq);
   }
   cudaFree(c->meta);
@@ -2821,7 +2861,7 @@ int adg_step(adg_ctx *c, int64_t nsteps) {
   const bool carry = fixed_state(c);
   // CUDA graphs of G steps where launches dominate; larger runs launch chunks of up to
   // kDirectChunk steps directly (direct_launches)
-  const bool graphs = !direct_launches(c);
+  const bool graphs = !direct_launches(c) && !c->inst[0].run;
   int64_t left = nsteps;
   while (left > 0) {
     const int chunk = (int)std::min<int64_t>(left, graphs ? c->G : kDirectChunk);
@@ -2866,7 +2906,10 @@ int adg_get_state(adg_ctx *c, int32_t index, double *u_dev, int64_t *step_out) {
     int r0 = state_rows(c, c->inst[index], u_dev);
     if (r0) return r0;
   }
-  CK(cudaStreamSynchronize(c->stream));
+  {
+    int r0 = sync_stream(c);
+    if (r0) return r0;
+  }
   if (step_out) *step_out = c->n;
   return ADG_OK;
 }
@@ -2893,7 +2936,10 @@ int adg_get_state_host(adg_ctx *c, int32_t index, double *u_host, int64_t *step_
   }
   if (!view)
     CK(cudaMemcpyAsync(u_host, dst, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  {
+    int r0 = sync_stream(c);
+    if (r0) return r0;
+  }
   if (step_out) *step_out = c->n;
   return ADG_OK;
 }

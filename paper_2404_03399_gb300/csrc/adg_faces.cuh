@@ -1,5 +1,6 @@
 // PE faces of the composed steps (upwind advection, a > 0): the loads of a face, the synchronous
-// traces of its element's stage inputs and the stage differences (adg_kernels.cu).
+// traces of its element's stage inputs and the stage differences, shared by the face kernels
+// (adg_kernels.cu) and the fixed-point run kernel (adg_fixed_run.cu).
 #pragma once
 
 #include "adg_bfp.cuh"
@@ -116,7 +117,7 @@ __device__ __forceinline__ void face_diffs(const Inst &I, int j, const FaceLoads
 // the stages' values side by side take a third of one thread's (a lane per face), and the
 // integers about half of FP64's, whose instruction holds a sub-partition's pipe for 64
 // clocks. Every function is called by all 32 lanes of a warp together, those without a face too
-// (shuffles under a mask known only at run time are slower).
+// (under a mask known only at run time the shuffles cost the run kernel a microsecond a step).
 constexpr unsigned kFullWarp = 0xffffffffu;
 template <int S>
 constexpr int kFaceLanes = S <= 3 ? 4 : 8;

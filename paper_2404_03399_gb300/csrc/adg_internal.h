@@ -286,6 +286,21 @@ cudaError_t launch_fused_step(const Inst &I, const void *uin, void *uout, int re
 // The fixed-point composed step alone (adg_fixed.cu).
 cudaError_t launch_fixed_step(const Inst &I, const void *uin, void *uout, int rel, int fmt,
                               cudaStream_t s, bool pdl = false);
+// A run of fixed-point composed steps in one cooperative launch (adg_fixed_run.cu; meshes of up
+// to about 900 elements per SM): its device buffer's size (0: the instance takes the step and
+// face kernels), the buffer's parts, and nsteps steps from the int64 field in (state of step
+// meta[0] + rel) to out (the same results as launch_fixed_step and launch_face_step). *err
+// (host-mapped) is set when its bounded wait ran out.
+struct FixedRun {
+  void *words;
+  long long *exch;
+  int *err;
+};
+constexpr int kRunSteps = 256;   // of one launch
+size_t fixed_run_bytes(const Inst &I);
+FixedRun fixed_run(void *buf, int *err);
+cudaError_t launch_fixed_run(const Inst &I, const FixedRun &R, const void *in, void *out, int rel,
+                             int nsteps, cudaStream_t s);
 // A launch with the programmatic-stream-serialization attribute when pdl is set.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_maybe_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
