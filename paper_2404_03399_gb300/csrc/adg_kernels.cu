@@ -589,15 +589,12 @@ __device__ __forceinline__ void fixup_fixed(const Inst &I, int j, bool act,
                       T, dr);
   int dh[S], dlo[S];
   const int how = face_limbs<S>(I, g, on, dr, sc.sigma, dh, dlo);
-  long long add[NP];
-  if (how == 2) {
-    double d[S];
+  double d[S];   // in every lane (the groups of a warp may differ in `how`)
 #pragma unroll
-    for (int s = 0; s < S; ++s) d[s] = __shfl_sync(kFullWarp, dr, g.base + s);
-    face_correction_fp64<NP, S>(I, r, d, sc.sigma, add);
-  } else {
-    face_correction<NP, S>(I, r, dh, dlo, add);
-  }
+  for (int s = 0; s < S; ++s) d[s] = __shfl_sync(kFullWarp, dr, g.base + s);
+  long long add[NP];
+  if (how == 2) face_correction_fp64<NP, S>(I, r, d, sc.sigma, add);
+  else face_correction<NP, S>(I, r, dh, dlo, add);
   pdl_wait();
   pdl_trigger();
   if (on) I.ring[((size_t)nm * S + r) * I.P + j] = make_double2(T, 0.0);
