@@ -9,6 +9,7 @@
 #include <complex>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <memory>
 #include <new>
 #include <string>
@@ -366,6 +367,7 @@ struct adg_ctx {
   std::string err;
   cudaStream_t stream = nullptr;
   cudaStream_t cap = nullptr;
+  cudaMemPool_t pool = nullptr;   // working memory of the gradient and the misfit
   int device = 0;
   std::vector<InstHost> inst;
   bool batch = false;
@@ -1888,11 +1890,11 @@ int launch_steps(adg_ctx *c, int nsteps, int kind = kChunkFP64) {
   }
   if (!c->batch && c->inst[0].I.pde == ADG_BURGERS) {
     const Inst &I = c->inst[0].I;
-    const bool pdl = direct_launches(c);
     int r = launch_alternating(c, nsteps, 1, (size_t)I.K * I.Np * sizeof(double),
                                [&](double *in, double *out, int rel, int) {
-                                 return adg::launch_burgers_step(I, in, out, nullptr, nullptr, rel,
-                                                                 c->stream, pdl && rel > 0);
+                                 return adg::launch_burgers_step(I, in, out, nullptr, nullptr,
+                                                                 c->n + rel, c->inst[0].tbase,
+                                                                 c->stream, rel > 0);
                                });
     if (r) return r;
     CK(adg::launch_advance(c->meta, 2, (int)c->inst.size(), nsteps, c->stream));
@@ -2048,21 +2050,49 @@ int begin_ctx(adg_ctx *c, void *stream) {
   return ADG_OK;
 }
 
-// Device memory owned for the duration of one adg_grad call.
+// Device memory owned for the duration of one call, from the context's pool in the order of its
+// stream (work on other streams that uses it is joined to that stream before it is freed).
 struct DevBuf {
   void *p = nullptr;
+  cudaStream_t s = nullptr;
   ~DevBuf() {
-    if (p) cudaFree(p);
+    if (p) cudaFreeAsync(p, s);
   }
   double *d() const { return static_cast<double *>(p); }
 };
 
+// The context's memory pool (the gradient's and the misfit's working fields): it keeps up to
+// kPoolKeep bytes between calls, which a repeated gradient would otherwise allocate and free
+// each time (some 1 ms for the 65536-element workload), and is destroyed with the context.
+constexpr uint64_t kPoolKeep = uint64_t(1) << 30;
+
+cudaError_t pool_alloc(adg_ctx *c, DevBuf &b, size_t bytes) {
+  if (!c->pool) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = c->device;
+    cudaError_t e = cudaMemPoolCreate(&c->pool, &props);
+    if (e != cudaSuccess) {
+      c->pool = nullptr;
+      return e;
+    }
+    uint64_t keep = kPoolKeep;
+    e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) return e;
+  }
+  cudaError_t e = cudaMallocFromPoolAsync(&b.p, bytes, c->pool, c->stream);
+  if (e != cudaSuccess) b.p = nullptr;
+  b.s = c->stream;
+  return e;
+}
+
 int dev_alloc(adg_ctx *c, DevBuf &b, size_t bytes) {
   if (bytes == 0) return ADG_OK;
-  cudaError_t e = cudaMalloc(&b.p, bytes);
+  cudaError_t e = pool_alloc(c, b, bytes);
   if (e != cudaSuccess) {
-    b.p = nullptr;
-    return fail(c, ADG_ENOMEM, std::string("adg_grad: cudaMalloc: ") + cudaGetErrorString(e));
+    (void)cudaGetLastError();
+    return fail(c, ADG_ENOMEM, std::string("working memory: ") + cudaGetErrorString(e));
   }
   return ADG_OK;
 }
@@ -2109,17 +2139,15 @@ int capture(adg_ctx *c, GraphExec &out, F &&body) {
   return ADG_OK;
 }
 
-// Forward over one segment of `len` steps starting at meta[0], recording the stage inputs
+// Forward over one segment of `len` steps starting at step n, recording the stage inputs
 // of step t in slot t of `seg` (u^n, v1, v2); slot t+1's u receives u^{n+1}, so slot 0's u
 // must hold the segment's first state and slot len's u holds the last.
-// rel0 shifts the step indices: a segment that starts rel0 steps after meta[0] (the
-// overlapped recompute runs the segment before the one meta[0] names, rel0 = -len).
-int sweep_recompute(adg_ctx *c, InstHost &h, double *seg, int len, int rel0 = 0) {
+int sweep_recompute(adg_ctx *c, InstHost &h, double *seg, int len, int64_t n, cudaStream_t st) {
   const size_t nd = (size_t)h.I.K * h.I.Np;
   for (int t = 0; t < len; ++t) {
     double *slot = seg + (size_t)t * kStages * nd;
-    CK(adg::launch_burgers_step(h.I, slot, slot + kStages * nd, slot + nd, slot + 2 * nd, rel0 + t,
-                                c->stream));
+    CK(adg::launch_burgers_step(h.I, slot, slot + kStages * nd, slot + nd, slot + 2 * nd, n + t,
+                                h.tbase, st, t > 0));
   }
   return ADG_OK;
 }
@@ -2135,7 +2163,8 @@ int sweep_reverse(adg_ctx *c, InstHost &h, const double *seg, double *lam, doubl
   for (int t = len - 1; t >= 0; --t) {
     double *Lu = lam + (size_t)par * nd, *Lacc = lam + (size_t)(1 - par) * nd;
     if (seg) {   // Burgers: one kernel per step
-      CK(adg::launch_burgers_adj(I, seg + (size_t)t * kStages * nd, Lu, Lacc, lring, t, c->stream));
+      CK(adg::launch_burgers_adj(I, seg + (size_t)t * kStages * nd, Lu, Lacc, lring, c->n + t,
+                                 h.tbase, c->stream, t < len - 1));
       par = 1 - par;
       continue;
     }
@@ -2192,6 +2221,7 @@ struct SideStream {
   cudaStream_t s = nullptr;
   cudaEvent_t meta_set = nullptr, rec_done = nullptr;
   ~SideStream() {
+    if (s) cudaStreamSynchronize(s);   // before the buffers it uses are freed, on every path
     if (meta_set) cudaEventDestroy(meta_set);
     if (rec_done) cudaEventDestroy(rec_done);
     if (s) cudaStreamDestroy(s);
@@ -2205,9 +2235,7 @@ struct SideStream {
 //
 // Burgers with two or more segments: the recompute of segment s-1 runs on a second stream
 // into a second segment buffer while the adjoint of segment s runs on the context's stream
-// (the two share only read-only data, the delay table and meta[0]; the recompute's step
-// indices are taken relative to segment s's start, so meta[0] changes only once both are
-// done). Order per segment s on the context's stream: wait for the recompute of s, refill
+// (the two share only read-only data and the delay table). Order per segment s on the context's stream: wait for the recompute of s, refill
 // the delay table if it does not cover steps [start(s) - C, end(s)), set meta[0] = start(s),
 // record `meta_set`, run the adjoint of s; on the second stream: wait for `meta_set` (which
 // also orders it after the adjoint of s+1, the last reader of the buffer it overwrites),
@@ -2221,13 +2249,24 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
   const int K = I.K, Np = I.Np;
   const size_t nd = (size_t)K * Np;
   const int64_t n0 = c->n;
-  const int64_t nseg = nsteps == 0 ? 0 : (nsteps + C - 1) / C;
   const bool states = I.pde == ADG_BURGERS;
+  DevBuf g, ck_u, ck_ring, seg, lam, lring, ck_fx;
+  // a segment's delays are one window of the table; and a run whose recorded stage inputs all
+  // fit in what the pool keeps is one segment, recorded on the way (nothing is recomputed; the
+  // gradient does not depend on C)
+  if (I.async) C = std::min(C, h.TR);
+  if (states && nsteps > C && nsteps <= (I.async ? h.TR : std::numeric_limits<int>::max()) &&
+      ((size_t)nsteps * kStages + 1) * nd * sizeof(double) <= kPoolKeep) {
+    if (pool_alloc(c, seg, ((size_t)nsteps * kStages + 1) * nd * sizeof(double)) == cudaSuccess)
+      C = (int)nsteps;
+    else
+      (void)cudaGetLastError();
+  }
+  const int64_t nseg = nsteps == 0 ? 0 : (nsteps + C - 1) / C;
   const int64_t nck = states ? nseg : std::min<int64_t>(nseg, 1);
   const size_t ring_n = I.async ? (size_t)I.R * kStages * I.P : 0;
   const int dir = I.a >= 0.0 ? 1 : -1;
 
-  DevBuf g, ck_u, ck_ring, seg, lam, lring, ck_fx;
   // the fixed-point state (int64 field and its scale slots) is put back exactly at the end
   const int live0 = c->fx_live;
   int r = ADG_OK;
@@ -2242,7 +2281,7 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
   r = dev_alloc(c, g, nd * sizeof(double));
   if (!r) r = dev_alloc(c, ck_u, (size_t)nck * nd * sizeof(double));
   if (!r) r = dev_alloc(c, ck_ring, (size_t)nck * ring_n * sizeof(double2));
-  if (!r && states) r = dev_alloc(c, seg, ((size_t)C * kStages + 1) * nd * sizeof(double));
+  if (!r && states && !seg.p) r = dev_alloc(c, seg, ((size_t)C * kStages + 1) * nd * sizeof(double));
   if (!r) r = dev_alloc(c, lam, 4 * nd * sizeof(double));
   if (!r) r = dev_alloc(c, lring, ring_n * sizeof(double));
   if (r) return r;
@@ -2250,7 +2289,6 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
 
   // Forward pass with checkpoints (u^n and the forward ring at each segment start). The last
   // segment's stage inputs are recorded on the way, so it is not recomputed.
-  GraphExec rec_full, rec_last;
   const int64_t last_len = nseg > 0 ? nsteps - (nseg - 1) * C : 0;
   for (int64_t sidx = 0; sidx < nseg; ++sidx) {
     if (sidx < nck) {
@@ -2265,10 +2303,8 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
       if (!r) r = set_step(c, h, c->n);
       if (r) return r;
       CK(cudaMemcpyAsync(seg.d(), I.u, nd * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-      GraphExec &ge = len == C ? rec_full : rec_last;
-      r = capture(c, ge, [&] { return sweep_recompute(c, h, seg.d(), len); });
+      r = sweep_recompute(c, h, seg.d(), len, c->n, c->stream);
       if (r) return r;
-      CK(cudaGraphLaunch(ge.g, c->stream));
       CK(cudaMemcpyAsync(I.u, seg.d() + (size_t)len * kStages * nd, nd * sizeof(double),
                          cudaMemcpyDeviceToDevice, c->stream));
       r = set_step(c, h, c->n + len);
@@ -2291,8 +2327,7 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
   SideStream side;
   bool overlap = states && nseg >= 2 && (!I.async || 2 * (int64_t)C <= h.TR);
   if (overlap) {
-    if (cudaMalloc(&seg2.p, ((size_t)C * kStages + 1) * nd * sizeof(double)) != cudaSuccess) {
-      seg2.p = nullptr;
+    if (pool_alloc(c, seg2, ((size_t)C * kStages + 1) * nd * sizeof(double)) != cudaSuccess) {
       (void)cudaGetLastError();   // clear the failed allocation; run segments serially
       overlap = false;
     }
@@ -2304,9 +2339,9 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
   }
   double *segb[2] = {seg.d(), seg2.d()};
 
-  // Segment sweeps replay graphs captured once per (segment length, buffer parity, segment
-  // buffer); the overlapped recompute has one graph per segment buffer.
-  GraphExec rev[2][2][2], rec_prev[2];
+  // Advection's reverse sweeps (three kernels a step) replay graphs captured once per (segment
+  // length, buffer parity).
+  GraphExec rev[2][2];
   int par = 0, cur = 0;
   for (int64_t sidx = nseg - 1; sidx >= 0; --sidx) {
     const int64_t start = n0 + sidx * C;
@@ -2333,12 +2368,8 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
         if (ring_n)
           CK(cudaMemcpyAsync(I.ring, static_cast<double2 *>(ck_ring.p) + (sidx - 1) * ring_n,
                              ring_n * sizeof(double2), cudaMemcpyDeviceToDevice, side.s));
-        GraphExec &gp = rec_prev[1 - cur];
-        if (!gp.g) {
-          r = capture(c, gp, [&] { return sweep_recompute(c, h, nb, C, -C); });
-          if (r) return r;
-        }
-        CK(cudaGraphLaunch(gp.g, side.s));
+        r = sweep_recompute(c, h, nb, C, start - C, side.s);
+        if (r) return r;
         CK(cudaEventRecord(side.rec_done, side.s));
       }
     } else {
@@ -2351,21 +2382,23 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
         if (ring_n)
           CK(cudaMemcpyAsync(I.ring, static_cast<double2 *>(ck_ring.p) + sidx * ring_n,
                              ring_n * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
-        GraphExec &ge = is_last ? rec_last : rec_full;
-        if (!ge.g) {
-          r = capture(c, ge, [&] { return sweep_recompute(c, h, seg.d(), len); });
-          if (r) return r;
-        }
-        CK(cudaGraphLaunch(ge.g, c->stream));
+        r = sweep_recompute(c, h, seg.d(), len, start, c->stream);
+        if (r) return r;
       }
     }
-    double *sb = states ? segb[cur] : nullptr;
-    GraphExec &gr = rev[is_last ? 1 : 0][par][cur];
-    if (!gr.g) {
-      r = capture(c, gr, [&] { return sweep_reverse(c, h, sb, lam.d(), lring.d(), len, par); });
+    if (states) {
+      // one kernel per step: launched directly (capturing and instantiating the sweeps' graphs
+      // took about 0.9 of the 3.9 ms of 100 steps on 65536 elements)
+      r = sweep_reverse(c, h, segb[cur], lam.d(), lring.d(), len, par);
       if (r) return r;
+    } else {
+      GraphExec &gr = rev[is_last ? 1 : 0][par];
+      if (!gr.g) {
+        r = capture(c, gr, [&] { return sweep_reverse(c, h, nullptr, lam.d(), lring.d(), len, par); });
+        if (r) return r;
+      }
+      CK(cudaGraphLaunch(gr.g, c->stream));
     }
-    CK(cudaGraphLaunch(gr.g, c->stream));
     if (len % 2) par = 1 - par;
     if (overlap) cur = 1 - cur;
   }
@@ -2478,6 +2511,7 @@ void adg_destroy(adg_ctx *c) {
   cudaFree(c->partials);   // red_out lies inside it
   if (c->pinned) cudaFreeHost(c->pinned);
   if (c->cap) cudaStreamDestroy(c->cap);
+  if (c->pool) cudaMemPoolDestroy(c->pool);
   delete c;
 }
 
@@ -2861,7 +2895,9 @@ int adg_step(adg_ctx *c, int64_t nsteps) {
   const bool carry = fixed_state(c);
   // CUDA graphs of G steps where launches dominate; larger runs launch chunks of up to
   // kDirectChunk steps directly (direct_launches)
-  const bool graphs = !direct_launches(c) && !c->inst[0].run;
+  // (Burgers steps, one launch each, directly too, as programmatic dependents)
+  const bool graphs =
+      !direct_launches(c) && !c->inst[0].run && c->inst[0].I.pde != ADG_BURGERS;
   int64_t left = nsteps;
   while (left > 0) {
     const int chunk = (int)std::min<int64_t>(left, graphs ? c->G : kDirectChunk);

@@ -5,19 +5,22 @@
 // clock per SM), a 32 x 32 -> 64-bit integer product the heavy FMA pipe of one of the four
 // sub-partitions for 4, and shifts and adds run beside it. A stage evaluated in FP64 is bound
 // by that pipe (73-84 FP64 instructions per element at p = 4), so the stages here load FP64
-// values, bring the elements of one warp to a common scale, work in integers, and round once
+// values, bring each element to a scale of its neighbourhood, work in integers, and round once
 // to FP64 when the step is done.
 //
-// A warp's values are X = x 2^(57 - E), |x| < 2^E over all of its elements, so |X| < 2^57 at
-// the start of the step; every intermediate value is checked to stay below 2^58. Squares and
-// face fluxes are held in units of 2^(2E - 56): G = X^2 2^-58. An operator coefficient c is
-// C = round(c 2^(58 - sc)), |C| <= 2^58, split as in adg_fixed.cuh, and sums of products are
-// rounded once. Against FP64: a value is exact to 2^-57 of the warp's largest; the warp takes
-// this path only if every non-zero element reaches 2^-6 of that largest value (kBfSpan), so
-// an element's error per stage is at most about 2^-51 of its own largest value, as the chain of
-// FP64 roundings gives; other warps (and exponents near the ends of the FP64 range, NaN,
-// infinities, growth past the headroom within a step, Courant numbers whose coefficients
-// do not fit) take the FP64 stages.
+// An element's values are X = x 2^(57 - E), |x| < 2^E over the element and those that reach it
+// within the step (one on either side per stage), so |X| < 2^57 at the start of the step;
+// every intermediate value is checked to stay below 2^58, and what comes from a neighbour is
+// shifted from its scale. Squares and face fluxes are held in units of 2^(2E - 56): G = X^2
+// 2^-58. An operator coefficient c is C = round(c 2^(58 - sc)), |C| <= 2^58, split as in
+// adg_fixed.cuh, and sums of products are rounded once. Against FP64: a value is exact to 2^-57
+// of the largest one near it; the integer path is taken only if every non-zero element reaches
+// 2^-6 of that largest value (kBfSpan), so an element's error per stage is at most about 2^-51
+// of its own largest value, as the chain of FP64 roundings gives. Warps with an element outside
+// that (or exponents near the ends of the FP64 range, NaN, infinities, growth past the headroom
+// within a step, Courant numbers whose coefficients do not fit) take the FP64 stages, some
+// 8 us for a warp: with one scale per warp instead, the warps at a smooth wave's zeros did, and
+// were the longest part of a step on 65536 elements (13 of 14 us).
 #pragma once
 
 #include "adg_fixed.cuh"
@@ -25,8 +28,8 @@
 namespace adg {
 namespace {
 
-constexpr int kBfSpan = 6;      // exponent span of a warp's elements on the integer path
-constexpr int kBfMinE = 600;    // biased exponents of the warp's largest value
+constexpr int kBfSpan = 6;      // exponent of an element below its scale on the integer path
+constexpr int kBfMinE = 600;    // biased exponents of the scales
 constexpr int kBfMaxE = 1400;
 constexpr int kBfTop = 58;      // every intermediate value below 2^kBfTop
 
@@ -84,6 +87,26 @@ constexpr int kThirdHi = (int)((kThird - kThirdLo) >> 29);
 // v 2^-d (d < 0: a left shift; the caller has checked that the result fits).
 __device__ __forceinline__ long long bf_shift(long long v, int d) {
   return d >= 0 ? v >> d : (long long)((unsigned long long)v << (-d));
+}
+
+// A neighbour's value v brought to this lane's unit, d exponents above the neighbour's (rounded);
+// raises `mag` past the headroom where it does not stay below 2^60.
+__device__ __forceinline__ long long bf_bring(long long v, int d, unsigned long long &mag) {
+  if (d == 0) return v;
+  d = d > 62 ? 62 : d;
+  if (d > 0) return (v + (1ll << (d - 1))) >> d;
+  if (d < -60 || (fx_mag(v) >> (60 + d)) != 0) {
+    mag |= v ? 1ull << kBfTop : 0ull;
+    return 0;
+  }
+  return (long long)((unsigned long long)v << (-d));
+}
+
+// The largest of x over the lanes within n of this one.
+__device__ __forceinline__ int bf_window_max(int x, int n) {
+  for (int k = 0; k < n; ++k)
+    x = max(x, max(__shfl_up_sync(0xffffffffu, x, 1), __shfl_down_sync(0xffffffffu, x, 1)));
+  return x;
 }
 
 }  // namespace

@@ -28,23 +28,52 @@ __device__ __forceinline__ int warp_element(int K, int warp, int lane, int H, in
 template <bool VISC>
 constexpr int kFaceVals = VISC ? 3 : 1;
 
-// Value `which` of ring level n - m (slot sl): flux and u^- in I.ring, y in I.ringq.
-__device__ __forceinline__ double ring_value(const Inst &I, int which, int sl, int s, int j) {
-  const size_t at = ((size_t)sl * I.ns + s) * I.P + j;
-  return which == 0 ? I.ring[at].x : (which == 1 ? I.ring[at].y : I.ringq[at]);
+// The delay of PE face j at step n and its AT coefficients, from the step and the first row of
+// the delay table as the host knows them (one load ahead of the coefficients and the ring).
+__device__ __forceinline__ DelayAt step_delay(const Inst &I, int j, int64_t n, int64_t tbase) {
+  int64_t k = I.table[(n - tbase) * I.P + j];
+  if (k > n) k = n;
+  const int64_t qe = n - k + 1 < I.q ? n - k + 1 : I.q;
+  return {(int)k, (int)qe, I.coef + ((size_t)k * I.q + (qe - 1)) * I.q};
 }
 
-// The delayed / AT value of PE face j at stage s (d.k > 0) from the ring.
-__device__ __forceinline__ double ring_sum(const Inst &I, const DelayAt &d, int which, int j, int nm,
-                                           int s) {
-  double V = 0.0;
-  for (int i = 0; i < d.qe; ++i) {
+// The delayed / AT values of PE face j (d.k > 0) at stages s0 .. s0 + NS - 1, NV of them each (the
+// flux, u^-, y), into V[value * S + stage][lane]; every level's load is issued before any is
+// used.
+template <int NV, int NS>
+__device__ __forceinline__ void ring_sums(const Inst &I, const DelayAt &d, int j, int nm, int S, int s0,
+                                          double (*V)[32], int &fmax, int &umax) {
+  const int lane = threadIdx.x & 31;
+  double c[kMaxQ], x[NS][NV][kMaxQ];
+#pragma unroll
+  for (int i = 0; i < kMaxQ; ++i) {
     int sl = nm - d.k - i;
     if (sl < 0) sl += I.R;
-    const double x = __dmul_rn(d.c[i], ring_value(I, which, sl, s, j));
-    V = i ? __dadd_rn(V, x) : x;
+    const bool use = i < d.qe;
+    c[i] = use ? d.c[i] : 0.0;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const size_t at = ((size_t)sl * I.ns + s0 + s) * I.P + j;
+      x[s][0][i] = use ? I.ring[at].x : 0.0;
+      if constexpr (NV == 3) {
+        x[s][1][i] = use ? I.ring[at].y : 0.0;
+        x[s][2][i] = use ? I.ringq[at] : 0.0;
+      }
+    }
   }
-  return V;
+#pragma unroll
+  for (int s = 0; s < NS; ++s)
+#pragma unroll
+    for (int w = 0; w < NV; ++w) {
+      double v = __dmul_rn(c[0], x[s][w][0]);
+#pragma unroll
+      for (int i = 1; i < kMaxQ; ++i)
+        if (i < d.qe) v = __dadd_rn(v, __dmul_rn(c[i], x[s][w][i]));
+      V[w * S + s0 + s][lane] = v;
+      const int h = __double2hiint(v) & 0x7fffffff;
+      if (w == 0) fmax = max(fmax, h);
+      if (w == 1) umax = max(umax, h);
+    }
 }
 
 // Fields of a step and what it writes besides.
@@ -52,7 +81,8 @@ struct StepArgs {
   const double *uin;
   double *uout;
   double *r1, *r2;   // REC: the inputs of stages 1 and 2
-  int rel, H, HR;
+  int64_t n, tbase;   // the step, and the first step of the delay table
+  int H, HR;
 };
 
 // The step in FP64 (warps that the integer path does not take): stage by stage in the staged
@@ -182,7 +212,7 @@ __device__ __forceinline__ void burgers_operator(const BurgersFixed &B, const lo
 // (BurgersFixed). REC also writes the stage inputs v1, v2 (recorded sweeps of the gradient).
 // VISC: with (g, F) = (2 v, uhat) the same operator gives Z = -dt q of the local DG method
 // (uhat = u^-), and (g, F) = (v^2 - 2 nu q, F - nu qhat) (qhat = q^+) the whole dt L; Z is
-// brought to 58 bits by its largest value over the warp, since smooth fields leave it far
+// brought to 58 bits by its largest value in the element, since smooth fields leave it far
 // below its bound.
 // Bound by instruction issue (integer). K = 2^20, p = 4, ADG-AT2, SSP-RK3: 0.50 ms a step as
 // three FP64 stage kernels (80% of the FP64 pipe, eight field passes), 0.078 ms so; K = 10125,
@@ -213,27 +243,22 @@ __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ In
   int fmax = 0, umax = 0;   // largest high words of the delayed fluxes and traces
   if (FACES) {
     const int j = e / I.Kpe;
-    const int64_t n = I.meta[0] + A.rel;
-    nm = mod_step(n, I.R);
+    nm = mod_step(A.n, I.R);
     pe = e == j * I.Kpe;
     if (pe) {
-      const DelayAt d = delay_at(I, j, n);
+      const DelayAt d = step_delay(I, j, A.n, A.tbase);
       late = d.k > 0;
       if (late) {
-        for (int s = 0; s < S; ++s)
-#pragma unroll
-          for (int w = 0; w < NV; ++w) {
-            const double V = ring_sum(I, d, w, j, nm, s);
-            sV[w * S + s][lane] = V;
-            const int h = __double2hiint(V) & 0x7fffffff;
-            if (w == 0) fmax = max(fmax, h);
-            if (w == 1) umax = max(umax, h);
-          }
+if constexpr (!LS && !VISC) {
+          ring_sums<1, kStages>(I, d, j, nm, S, 0, sV, fmax, umax);
+        } else {
+          for (int s = 0; s < S; ++s) ring_sums<NV, 1>(I, d, j, nm, S, s, sV, fmax, umax);
+        }
       }
     }
   }
 
-  // the warp's scale, and whether the integer path takes it
+  // the element's scale, and whether the integer path takes the warp
   int hi = 0;
   unsigned lo = 0;
 #pragma unroll
@@ -241,7 +266,7 @@ __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ In
     hi = max(hi, __double2hiint(ud[i]) & 0x7fffffff);
     lo |= (unsigned)__double2loint(ud[i]);
   }
-  const int be = __reduce_max_sync(full, hi) >> 20;
+  const int be = bf_window_max(hi >> 20, S);
   const int E = be - 1022;              // |u| < 2^E
   const BurgersFixed &B = I.bf;
   const int d0 = -(B.sc + E + 1);       // operator sums -> value units (inviscid)
@@ -253,6 +278,8 @@ __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ In
 
   if (!__any_sync(full, bad)) {
     const int sg = 2 * E - 56;   // unit of the squares and fluxes
+    // scales of the neighbours below this lane's
+    const int dEL = E - __shfl_up_sync(full, E, 1), dER = E - __shfl_down_sync(full, E, 1);
     long long u[NP], v[NP];      // u: u^n, or dU of a 2N scheme
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
@@ -268,33 +295,40 @@ __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ In
         fx_split(v[i], xh, xl);
         G[i] = bf_square(xh, xl);
       }
-      const long long vl = __shfl_up_sync(full, v[NP - 1], 1);
-      const long long gl = __shfl_up_sync(full, G[NP - 1], 1);
+      long long vl = __shfl_up_sync(full, v[NP - 1], 1);
+      long long gl = __shfl_up_sync(full, G[NP - 1], 1);
+      if (dEL != 0) {   // rarely: most neighbours have one scale
+        vl = bf_bring(vl, dEL, mag);
+        int xh, xl;
+        fx_split(vl, xh, xl);
+        gl = bf_square(xh, xl);
+      }
       long long FL = bf_llf(vl, v[0], gl, G[0]);
       const size_t at = FACES && pe ? ((size_t)nm * I.ns + s) * I.P + e / I.Kpe : 0;
       if (FACES && pe) {
         if (own) I.ring[at] = make_double2(bf_to(FL, sg), VISC ? bf_to(vl, E - 57) : 0.0);
         if (late) FL = bf_from(sV[s][lane], 2 * E + 1023);
       }
-      int d = d0;
+      int d = d0, uf = sg;   // unit of the nodes' and faces' fluxes
       if (VISC) {
         long long uL = vl;
         if (FACES && late) uL = bf_from(sV[S + s][lane], be + 1) << 1;
-        const long long uN = __shfl_down_sync(full, uL, 1);
-        const long long uR = FACES && lane < 31 ? uN : v[NP - 1];   // v_p but at delayed faces
+        const long long uN = bf_bring(__shfl_down_sync(full, uL, 1), dER, mag);
+        const bool lateR = FACES && __shfl_down_sync(full, late ? 1 : 0, 1) != 0 && lane < 31;
+        const long long uR = lateR ? uN : v[NP - 1];   // v_p but at delayed faces
         long long g2[NP], Z[NP];
 #pragma unroll
         for (int i = 0; i < NP; ++i) g2[i] = 2 * v[i];
         burgers_operator<NP>(B, g2, uL, uR, 0, Z);
-        // Z 2^nz below 2^58 over the warp
+        // Z 2^nz below 2^58
         unsigned zh = 0;
 #pragma unroll
         for (int i = 0; i < NP; ++i) zh = max(zh, (unsigned)(fx_mag(Z[i]) >> 32));
-        zh = __reduce_max_sync(full, zh);
         const int nz = __clz((int)zh) - 6;   // bit length of |Z| at most 64 - clz(zh)
         // y = -2 nu q = (2 nu / dt) Z: limbs of (2 nu / dt) 2^-sn, in units of 2^uq
         const int uq = B.sc + E - 57 - nz + B.sn;
-        const int uphi = max(uq, sg), sq = min(uphi - uq, 60), sf = min(uphi - sg, 60);
+        uf = max(uq, sg);
+        const int sq = min(uf - uq, 60), sf = min(uf - sg, 60);
         const long long hq = sq > 0 ? 1ll << (sq - 1) : 0, hf = sf > 0 ? 1ll << (sf - 1) : 0;
         long long y0 = 0;
 #pragma unroll
@@ -309,22 +343,24 @@ __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ In
         }
         FL = (FL + hf) >> sf;
         if (FACES && pe) {
-          if (own) I.ringq[at] = bf_to(y0, uphi);
+          if (own) I.ringq[at] = bf_to(y0, uf);
           if (late) {
             const double y = sV[2 * S + s][lane];
-            // |y| < 2^(uphi + 58)
-            if (((__double2hiint(y) & 0x7fffffff) >> 20) > uphi + 1080) mag |= 1ull << kBfTop;
-            else y0 = bf_from(y, uphi + 1080) << 1;
+            // |y| < 2^(uf + 58)
+            if (((__double2hiint(y) & 0x7fffffff) >> 20) > uf + 1080) mag |= 1ull << kBfTop;
+            else y0 = bf_from(y, uf + 1080) << 1;
           }
         }
         FL += (y0 + 1) >> 1;
-        d = -(B.sc + uphi - E + 57);
+        d = -(B.sc + uf - E + 57);
         if (d < -2) {
           mag |= 1ull << kBfTop;
           d = -2;
         }
       }
-      const long long FR = __shfl_down_sync(full, FL, 1);
+      const int dF = VISC ? uf - __shfl_down_sync(full, uf, 1) : 2 * dER;
+      long long FR = __shfl_down_sync(full, FL, 1);
+      if (dF != 0) FR = bf_bring(FR, dF, mag);
       // shift of the operator's sums: in SSP-RK3 stage 1 takes a quarter of them, stage 2
       // (inside the sum divided by 3) twice
       if (!LS) d = s == 0 ? d : (s == 1 ? d + 2 : d - 1);
@@ -396,7 +432,7 @@ struct AdjArgs {
   const double *w;
   double *out;
   double *lring;
-  int rel;
+  int64_t n, tbase;
 };
 
 // Partial derivatives of the local Lax-Friedrichs flux (adg_adjoint.cu), doubled and in
@@ -424,15 +460,15 @@ __device__ __forceinline__ void llf_partials_fp64(double a, double b, double &dl
 }
 
 // A PE face in the reverse sweep: the flux adjoint mu of the stage is posted, times the AT
-// coefficients, to the delayed levels' ring entries (its owner only).
+// coefficients, to the delayed levels' ring entries (its owner only; one addition per entry in
+// a step, so the atomic's order does not matter and its latency is not waited for).
 __device__ __forceinline__ void post_levels(const Inst &I, double *lring, int j, int nm, int s,
                                             int k, int qe, const double *c, double mu) {
   for (int i = 0; i < qe; ++i) {
     if (k + i < 1 || c[i] == 0.0) continue;
     int sl = nm - k - i;
     if (sl < 0) sl += I.R;
-    double *q = lring + ((size_t)sl * kStages + s) * I.P + j;
-    *q += c[i] * mu;
+    atomicAdd(lring + ((size_t)sl * kStages + s) * I.P + j, c[i] * mu);
   }
 }
 
@@ -497,7 +533,7 @@ __device__ __noinline__ void burgers_adj_fp64(const Inst &I, const AdjArgs &A, i
 
 // The adjoint of one SSP-RK3 step of inviscid Burgers, from the recorded stage inputs: the
 // layout and the integer arithmetic of k_burgers_step, with a second scale for the adjoint
-// (Ew: |w| < 2^Ew over the warp). For the adjoint w of a stage's output the adjoint of its
+// (|w| < 2^Ew near the element). For the adjoint w of a stage's output the adjoint of its
 // input v is beta (w + Z),
 //   Z_j = 2 v_j (W^T w)_j + (mu_L dF_L/du^+ at j = 0) + (mu_R dF_R/du^- at j = p),
 // mu the flux adjoints a . w^e + b . w^{e-1}; W^T, a and b act on sums and differences of
@@ -512,6 +548,8 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
                                                      const __grid_constant__ AdjArgs A) {
   constexpr int HP = NP / 2, MID = NP % 2;
   __shared__ double sR_[FACES ? 4 * kStages : 1][32];
+  pdl_wait();
+  pdl_trigger();
   const int K = I.K;
   const size_t nd = (size_t)K * NP;
   const int lane = threadIdx.x & 31;
@@ -532,11 +570,10 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
   int rmax = 0;
   if (FACES) {
     const int j = e / I.Kpe;
-    const int64_t n = I.meta[0] + A.rel;
-    nm = (int)(n % I.R);
+    nm = mod_step(A.n, I.R);
     pe = e == j * I.Kpe;
     if (pe) {
-      const DelayAt d = delay_at(I, j, n);
+      const DelayAt d = step_delay(I, j, A.n, A.tbase);
       k = d.k;
       qe = d.qe;
       c = d.c;
@@ -551,8 +588,8 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
     }
   }
 
-  // the scales: of the adjoint (every non-zero element near the warp's largest, as in the
-  // forward step), and of the stage inputs (2^E, which enter as factors of w)
+  // the scales: of the adjoint (as the forward step's), and of the stage inputs of the element
+  // and its neighbours (2^E, which enter as factors of w)
   int hw = 0, hv = 0;
   unsigned lo = 0;
 #pragma unroll
@@ -562,7 +599,7 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
 #pragma unroll
     for (int s = 0; s < kStages; ++s) hv = max(hv, __double2hiint(yd[s][i]) & 0x7fffffff);
   }
-  const int bw = __reduce_max_sync(full, hw) >> 20, bv = __reduce_max_sync(full, hv) >> 20;
+  const int bw = bf_window_max(hw >> 20, kStages), bv = bf_window_max(hv >> 20, 1);
   const int Ew = bw - 1022, E = bv - 1022;
   const int d0 = -(I.bf.sc + E + 1) - 2;   // (2 P + P') -> units of w
   bool bad = bw < kBfMinE || bw > kBfMaxE || bv < kBfMinE || bv > kBfMaxE || d0 < -3 || !I.bf.ok;
@@ -573,6 +610,9 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
   if (!__any_sync(full, bad)) {
     const BurgersFixed &B = I.bf;
     const int smu = I.bf.sc + Ew - 57;   // unit of the flux adjoints
+    // scales of the neighbours below this lane's
+    const int dWL = Ew - __shfl_up_sync(full, Ew, 1), dWR = Ew - __shfl_down_sync(full, Ew, 1);
+    const int dVL = E - __shfl_up_sync(full, E, 1);
     const int d = d0 > 60 ? 60 : d0;
     const long long half = d > 0 ? 1ll << (d - 1) : 0;
     long long w[NP], acc[NP];
@@ -611,9 +651,11 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
 #pragma unroll
       for (int i = 0; i < HP; ++i) fx_mac(ao, B.D[i][HP + MID], th[i], tl[i]);
       const long long ev = fx_round(ae), od = fx_round(ao);
-      long long mu = ev + od + __shfl_up_sync(full, od - ev, 1);
+      // (|od - ev| < 2^62: brought with two bits less)
+      const long long bl = bf_bring(__shfl_up_sync(full, (od - ev + 2) >> 2, 1), dWL, mag);
+      long long mu = ev + od + 4 * bl;
       long long dl, dr;
-      bf_llf_partials2(__shfl_up_sync(full, v[NP - 1], 1), v[0], dl, dr);
+      bf_llf_partials2(bf_bring(__shfl_up_sync(full, v[NP - 1], 1), dVL, mag), v[0], dl, dr);
       if (FACES && pe) {
         const long long r = bf_from(sR[s][lane], B.sc + Ew + 1025) << 3;
         mag |= fx_mag(mu) >> 4;   // below 2^62
@@ -630,7 +672,9 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
       const long long pl = mul(mh, ml, xh, xl);
       fx_split(dr, xh, xl);
       const long long pr = mul(mh, ml, xh, xl);
-      const long long pR = __shfl_down_sync(full, pl, 1);
+      // the left element's part, in units of this lane's w, from the lane above
+      if (d < 0 && (fx_mag(pl) >> (kBfTop + d))) mag |= 1ull << kBfTop;
+      const long long pR = bf_bring(__shfl_down_sync(full, bf_shift(pl + half, d), 1), dWR, mag);
 #pragma unroll
       for (int j = 0; j < HP + MID; ++j) {
         // half the sum and half the difference of (W^T w)_j and (W^T w)_{p-j}
@@ -652,9 +696,8 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
           fx_split(v[q], vh, vl);
           long long z = 2 * mul(rh, rl, vh, vl) + half;
           if (q == 0) z += pr;
-          if (q == NP - 1) z += pR;
           if (d < 0 && (fx_mag(z) >> (kBfTop + d))) mag |= 1ull << kBfTop;
-          const long long x = w[q] + bf_shift(z, d);
+          const long long x = w[q] + bf_shift(z, d) + (q == NP - 1 ? pR : 0);
           mag |= fx_mag(x);
           if (s == 2) {
             acc[q] = third(w[q]);
@@ -704,34 +747,33 @@ cudaError_t burgers_np(const Inst &I, const StepArgs &A, cudaStream_t s, bool pd
 }
 
 template <int NP>
-cudaError_t burgers_adj_np(const Inst &I, const AdjArgs &A, cudaStream_t s) {
+cudaError_t burgers_adj_np(const Inst &I, const AdjArgs &A, cudaStream_t s, bool pdl) {
   const int64_t warps = ((int64_t)I.K + kOwn - 1) / kOwn;
   const int bs = burgers_block(warps);
-  const unsigned g = (unsigned)((warps * 32 + bs - 1) / bs);
-  if (I.async) k_burgers_adj<NP, true><<<g, bs, 0, s>>>(I, A);
-  else k_burgers_adj<NP, false><<<g, bs, 0, s>>>(I, A);
-  return cudaGetLastError();
+  const dim3 g((unsigned)((warps * 32 + bs - 1) / bs)), b(bs);
+  return I.async ? launch_maybe_pdl(k_burgers_adj<NP, true>, g, b, s, pdl, I, A)
+                 : launch_maybe_pdl(k_burgers_adj<NP, false>, g, b, s, pdl, I, A);
 }
 
 }  // namespace
 
 cudaError_t launch_burgers_adj(const Inst &I, const double *y, const double *w, double *out,
-                               double *lring, int rel, cudaStream_t s) {
+                               double *lring, int64_t n, int64_t tbase, cudaStream_t s, bool pdl) {
   if (w == out) return cudaErrorInvalidValue;
-  const AdjArgs A{y, w, out, lring, rel};
+  const AdjArgs A{y, w, out, lring, n, tbase};
   switch (I.Np) {
-    case 2: return burgers_adj_np<2>(I, A, s);
-    case 3: return burgers_adj_np<3>(I, A, s);
-    case 4: return burgers_adj_np<4>(I, A, s);
-    case 5: return burgers_adj_np<5>(I, A, s);
+    case 2: return burgers_adj_np<2>(I, A, s, pdl);
+    case 3: return burgers_adj_np<3>(I, A, s, pdl);
+    case 4: return burgers_adj_np<4>(I, A, s, pdl);
+    case 5: return burgers_adj_np<5>(I, A, s, pdl);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_burgers_step(const Inst &I, const double *uin, double *uout, double *r1,
-                                double *r2, int rel, cudaStream_t s, bool pdl) {
+                                double *r2, int64_t n, int64_t tbase, cudaStream_t s, bool pdl) {
   if (uin == uout || (r1 && (I.ls || I.visc))) return cudaErrorInvalidValue;
-  const StepArgs A{uin, uout, r1, r2, rel, I.ns, I.ns + (I.visc ? 1 : 0)};
+  const StepArgs A{uin, uout, r1, r2, n, tbase, I.ns, I.ns + (I.visc ? 1 : 0)};
   switch (I.Np) {
     case 2: return I.async ? burgers_np<2, true>(I, A, s, pdl) : burgers_np<2, false>(I, A, s, pdl);
     case 3: return I.async ? burgers_np<3, true>(I, A, s, pdl) : burgers_np<3, false>(I, A, s, pdl);
