@@ -1291,6 +1291,10 @@ void fold_step_constants(InstHost &h, bool allow_basis) {
       h.I.Tb[i] = (double)Tm[i];
       h.I.Tbi[i] = (double)Tim[i];
     }
+    ld top = 0;
+    for (int i = 0; i < Np * Np; ++i) top = std::max(top, std::fabs(Tm[i]));
+    std::frexp(top, &h.I.sT);
+    for (int i = 0; i < Np * Np; ++i) h.I.Tf[i] = limbs58(std::ldexp(Tm[i], -h.I.sT));
   }
   // the PE-face responses likewise (from the long double values), for the integer correction
   // of differences below 2^57

@@ -160,6 +160,8 @@ struct alignas(16) Inst {
   // 2^(E - 1079 + fxe) (fxe >= fxh + log2 of the row sums of Tbi).
   int basis, fxh, fxe, pad0_;
   double Tb[kMaxNp * kMaxNp], Tbi[kMaxNp * kMaxNp];
+  int2 Tf[kMaxNp * kMaxNp];   // Tb 2^-sT (at most 1 in magnitude) in limbs as in StepFixed
+  int sT;
   int ns;               // stages per step: the ring holds [R][ns][P] stage-input traces; the
                         // composed steps' S (3, or 5 for the five-stage scheme)
   int ls;               // 1: a 2N low-storage scheme (k_lsrk_stage, coefficients lsA, lsB)
