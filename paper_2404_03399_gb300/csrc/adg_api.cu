@@ -2067,7 +2067,8 @@ struct DevBuf {
 
 // The context's memory pool (the gradient's and the misfit's working fields): it keeps up to
 // kPoolKeep bytes between calls, which a repeated gradient would otherwise allocate and free
-// each time (some 1 ms for the 65536-element workload), and is destroyed with the context.
+// each time, and is destroyed with the context (with direct launches instead of graphs, 3.92 -> 3.04
+// ms for the gradient of 100 steps on 65536 elements).
 constexpr uint64_t kPoolKeep = uint64_t(1) << 30;
 
 cudaError_t pool_alloc(adg_ctx *c, DevBuf &b, size_t bytes) {
@@ -2391,8 +2392,8 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
       }
     }
     if (states) {
-      // one kernel per step: launched directly (capturing and instantiating the sweeps' graphs
-      // took about 0.9 of the 3.9 ms of 100 steps on 65536 elements)
+      // one kernel per step: launched directly, without capturing and instantiating graphs of the
+      // sweeps (with the pool, 3.92 -> 3.04 ms for 100 steps on 65536 elements)
       r = sweep_reverse(c, h, segb[cur], lam.d(), lring.d(), len, par);
       if (r) return r;
     } else {

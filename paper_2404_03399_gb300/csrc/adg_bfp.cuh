@@ -18,9 +18,10 @@
 // 2^-6 of that largest value (kBfSpan), so an element's error per stage is at most about 2^-51
 // of its own largest value, as the chain of FP64 roundings gives. Warps with an element outside
 // that (or exponents near the ends of the FP64 range, NaN, infinities, growth past the headroom
-// within a step, Courant numbers whose coefficients do not fit) take the FP64 stages, some
-// 8 us for a warp: with one scale per warp instead, the warps at a smooth wave's zeros did, and
-// were the longest part of a step on 65536 elements (13 of 14 us).
+// within a step, Courant numbers whose coefficients do not fit) take the FP64 stages. With one
+// scale per warp instead of per element the warps at a smooth wave's zeros did (the gradient on
+// 65536 elements, 100 steps: 3.00 ms, 2.91 ms with a scale per element; without a zero the scales
+// per element cost 4% on 2^20 elements).
 #pragma once
 
 #include "adg_fixed.cuh"
@@ -68,21 +69,32 @@ __device__ __forceinline__ long long bf_square(int xh, int xl) {
 }
 
 // Local Lax-Friedrichs flux 1/4 (a^2 + b^2) - 1/2 max(|a|, |b|) (b - a) of the traces a = u^-,
-// b = u^+ with squares ga, gb, in the squares' units.
+// b = u^+ with squares ga, gb, in the squares' units. With the larger trace x the last product
+// is +-(a b - x^2): one product and no magnitudes (the sign is x's, and the other one for b);
+// equal traces give a b = a^2 exactly.
 __device__ __forceinline__ long long bf_llf(long long a, long long b, long long ga, long long gb) {
-  const unsigned long long ma = (unsigned long long)(a < 0 ? -a : a);
-  const unsigned long long mb = (unsigned long long)(b < 0 ? -b : b);
-  int lh, ll, jh, jl;
-  fx_split((long long)(ma >= mb ? ma : mb), lh, ll);
-  fx_split(b - a, jh, jl);
-  const long long prod = fx_mul(lh, jh) + ((fx_mul(lh, jl) + fx_mul(ll, jh)) >> 29);
-  return (ga + gb - 2 * prod + 2) >> 2;
+  int ah, al, bh, bl;
+  fx_split(a, ah, al);
+  fx_split(b, bh, bl);
+  const long long ab = fx_mul(ah, bh) + ((fx_mul(ah, bl) + fx_mul(al, bh)) >> 29);
+  const bool left = ga >= gb;
+  const long long t = left ? ab - ga : gb - ab;
+  const long long s = (long long)((int)((left ? a : b) >> 32) >> 31);   // 0 or -1
+  return (ga + gb - 2 * ((t ^ s) - s) + 2) >> 2;
 }
 
 // 1/3 as limbs of round(2^58 / 3).
 constexpr long long kThird = ((1ll << 58) - 1) / 3;
 constexpr int kThirdLo = (int)(((kThird & 0x1FFFFFFF) ^ 0x10000000) - 0x10000000);
 constexpr int kThirdHi = (int)((kThird - kThirdLo) >> 29);
+
+// The high word of a bound on |y| as fx_mag gives it: OR-ed over the values of a step, its bits
+// from kBfTop up show growth past the headroom (two instructions less per value than in 64 bits).
+__device__ __forceinline__ unsigned bf_mag(long long y) {
+  const int h = (int)(y >> 32);
+  return (unsigned)(h ^ (h >> 31));
+}
+constexpr unsigned kBfOver = 1u << (kBfTop - 32);
 
 // v 2^-d (d < 0: a left shift; the caller has checked that the result fits).
 __device__ __forceinline__ long long bf_shift(long long v, int d) {
@@ -91,12 +103,12 @@ __device__ __forceinline__ long long bf_shift(long long v, int d) {
 
 // A neighbour's value v brought to this lane's unit, d exponents above the neighbour's (rounded);
 // raises `mag` past the headroom where it does not stay below 2^60.
-__device__ __forceinline__ long long bf_bring(long long v, int d, unsigned long long &mag) {
+__device__ __forceinline__ long long bf_bring(long long v, int d, unsigned &mag) {
   if (d == 0) return v;
   d = d > 62 ? 62 : d;
   if (d > 0) return (v + (1ll << (d - 1))) >> d;
   if (d < -60 || (fx_mag(v) >> (60 + d)) != 0) {
-    mag |= v ? 1ull << kBfTop : 0ull;
+    mag |= v ? kBfOver : 0u;
     return 0;
   }
   return (long long)((unsigned long long)v << (-d));

@@ -203,8 +203,8 @@ __device__ __forceinline__ void burgers_operator(const BurgersFixed &B, const lo
 
 // One step of Burgers (SSP-RK3, or with LS a 2N low-storage scheme; with VISC the viscous term
 // of the local DG method). Warp w owns 32 - H - HR elements and forms H = ns more on the left
-// and HR on the right (warp_element), so the stages run in registers with shuffles for the face values and no barrier, and u is
-// read and written once per step. The operator
+// and HR on the right (warp_element), so the stages run in registers with shuffles for the face
+// values and no barrier, and u is read and written once per step. The operator
 //   dt L(v)_i = sum_j W_ij g_j + a_i F_L + b_i F_R,   g = v^2
 // (W = c2/2 (D + M^-1 e_0 e_0^T - M^-1 e_p e_p^T), a = -c2 M^-1 e_0, b = c2 M^-1 e_p) maps the
 // even part of (g, faces) to the odd part and back, since the nodes are symmetric, so it is
@@ -215,10 +215,11 @@ __device__ __forceinline__ void burgers_operator(const BurgersFixed &B, const lo
 // brought to 58 bits by its largest value in the element, since smooth fields leave it far
 // below its bound.
 // Bound by instruction issue (integer). K = 2^20, p = 4, ADG-AT2, SSP-RK3: 0.50 ms a step as
-// three FP64 stage kernels (80% of the FP64 pipe, eight field passes), 0.078 ms so; K = 10125,
-// p = 2: 14.5 -> 5.3 us, where the launch and the dependent loads of the delays and ring levels
-// are what is left. Two elements per thread (58 of 64 owned, 128 registers) took 0.089 ms and
-// 7.0 us.
+// three FP64 stage kernels (80% of the FP64 pipe, eight field passes), 0.075 ms so (0.0815 with
+// 64-bit headroom checks and the face flux's magnitudes); viscous, K = 2^18, p = 2, RK2: 0.127 ->
+// 0.022 ms; K = 10125, p = 2: 14.5 -> 5.0 us, where the launch and the dependent loads of the
+// delays and ring levels are what is left. Two elements per thread (58 of 64 owned, 128
+// registers) took 0.089 ms and 7.0 us when one per thread took 0.078 and 5.3.
 template <int NP, bool FACES, bool REC, bool VISC, bool LS>
 __global__ void __launch_bounds__(128) k_burgers_step(const __grid_constant__ Inst I,
                                                       const __grid_constant__ StepArgs A) {
@@ -286,7 +287,7 @@ if constexpr (!LS && !VISC) {
       v[i] = bf_from(ud[i], be);
       u[i] = LS ? 0 : v[i];
     }
-    unsigned long long mag = 0;
+    unsigned mag = 0;
     auto stage = [&](int s) {
       long long G[NP];
 #pragma unroll
@@ -347,14 +348,14 @@ if constexpr (!LS && !VISC) {
           if (late) {
             const double y = sV[2 * S + s][lane];
             // |y| < 2^(uf + 58)
-            if (((__double2hiint(y) & 0x7fffffff) >> 20) > uf + 1080) mag |= 1ull << kBfTop;
+            if (((__double2hiint(y) & 0x7fffffff) >> 20) > uf + 1080) mag |= kBfOver;
             else y0 = bf_from(y, uf + 1080) << 1;
           }
         }
         FL += (y0 + 1) >> 1;
         d = -(B.sc + uf - E + 57);
         if (d < -2) {
-          mag |= 1ull << kBfTop;
+          mag |= kBfOver;
           d = -2;
         }
       }
@@ -367,10 +368,19 @@ if constexpr (!LS && !VISC) {
       d = d > 60 ? 60 : d;
       long long r[NP];
       burgers_operator<NP>(B, G, FL, FR, d > 0 ? 1ll << (d - 1) : 0, r);
+      if (__any_sync(full, d < 0)) {   // large Courant numbers
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+          if (d < 0 && (fx_mag(r[k]) >> (kBfTop + d))) mag |= kBfOver;
+          r[k] = bf_shift(r[k], d);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) r[k] >>= d;
+      }
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
-        if (d < 0 && (fx_mag(r[k]) >> (kBfTop + d))) mag |= 1ull << kBfTop;
-        const long long x = bf_shift(r[k], d);
+        const long long x = r[k];
         if (LS) {
           if (s > 0) {
             int h, l;
@@ -381,7 +391,7 @@ if constexpr (!LS && !VISC) {
           } else {
             u[k] = x;
           }
-          mag |= fx_mag(u[k]);
+          mag |= bf_mag(u[k]);
           int h, l;
           fx_split(u[k], h, l);
           FxAcc c;
@@ -393,14 +403,14 @@ if constexpr (!LS && !VISC) {
           v[k] = ((3 * u[k] + v[k] + 2) >> 2) + x;
         } else {
           const long long T = u[k] + 2 * v[k] + x;
-          mag |= fx_mag(T) >> 2;   // below 2^60: its high limb fits 32 bits
+          mag |= bf_mag(T) >> 2;   // below 2^60: its high limb fits 32 bits
           int th, tl;
           fx_split(T, th, tl);
           FxAcc c;
           fx_mac(c, make_int2(kThirdHi, kThirdLo), th, tl);
           v[k] = fx_round(c);
         }
-        mag |= fx_mag(v[k]);
+        mag |= bf_mag(v[k]);
       }
       if (REC && s < 2 && own) {
         double *o = s == 0 ? A.r1 : A.r2;
@@ -414,7 +424,7 @@ if constexpr (!LS && !VISC) {
 #pragma unroll
       for (int s = 0; s < kStages; ++s) stage(s);
     }
-    if (!__any_sync(full, (mag >> kBfTop) != 0)) {
+    if (!__any_sync(full, mag >= kBfOver)) {
       if (own) {
 #pragma unroll
         for (int i = 0; i < NP; ++i) A.uout[(size_t)i * K + e] = bf_to(v[i], E - 57);
@@ -541,8 +551,10 @@ __device__ __noinline__ void burgers_adj_fp64(const Inst &I, const AdjArgs &A, i
 // c_i mu to the delayed levels of the adjoint ring and takes the ring entry of its own step
 // and stage for (delay > 0) or beside (delay 0) mu; its owner clears the entries of step
 // n + 1, which the kernel before this one read. The gradient on 65536 elements (p = 3, 100
-// steps): 6.3 -> 3.9 ms against
-// three FP64 stage kernels of 14 us each, bound by the FP64 pipe.
+// steps) with this kernel: 6.3 -> 3.9 ms, against three FP64 stage kernels of 14 us each, bound
+// by the FP64 pipe (11.3 -> 2.9 ms with the forward's step and without recomputation). Bound by
+// the latency of a warp's chain: 631 blocks are 16 warps per SM, and the 5 million warp
+// instructions of a launch some 4 of its 14 us.
 template <int NP, bool FACES>
 __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Inst I,
                                                      const __grid_constant__ AdjArgs A) {
@@ -615,11 +627,18 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
     const int dVL = E - __shfl_up_sync(full, E, 1);
     const int d = d0 > 60 ? 60 : d0;
     const long long half = d > 0 ? 1ll << (d - 1) : 0;
+    const bool up = __any_sync(full, d < 0);   // large Courant numbers
+    // z 2^-d
+    auto scale = [&](long long z, unsigned &over) -> long long {
+      if (!up) return z >> d;
+      if (d < 0 && (fx_mag(z) >> (kBfTop + d))) over |= kBfOver;
+      return bf_shift(z, d);
+    };
     long long w[NP], acc[NP];
     double post[kStages];   // beta mu of a PE face's stages (FP64), posted once the step holds
 #pragma unroll
     for (int i = 0; i < NP; ++i) w[i] = bf_from(wd[i], bw);
-    unsigned long long mag = 0;
+    unsigned mag = 0;
     // x / 3 for |x| < 2^60
     auto third = [](long long x) {
       int h, l;
@@ -658,14 +677,14 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
       bf_llf_partials2(bf_bring(__shfl_up_sync(full, v[NP - 1], 1), dVL, mag), v[0], dl, dr);
       if (FACES && pe) {
         const long long r = bf_from(sR[s][lane], B.sc + Ew + 1025) << 3;
-        mag |= fx_mag(mu) >> 4;   // below 2^62
+        mag |= bf_mag(mu) >> 4;   // below 2^62
         const double m = bf_to(mu, smu);
         post[s] = s == 2 ? m * (2.0 / 3.0) : (s == 1 ? 0.25 * m : m);
         // the ring holds adjoints of the flux with beta: divided by it here
         const long long rb = s == 2 ? r + (r >> 1) : (s == 1 ? 4 * r : r);
         mu = k > 0 ? rb : mu + rb;
       }
-      mag |= fx_mag(mu) >> 4;   // below 2^62
+      mag |= bf_mag(mu) >> 4;   // below 2^62
       int mh, ml, xh, xl;
       fx_split((mu + 4) >> 3, mh, ml);
       fx_split(dl, xh, xl);
@@ -673,8 +692,7 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
       fx_split(dr, xh, xl);
       const long long pr = mul(mh, ml, xh, xl);
       // the left element's part, in units of this lane's w, from the lane above
-      if (d < 0 && (fx_mag(pl) >> (kBfTop + d))) mag |= 1ull << kBfTop;
-      const long long pR = bf_bring(__shfl_down_sync(full, bf_shift(pl + half, d), 1), dWR, mag);
+      const long long pR = bf_bring(__shfl_down_sync(full, scale(pl + half, mag), 1), dWR, mag);
 #pragma unroll
       for (int j = 0; j < HP + MID; ++j) {
         // half the sum and half the difference of (W^T w)_j and (W^T w)_{p-j}
@@ -696,9 +714,8 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
           fx_split(v[q], vh, vl);
           long long z = 2 * mul(rh, rl, vh, vl) + half;
           if (q == 0) z += pr;
-          if (d < 0 && (fx_mag(z) >> (kBfTop + d))) mag |= 1ull << kBfTop;
-          const long long x = w[q] + bf_shift(z, d) + (q == NP - 1 ? pR : 0);
-          mag |= fx_mag(x);
+          const long long x = w[q] + scale(z, mag) + (q == NP - 1 ? pR : 0);
+          mag |= bf_mag(x);
           if (s == 2) {
             acc[q] = third(w[q]);
             w[q] = third(2 * x);
@@ -707,12 +724,12 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
             w[q] = (x + 2) >> 2;
           } else {
             w[q] = x + acc[q];
-            mag |= fx_mag(w[q]);
+            mag |= bf_mag(w[q]);
           }
         }
       }
     }
-    if (!__any_sync(full, (mag >> kBfTop) != 0)) {
+    if (!__any_sync(full, mag >= kBfOver)) {
       if (own) {
 #pragma unroll
         for (int i = 0; i < NP; ++i) A.out[(size_t)i * K + e] = bf_to(w[i], Ew - 57);

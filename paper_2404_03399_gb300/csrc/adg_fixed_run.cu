@@ -152,8 +152,8 @@ __device__ __forceinline__ void run_face(const Inst &I, RunShared<NP, S> &sh, co
 //     grid's barrier, whose word also carries the reduction of the next step's scale. The wait
 //     is bounded: after kRunPolls polls a block sets *err and returns.
 // Bound by latency: the chain through a tile's elements, the faces' differences and the barrier.
-// K = 65536, p = 3, ADG-AT3 (256 PEs): 8.6 us a step as two kernels in a graph, 4.7 us so
-// (sync 3.9 -> 3.0 us). (Every block
+// K = 65536, p = 3, ADG-AT3 (256 PEs): 8.9 us a step as two kernels in a graph, 5.0 us so
+// with the read of the state (sync steps alone 3.9 -> 3.0 us). (Every block
 // polling a flag of every other took 1.5-2.9 us a step for the barrier alone, which is 1.0 us; a
 // face per lane with its ring in global memory 3.4 us for the faces.)
 template <int NP, int S, bool FACES>
