@@ -4,7 +4,8 @@
  * The library advances 1D nodal DG discretisations of u_t + f(u)_x = 0 on a periodic
  * interval with the fully discrete strong-stability-preserving RK3 step (or the paper's
  * low-storage schemes), on one GPU, in FP64 (the composed step of upwind advection in 58-bit
- * block fixed point: adg_config.variant). Elements are split into P contiguous "processing elements" (PEs); at PE faces the
+ * block fixed point: adg_config.variant; the Burgers steps with FP64 fields and 57-bit local
+ * block fixed point inside a step, see pde). Elements are split into P contiguous "processing elements" (PEs); at PE faces the
  * numerical flux uses data of a delayed time level taken from a seeded delay table and a
  * device ring buffer, combined by the standard flux or the asynchrony-tolerant (AT) flux.
  *
@@ -45,7 +46,8 @@ typedef enum {
   ADG_ENOMEM = -2,     /* device or host allocation failed */
   ADG_ECUDA = -3,      /* CUDA runtime error (or no device) */
   ADG_ENONFINITE = -4, /* a NaN or Inf was found in the state */
-  ADG_ETIMEOUT = -5,   /* a bounded device wait ran out */
+  ADG_ETIMEOUT = -5,   /* a bounded device wait ran out (reported by the next call that waits
+                          for the stream; the state is lost) */
   ADG_ESTATE = -6      /* call not valid in the context's current state */
 } adg_status;
 
@@ -74,6 +76,11 @@ enum {
  * Run configuration (Section 2: mesh, degree, flux, RK; Section 3: P and L; Section 5:
  * AT order; Section 6.1: probability set and seeded draws).
  *   pde, flux : ADG_ADVECTION with ADG_UPWIND, or ADG_BURGERS with ADG_LLF.
+ *               A Burgers step reads and writes FP64; inside it an element's values are integers
+ *               at the scale of the largest value of the element and those that reach it within
+ *               the step, each rounding below 2^-56 of that value, and only where the element
+ *               itself reaches 2^-6 of it (elsewhere, and for NaN, infinities, exponents near
+ *               FP64's ends and growth past the headroom, FP64 arithmetic).
  *   rk        : ADG_SSPRK3 (default; every variant, adg_grad and batches), or one of the
  *               low-storage schemes of the kind Section 6 integrates with, run in Williamson's
  *               2N form (dU_s = A_s dU_{s-1} + dt L(U_{s-1}), U_s = U_{s-1} + B_s dU_s) by the
@@ -250,8 +257,11 @@ int adg_get_fixed_basis(adg_ctx *c, int32_t index, int32_t *basis_out);
  * with respect to the initial nodal field, for a single-instance context, over nsteps
  * steps starting from the current state (the state itself is left unchanged). The adjoint
  * is hand-written: transposed stage operators, flux partial derivatives, and a reverse
- * ring buffer over the delay table. Checkpoints every ckpt_every steps, recomputation in
- * between. target_dev and grad_u0_dev are device (K, p+1) row-major FP64; J_out is host.
+ * ring buffer over the delay table. Checkpoints every ckpt_every steps (at most the 512 steps
+ * of the delay table's window when delays are in use), recomputation in between; a run whose
+ * recorded states fit in 1 GiB is recorded whole instead (the result does not depend on it).
+ * The working memory comes from a pool of the context, which keeps up to 1 GiB of it until
+ * adg_destroy. target_dev and grad_u0_dev are device (K, p+1) row-major FP64; J_out is host.
  * The paper has no adjoint; this follows the discrete forward scheme exactly.
  */
 int adg_grad(adg_ctx *c, const double *target_dev, int64_t nsteps, int32_t ckpt_every,
