@@ -102,12 +102,13 @@ __device__ __forceinline__ long long bf_shift(long long v, int d) {
 }
 
 // A neighbour's value v brought to this lane's unit, d exponents above the neighbour's (rounded);
-// raises `mag` past the headroom where it does not stay below 2^60.
+// raises `mag` past the headroom where it does not stay below 2^Top.
+template <int Top = kBfTop>
 __device__ __forceinline__ long long bf_bring(long long v, int d, unsigned &mag) {
   if (d == 0) return v;
   d = d > 62 ? 62 : d;
   if (d > 0) return (v + (1ll << (d - 1))) >> d;
-  if (d < -60 || (fx_mag(v) >> (60 + d)) != 0) {
+  if (d < -Top || (fx_mag(v) >> (Top + d)) != 0) {
     mag |= v ? kBfOver : 0u;
     return 0;
   }

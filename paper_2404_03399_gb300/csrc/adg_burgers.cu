@@ -361,7 +361,7 @@ if constexpr (!LS && !VISC) {
       }
       const int dF = VISC ? uf - __shfl_down_sync(full, uf, 1) : 2 * dER;
       long long FR = __shfl_down_sync(full, FL, 1);
-      if (dF != 0) FR = bf_bring(FR, dF, mag);
+      if (dF != 0) FR = bf_bring<kBfTop + 1>(FR, dF, mag);   // faces below 2^59 (burgers_operator)
       // shift of the operator's sums: in SSP-RK3 stage 1 takes a quarter of them, stage 2
       // (inside the sum divided by 3) twice
       if (!LS) d = s == 0 ? d : (s == 1 ? d + 2 : d - 1);
@@ -671,7 +671,7 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
       for (int i = 0; i < HP; ++i) fx_mac(ao, B.D[i][HP + MID], th[i], tl[i]);
       const long long ev = fx_round(ae), od = fx_round(ao);
       // (|od - ev| < 2^62: brought with two bits less)
-      const long long bl = bf_bring(__shfl_up_sync(full, (od - ev + 2) >> 2, 1), dWL, mag);
+      const long long bl = bf_bring<kBfTop + 2>(__shfl_up_sync(full, (od - ev + 2) >> 2, 1), dWL, mag);
       long long mu = ev + od + 4 * bl;
       long long dl, dr;
       bf_llf_partials2(bf_bring(__shfl_up_sync(full, v[NP - 1], 1), dVL, mag), v[0], dl, dr);
@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
       fx_split(dr, xh, xl);
       const long long pr = mul(mh, ml, xh, xl);
       // the left element's part, in units of this lane's w, from the lane above
-      const long long pR = bf_bring(__shfl_down_sync(full, scale(pl + half, mag), 1), dWR, mag);
+      const long long pR = bf_bring<kBfTop + 2>(__shfl_down_sync(full, scale(pl + half, mag), 1), dWR, mag);
 #pragma unroll
       for (int j = 0; j < HP + MID; ++j) {
         // half the sum and half the difference of (W^T w)_j and (W^T w)_{p-j}
