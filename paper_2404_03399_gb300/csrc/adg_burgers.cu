@@ -553,10 +553,11 @@ __device__ __noinline__ void burgers_adj_fp64(const Inst &I, const AdjArgs &A, i
 // n + 1, which the kernel before this one read. The gradient on 65536 elements (p = 3, 100
 // steps) with this kernel: 6.3 -> 3.9 ms, against three FP64 stage kernels of 14 us each, bound
 // by the FP64 pipe (11.3 -> 2.9 ms with the forward's step and without recomputation). Bound by
-// the latency of a warp's chain: 631 blocks are 16 warps per SM, and the 5 million warp
-// instructions of a launch some 4 of its 14 us.
+// the latency of a warp's chain: 65536 elements are 17 warps per SM, and the 5 million warp
+// instructions of a launch some 4 of its 12 us. At p = 3 the compiler's own choice was 80
+// registers with spills (2.92 against 2.75 ms at the 96 of five blocks).
 template <int NP, bool FACES>
-__global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Inst I,
+__global__ void __launch_bounds__(128, NP == 4 ? 5 : 0) k_burgers_adj(const __grid_constant__ Inst I,
                                                      const __grid_constant__ AdjArgs A) {
   constexpr int HP = NP / 2, MID = NP % 2;
   __shared__ double sR_[FACES ? 4 * kStages : 1][32];
@@ -745,16 +746,40 @@ __global__ void __launch_bounds__(128) k_burgers_adj(const __grid_constant__ Ins
   burgers_adj_fp64<NP, FACES>(I, A, warp, nm, sR, pe, k, qe, c);
 }
 
-// One-warp blocks while the mesh gives fewer than 16 warps per SM (they spread evenly).
-int burgers_block(int64_t warps) { return warps < 16 * sm_count() ? 32 : 128; }
+// One-warp blocks while the mesh gives fewer than 32 warps per SM: they spread evenly, and all
+// are resident at once. Larger meshes run several waves of four-warp blocks; so do viscous ones
+// from 16 warps per SM, whose blocks' shared memory (fixed, four warps' worth) leaves no room for
+// 32 on an SM.
+constexpr size_t kSmemSM = 228 * 1024;   // of an SM; a block takes 1 KB besides its own
+int burgers_block(int64_t warps, size_t fixed) {
+  const int per = fixed + 1024 <= kSmemSM / 32 ? 32 : 16;
+  return warps < per * sm_count() ? 32 : 128;
+}
+
+// Dynamic shared memory (never read) that lets an SM hold only its even share of the blocks, for
+// grids of 16 to 32 one-warp blocks per SM. A step's blocks become resident while the step before
+// still runs, so without it the SMs that drain first take too many of them and the others too
+// few: 50 steps on 65536 elements, p = 3: 591 us in four-warp blocks, 512 with those held to
+// their share, 490 in one-warp blocks so; p = 1: 515 -> 413; the gradient of 50 steps 1.50 ->
+// 1.30 ms. Below 16 warps per SM the next step's blocks all wait beside the present ones and
+// hide their launch (16384 elements: 299 us, 302 with their share only).
+size_t burgers_smem(int64_t grid, int bs, size_t fixed) {
+  const int64_t per = (grid + sm_count() - 1) / sm_count();
+  if (bs != 32 || per < 16) return 0;
+  const size_t block = kSmemSM / (per + 1) + 128;
+  return block > fixed + 1024 ? block - fixed - 1024 : 0;
+}
 
 template <int NP, bool FACES>
 cudaError_t burgers_np(const Inst &I, const StepArgs &A, cudaStream_t s, bool pdl) {
   const int own = 32 - A.H - A.HR;
   const int64_t warps = ((int64_t)I.K + own - 1) / own;
-  const int bs = burgers_block(warps);
+  const size_t fixed = FACES ? sizeof(double) * 32 * 4 * (I.visc ? kFaceVals<true> : kFaceVals<false>) *
+                                   (I.ls ? kMaxStages : kStages) : 0;   // sV_
+  const int bs = burgers_block(warps, fixed);
   const dim3 g((unsigned)((warps * 32 + bs - 1) / bs)), b(bs);
-  auto go = [&](auto kernel) { return launch_maybe_pdl(kernel, g, b, s, pdl, I, A); };
+  const size_t smem = burgers_smem(g.x, bs, fixed);
+  auto go = [&](auto kernel) { return launch_smem_pdl(kernel, g, b, smem, s, pdl, I, A); };
   if (A.r1) return go(k_burgers_step<NP, FACES, true, false, false>);
   if (I.ls)
     return I.visc ? go(k_burgers_step<NP, FACES, false, true, true>)
@@ -766,10 +791,12 @@ cudaError_t burgers_np(const Inst &I, const StepArgs &A, cudaStream_t s, bool pd
 template <int NP>
 cudaError_t burgers_adj_np(const Inst &I, const AdjArgs &A, cudaStream_t s, bool pdl) {
   const int64_t warps = ((int64_t)I.K + kOwn - 1) / kOwn;
-  const int bs = burgers_block(warps);
+  const size_t fixed = I.async ? sizeof(double) * 32 * 4 * kStages : 0;   // sR_
+  const int bs = burgers_block(warps, fixed);
   const dim3 g((unsigned)((warps * 32 + bs - 1) / bs)), b(bs);
-  return I.async ? launch_maybe_pdl(k_burgers_adj<NP, true>, g, b, s, pdl, I, A)
-                 : launch_maybe_pdl(k_burgers_adj<NP, false>, g, b, s, pdl, I, A);
+  const size_t smem = burgers_smem(g.x, bs, fixed);
+  return I.async ? launch_smem_pdl(k_burgers_adj<NP, true>, g, b, smem, s, pdl, I, A)
+                 : launch_smem_pdl(k_burgers_adj<NP, false>, g, b, smem, s, pdl, I, A);
 }
 
 }  // namespace

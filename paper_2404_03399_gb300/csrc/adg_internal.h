@@ -305,14 +305,15 @@ size_t fixed_run_bytes(const Inst &I);
 FixedRun fixed_run(void *buf, int *err);
 cudaError_t launch_fixed_run(const Inst &I, const FixedRun &R, const void *in, void *out, int rel,
                              int nsteps, cudaStream_t s);
-// A launch with the programmatic-stream-serialization attribute when pdl is set.
+// A launch with the programmatic-stream-serialization attribute when pdl is set, with smem bytes
+// of dynamic shared memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_maybe_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
-                             bool pdl, Args &&...args) {
+cudaError_t launch_smem_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t s, bool pdl, Args &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -320,6 +321,11 @@ cudaError_t launch_maybe_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cu
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_maybe_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
+                             bool pdl, Args &&...args) {
+  return launch_smem_pdl(kernel, grid, block, 0, s, pdl, std::forward<Args>(args)...);
 }
 // The same with a scheduling priority for the launch's blocks (lower numbers first, within
 // cudaDeviceGetStreamPriorityRange): blocks of a short kernel on the critical path get SM
