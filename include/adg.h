@@ -77,10 +77,11 @@ enum {
  * AT order; Section 6.1: probability set and seeded draws).
  *   pde, flux : ADG_ADVECTION with ADG_UPWIND, or ADG_BURGERS with ADG_LLF.
  *               A Burgers step reads and writes FP64; inside it an element's values are integers
- *               at the scale of the largest value of the element and those that reach it within
- *               the step, each rounding below 2^-56 of that value, and only where the element
- *               itself reaches 2^-6 of it (elsewhere, and for NaN, infinities, exponents near
- *               FP64's ends and growth past the headroom, FP64 arithmetic).
+ *               at the scale of the largest value of the element and the two beside it (units
+ *               below 2^-55 of that value), where the element itself reaches 2^-4 of it (2^-2
+ *               with a low-storage scheme). Elsewhere, with ADG_RK1, and for NaN, infinities,
+ *               exponents near FP64's ends and growth past the headroom: FP64 arithmetic. The
+ *               error is no larger than that of FP64 stages.
  *   rk        : ADG_SSPRK3 (default; every variant, adg_grad and batches), or one of the
  *               low-storage schemes of the kind Section 6 integrates with, run in Williamson's
  *               2N form (dU_s = A_s dU_{s-1} + dt L(U_{s-1}), U_s = U_{s-1} + B_s dU_s) by the

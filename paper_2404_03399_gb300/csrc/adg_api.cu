@@ -533,7 +533,18 @@ void fold_burgers(InstHost &h) {
     const ld vn = std::frexp(2.0L * (ld)h.I.nu / (ld)h.dt, &B.sn);
     B.vn = limbs58(vn);
   }
-  B.ok = std::abs(B.sc) < 300 && std::abs(B.sn) < 300;   // far from the ends of FP64's range
+  for (int i = 0; i < H + mid; ++i) {
+    long long lo = 0;
+    for (int j = 0; j <= H; ++j) lo += B.S[i][j].y;
+    B.rS[i] = (1ll << 28) + (lo >> 1);
+  }
+  for (int i = 0; i < H; ++i) {
+    long long lo = 0;
+    for (int j = 0; j <= H + mid; ++j) lo += B.D[i][j].y;
+    B.rD[i] = (1ll << 28) + (lo >> 1);
+  }
+  // far from the ends of FP64's range; forward Euler's FP64 stage is one rounding (adg_bfp.cuh)
+  B.ok = std::abs(B.sc) < 300 && std::abs(B.sn) < 300 && h.I.ns > 1;
 }
 
 // Composed step constants (StepConsts in adg_internal.h), built in long double from the

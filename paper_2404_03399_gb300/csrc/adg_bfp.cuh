@@ -8,20 +8,32 @@
 // values, bring each element to a scale of its neighbourhood, work in integers, and round once
 // to FP64 when the step is done.
 //
-// An element's values are X = x 2^(57 - E), |x| < 2^E over the element and those that reach it
-// within the step (one on either side per stage), so |X| < 2^57 at the start of the step;
-// every intermediate value is checked to stay below 2^58, and what comes from a neighbour is
-// shifted from its scale. Squares and face fluxes are held in units of 2^(2E - 56): G = X^2
-// 2^-58. An operator coefficient c is C = round(c 2^(58 - sc)), |C| <= 2^58, split as in
-// adg_fixed.cuh, and sums of products are rounded once. Against FP64: a value is exact to 2^-57
-// of the largest one near it; the integer path is taken only if every non-zero element reaches
-// 2^-6 of that largest value (kBfSpan), so an element's error per stage is at most about 2^-51
-// of its own largest value, as the chain of FP64 roundings gives. Warps with an element outside
-// that (or exponents near the ends of the FP64 range, NaN, infinities, growth past the headroom
-// within a step, Courant numbers whose coefficients do not fit) take the FP64 stages. With one
-// scale per warp instead of per element the warps at a smooth wave's zeros did (the gradient on
-// 65536 elements, 100 steps: 3.00 ms, 2.91 ms with a scale per element; without a zero the scales
-// per element cost 4% on 2^20 elements).
+// An element's values are X = x 2^(57 - E), |x| < 2^E over the element and the two beside it, so
+// |X| < 2^57 at the start of the step; every intermediate value is checked to stay below 2^58,
+// and what comes from a neighbour is shifted from its scale. Squares and face fluxes are held in
+// units of 2^(2E - 56): G = X^2 2^-58. An operator coefficient c is C = round(c 2^(58 - sc)),
+// |C| <= 2^58, split as in adg_fixed.cuh, and sums of products are rounded once.
+//
+// Against FP64: a value's unit is 2^-56 of the largest one beside it, FP64's roundings are
+// 2^-53 of a value each, and the integer path is taken only where every non-zero element reaches
+// 2^-kBfSpan of that largest value. The span is where the error of an element, over its own
+// largest value, stays below that of the FP64 stages: emulated in integers and compared with
+// 113-bit arithmetic over p = 1..4, Courant numbers 0.002 to 0.05 and 20 steps, on smooth fields
+// and on rough ones whose patches of four elements differ by up to 50 (rms over the elements,
+// integer over FP64): SSP-RK3 0.17 at equal patches, 0.18 to 0.24 at a ratio of 8 and at most
+// 1.00 beyond with a span of 4; the 2N schemes, whose FP64 stages round once or twice, 0.46 (five
+// stages) to 0.78 (RK2) at equal patches and at most 1.05 beyond with a span of 2. (A span
+// of 6, the scale of the elements up to a stage count away, and sums without the means of what
+// they leave out gave up to 2.1 at a ratio of 50 with SSP-RK3 and 8.8 with RK2.)
+// A simple zero of a smooth field leaves its element within a third of its neighbours, inside
+// both spans. Forward Euler takes FP64: its stage is one rounding, which the integer path also
+// ends with. Warps with an element outside the span (or exponents near the ends of the FP64
+// range, NaN, infinities, growth past the headroom within a step, Courant numbers whose
+// coefficients do not fit) take the FP64 stages.
+//
+// With one scale per warp instead of per element the warps at a smooth wave's zeros did (the
+// gradient on 65536 elements, 100 steps: 3.00 ms, 2.91 ms with a scale per element; without a
+// zero the scales per element cost 4% on 2^20 elements).
 #pragma once
 
 #include "adg_fixed.cuh"
@@ -29,7 +41,9 @@
 namespace adg {
 namespace {
 
-constexpr int kBfSpan = 6;      // exponent of an element below its scale on the integer path
+// exponent of an element below its scale on the integer path, by the scheme (2N or SSP-RK3)
+template <bool LS>
+constexpr int kBfSpan = LS ? 2 : 4;
 constexpr int kBfMinE = 600;    // biased exponents of the scales
 constexpr int kBfMaxE = 1400;
 constexpr int kBfTop = 58;      // every intermediate value below 2^kBfTop
@@ -63,9 +77,11 @@ __device__ __forceinline__ double bf_to(long long y, int sigma) {
   return a == 0 ? 0.0 : __longlong_as_double((long long)(r | ((unsigned long long)s << 63)));
 }
 
-// X^2 2^-58 (|X| < 2^58; below 2 units of error).
+// X^2 2^-58 (|X| < 2^58), rounded, with the mean (a third of a unit) of the xl^2 2^-58 left out:
+// below 7/6 units of error.
+constexpr long long kSquareRound = (1ll << 27) + (1ll << 28) / 3;
 __device__ __forceinline__ long long bf_square(int xh, int xl) {
-  return fx_mul(xh, xh) + (fx_mul(xh, xl) >> 28);
+  return fx_mul(xh, xh) + ((fx_mul(xh, xl) + kSquareRound) >> 28);
 }
 
 // Local Lax-Friedrichs flux 1/4 (a^2 + b^2) - 1/2 max(|a|, |b|) (b - a) of the traces a = u^-,
@@ -76,7 +92,8 @@ __device__ __forceinline__ long long bf_llf(long long a, long long b, long long 
   int ah, al, bh, bl;
   fx_split(a, ah, al);
   fx_split(b, bh, bl);
-  const long long ab = fx_mul(ah, bh) + ((fx_mul(ah, bl) + fx_mul(al, bh)) >> 29);
+  const long long ab =
+      fx_mul(ah, bh) + ((fx_mul(ah, bl) + fx_mul(al, bh) + 2 * kSquareRound) >> 29);
   const bool left = ga >= gb;
   const long long t = left ? ab - ga : gb - ab;
   const long long s = (long long)((int)((left ? a : b) >> 32) >> 31);   // 0 or -1

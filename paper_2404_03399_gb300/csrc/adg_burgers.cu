@@ -183,13 +183,12 @@ __device__ __forceinline__ void burgers_operator(const BurgersFixed &B, const lo
   fx_split(FL + FR, sh[HP + MID], sl[HP + MID]);
 #pragma unroll
   for (int i = 0; i < HP + MID; ++i) {
-    FxAcc a;
-    a.a = half;
+    FxAcc a{half, B.rS[i]};
 #pragma unroll
     for (int j = 0; j <= HP; ++j) fx_mac(a, B.S[i][j], dh[j], dl[j]);
     const long long odd = fx_round(a);
     if (i < HP) {
-      FxAcc b;
+      FxAcc b{0, B.rD[i]};
 #pragma unroll
       for (int j = 0; j <= HP + MID; ++j) fx_mac(b, B.D[i][j], sh[j], sl[j]);
       const long long even = fx_round(b);
@@ -267,12 +266,12 @@ if constexpr (!LS && !VISC) {
     hi = max(hi, __double2hiint(ud[i]) & 0x7fffffff);
     lo |= (unsigned)__double2loint(ud[i]);
   }
-  const int be = bf_window_max(hi >> 20, S);
+  const int be = bf_window_max(hi >> 20, 1);
   const int E = be - 1022;              // |u| < 2^E
   const BurgersFixed &B = I.bf;
   const int d0 = -(B.sc + E + 1);       // operator sums -> value units (inviscid)
   bool bad = be < kBfMinE || be > kBfMaxE || d0 < -2 || !B.ok;
-  bad = bad || (hi ? (hi >> 20) < be - kBfSpan : lo != 0);
+  bad = bad || (hi ? (hi >> 20) < be - kBfSpan<LS> : lo != 0);
   // a delayed flux of 2^(2E + 1) or more, a delayed trace of 2^(E + 1) or more
   if (FACES) bad = bad || (fmax >> 20) > 2 * E + 1023;
   if (FACES && VISC) bad = bad || (umax >> 20) > be + 1;
@@ -336,9 +335,7 @@ if constexpr (!LS && !VISC) {
         for (int i = 0; i < NP; ++i) {
           int zh2, zl2;
           fx_split(bf_shift(Z[i], -nz), zh2, zl2);
-          FxAcc c;
-          fx_mac(c, B.vn, zh2, zl2);
-          const long long y = (fx_round(c) + hq) >> sq;
+          const long long y = (fx_scaled(B.vn, zh2, zl2) + hq) >> sq;
           G[i] = ((G[i] + hf) >> sf) + y;
           if (i == 0) y0 = y;
         }
@@ -385,16 +382,17 @@ if constexpr (!LS && !VISC) {
           if (s > 0) {
             int h, l;
             fx_split(u[k], h, l);
-            FxAcc c;
-            fx_mac(c, B.lsA[s], h, l);
-            u[k] = fx_round(c) + x;
+            u[k] = fx_scaled(B.lsA[s], h, l) + x;
           } else {
             u[k] = x;
           }
           mag |= bf_mag(u[k]);
           int h, l;
           fx_split(u[k], h, l);
+          // halves (the two-stage scheme's B = 1/2) up or down by v's last bit: always up, they
+          // moved the field by a quarter unit a step
           FxAcc c;
+          c.b += (B.lsB[s].y >> 1) - (int)(v[k] & 1);
           fx_mac(c, B.lsB[s], h, l);
           v[k] += fx_round(c);
         } else if (s == 0) {
@@ -406,9 +404,7 @@ if constexpr (!LS && !VISC) {
           mag |= bf_mag(T) >> 2;   // below 2^60: its high limb fits 32 bits
           int th, tl;
           fx_split(T, th, tl);
-          FxAcc c;
-          fx_mac(c, make_int2(kThirdHi, kThirdLo), th, tl);
-          v[k] = fx_round(c);
+          v[k] = fx_scaled(make_int2(kThirdHi, kThirdLo), th, tl);
         }
         mag |= bf_mag(v[k]);
       }
@@ -616,7 +612,7 @@ __global__ void __launch_bounds__(128, NP == 4 ? 5 : 0) k_burgers_adj(const __gr
   const int Ew = bw - 1022, E = bv - 1022;
   const int d0 = -(I.bf.sc + E + 1) - 2;   // (2 P + P') -> units of w
   bool bad = bw < kBfMinE || bw > kBfMaxE || bv < kBfMinE || bv > kBfMaxE || d0 < -3 || !I.bf.ok;
-  bad = bad || (hw ? (hw >> 20) < bw - kBfSpan : lo != 0);
+  bad = bad || (hw ? (hw >> 20) < bw - 6 : lo != 0);
   // ring entries below 2^60 in units of mu
   if (FACES) bad = bad || (rmax >> 20) > I.bf.sc + Ew + 1025;
 

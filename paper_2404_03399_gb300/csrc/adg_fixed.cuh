@@ -64,6 +64,14 @@ __device__ __forceinline__ void fx_mac(FxAcc &s, int2 c, int xh, int xl) {
 
 __device__ __forceinline__ long long fx_round(const FxAcc &s) { return s.a + (s.b >> 29); }
 
+// c x rounded, with the mean of the low limb product that fx_mac leaves out.
+__device__ __forceinline__ long long fx_scaled(int2 c, int xh, int xl) {
+  FxAcc s;
+  s.b += c.y >> 1;
+  fx_mac(s, c, xh, xl);
+  return fx_round(s);
+}
+
 // The 64-bit value with 32-bit halves lo, hi.
 __device__ __forceinline__ long long fx_join(unsigned lo, unsigned hi) {
   long long r;
