@@ -78,7 +78,7 @@ enum {
  *   pde, flux : ADG_ADVECTION with ADG_UPWIND, or ADG_BURGERS with ADG_LLF.
  *               A Burgers step reads and writes FP64; inside it an element's values are integers
  *               at the scale of the largest value of the element and the two beside it (units
- *               below 2^-55 of that value), where the element itself reaches 2^-4 of it (2^-2
+ *               below 2^-55 of that value), where the element itself reaches 2^-4 of it (2^-3
  *               with a low-storage scheme). Elsewhere, with ADG_RK1, and for NaN, infinities,
  *               exponents near FP64's ends and growth past the headroom: FP64 arithmetic. The
  *               error is no larger than that of FP64 stages.

@@ -18,13 +18,15 @@
 // 2^-53 of a value each, and the integer path is taken only where every non-zero element reaches
 // 2^-kBfSpan of that largest value. The span is where the error of an element, over its own
 // largest value, stays below that of the FP64 stages: emulated in integers and compared with
-// 113-bit arithmetic over p = 1..4, Courant numbers 0.002 to 0.05 and 20 steps, on smooth fields
-// and on rough ones whose patches of four elements differ by up to 50 (rms over the elements,
-// integer over FP64): SSP-RK3 0.17 at equal patches, 0.18 to 0.24 at a ratio of 8 and at most
-// 1.00 beyond with a span of 4; the 2N schemes, whose FP64 stages round once or twice, 0.46 (five
-// stages) to 0.78 (RK2) at equal patches and at most 1.05 beyond with a span of 2. (A span
-// of 6, the scale of the elements up to a stage count away, and sums without the means of what
-// they leave out gave up to 2.1 at a ratio of 50 with SSP-RK3 and 8.8 with RK2.)
+// 113-bit arithmetic over p = 1..4, Courant numbers 0.002 to 0.05, 20 and 200 steps, on smooth
+// fields and on rough ones whose patches of four elements differ by up to 50 (rms over the
+// elements, integer over FP64): SSP-RK3 0.17 at equal patches, 0.18 to 0.26 at a ratio of 8 and
+// at most 1.00 beyond with a span of 4; the 2N schemes, whose FP64 stages round once or twice,
+// 0.45 (five stages) to 0.72 (RK2) at equal patches, at most 0.89 at 8 and 1.06 beyond with a
+// span of 3. Roundings to the nearest integer that always sent halves up, and the means of the
+// products that sums leave out, would add up step by step (with them, RK2 reached 1.9 after 200
+// steps; with a span of 6 and the scale of the elements up to a stage count away besides, 8.8
+// at a ratio of 50, and SSP-RK3 2.1).
 // A simple zero of a smooth field leaves its element within a third of its neighbours, inside
 // both spans. Forward Euler takes FP64: its stage is one rounding, which the integer path also
 // ends with. Warps with an element outside the span (or exponents near the ends of the FP64
@@ -43,7 +45,7 @@ namespace {
 
 // exponent of an element below its scale on the integer path, by the scheme (2N or SSP-RK3)
 template <bool LS>
-constexpr int kBfSpan = LS ? 2 : 4;
+constexpr int kBfSpan = LS ? 3 : 4;
 constexpr int kBfMinE = 600;    // biased exponents of the scales
 constexpr int kBfMaxE = 1400;
 constexpr int kBfTop = 58;      // every intermediate value below 2^kBfTop
@@ -87,7 +89,7 @@ __device__ __forceinline__ long long bf_square(int xh, int xl) {
 // Local Lax-Friedrichs flux 1/4 (a^2 + b^2) - 1/2 max(|a|, |b|) (b - a) of the traces a = u^-,
 // b = u^+ with squares ga, gb, in the squares' units. With the larger trace x the last product
 // is +-(a b - x^2): one product and no magnitudes (the sign is x's, and the other one for b);
-// equal traces give a b = a^2 exactly.
+// equal traces give a b = a^2 exactly. Halves go up or down by a bit of gb.
 __device__ __forceinline__ long long bf_llf(long long a, long long b, long long ga, long long gb) {
   int ah, al, bh, bl;
   fx_split(a, ah, al);
@@ -97,7 +99,7 @@ __device__ __forceinline__ long long bf_llf(long long a, long long b, long long 
   const bool left = ga >= gb;
   const long long t = left ? ab - ga : gb - ab;
   const long long s = (long long)((int)((left ? a : b) >> 32) >> 31);   // 0 or -1
-  return (ga + gb - 2 * ((t ^ s) - s) + 2) >> 2;
+  return (ga + gb - 2 * ((t ^ s) - s) + 2 - ((gb >> 1) & 1)) >> 2;
 }
 
 // 1/3 as limbs of round(2^58 / 3).

@@ -364,7 +364,8 @@ if constexpr (!LS && !VISC) {
       if (!LS) d = s == 0 ? d : (s == 1 ? d + 2 : d - 1);
       d = d > 60 ? 60 : d;
       long long r[NP];
-      burgers_operator<NP>(B, G, FL, FR, d > 0 ? 1ll << (d - 1) : 0, r);
+      // (halves of the shift go up or down by a square's last bit)
+      burgers_operator<NP>(B, G, FL, FR, d > 0 ? (1ll << (d - 1)) - (G[0] & 1) : 0, r);
       if (__any_sync(full, d < 0)) {   // large Courant numbers
 #pragma unroll
         for (int k = 0; k < NP; ++k) {

@@ -100,20 +100,29 @@ def _rms(got, ref):
 @pytest.mark.parametrize("rk,ratio", [("ssprk3", 1.0), ("ssprk3", 8.0), ("ssprk3", 60.0), ("rk2", 1.0),
                                       ("rk2", 4.0), ("rk2", 25.0), ("lsrk3", 25.0)])
 def test_elements_keep_the_accuracy_of_fp64_stages(rk, ratio, p):
+    _compare(rk, ratio, p, 0.01, STEPS)
+
+
+@pytest.mark.parametrize("rk,ratio,p", [("rk2", 4.0, 1), ("lsrk3", 4.0, 1), ("rk2", 1.0, 3), ("ssprk3", 4.0, 1)])
+def test_roundings_do_not_add_up(rk, ratio, p):
+    _compare(rk, ratio, p, 0.05 if p == 1 else 0.01, 200)
+
+
+def _compare(rk, ratio, p, cfl, steps):
     # 1.25: the two errors are averages over some 400 elements each, equal where the step takes
     # FP64 itself, and the FP64 arithmetic here differs from the kernels' in its order
     dx = 2.0 * math.pi / K
-    dt = 0.01 * dx
+    dt = cfl * dx
     got = ref = 0.0
     for seed in range(SEEDS):
         u0 = _patches(np.random.default_rng(seed), p, ratio)
         s = adg.Solver(adg.Config(pde="burgers", K=K, p=p, dt=dt, rk=rk), torch.tensor(u0, device="cuda"))
-        s.step(STEPS)
+        s.step(steps)
         g = s.state().cpu().numpy()
         s.close()
         f, x = u0, u0.astype(X)
         fs, xs = Scheme(np.float64, p, dt, dx), Scheme(X, p, dt, dx)
-        for _ in range(STEPS):
+        for _ in range(steps):
             f, x = fs.step(f, rk), xs.step(x, rk)
         got, ref = got + _rms(g.astype(X), x), ref + _rms(f.astype(X), x)
     assert got <= 1.25 * ref
