@@ -543,6 +543,16 @@ void fold_burgers(InstHost &h) {
     for (int j = 0; j <= H + mid; ++j) lo += B.D[i][j].y;
     B.rD[i] = (1ll << 28) + (lo >> 1);
   }
+  for (int j = 0; j <= H; ++j) {
+    long long lo = 0;
+    for (int i = 0; i < H + mid; ++i) lo += B.S[i][j].y;
+    B.rSt[j] = (1ll << 28) + (lo >> 1);
+  }
+  for (int j = 0; j <= H + mid; ++j) {
+    long long lo = 0;
+    for (int i = 0; i < H; ++i) lo += B.D[i][j].y;
+    B.rDt[j] = (1ll << 28) + (lo >> 1);
+  }
   // far from the ends of FP64's range; forward Euler's FP64 stage is one rounding (adg_bfp.cuh)
   B.ok = std::abs(B.sc) < 300 && std::abs(B.sn) < 300 && h.I.ns > 1;
 }

@@ -26,7 +26,11 @@
 // span of 3. Roundings to the nearest integer that always sent halves up, and the means of the
 // products that sums leave out, would add up step by step (with them, RK2 reached 1.9 after 200
 // steps; with a span of 6 and the scale of the elements up to a stage count away besides, 8.8
-// at a ratio of 50, and SSP-RK3 2.1).
+// at a ratio of 50, and SSP-RK3 2.1). The reverse step, whose values' scale and span are those of
+// SSP-RK3: 0.18 to 0.23 with alike elements, at most 0.79 at any ratio and on waves through zero;
+// over 500 steps at most 0.40. (Its products rounded to a unit of 2^-57 of their bound, where smooth
+// fields leave them far below it, without what the low limbs give, it reached 4 on such a wave at
+// a Courant number of 0.01 and p = 3, 22 at 0.05.)
 // A simple zero of a smooth field leaves its element within a third of its neighbours, inside
 // both spans. Forward Euler takes FP64: its stage is one rounding, which the integer path also
 // ends with. Warps with an element outside the span (or exponents near the ends of the FP64

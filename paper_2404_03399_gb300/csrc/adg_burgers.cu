@@ -609,11 +609,11 @@ __global__ void __launch_bounds__(128, NP == 4 ? 5 : 0) k_burgers_adj(const __gr
 #pragma unroll
     for (int s = 0; s < kStages; ++s) hv = max(hv, __double2hiint(yd[s][i]) & 0x7fffffff);
   }
-  const int bw = bf_window_max(hw >> 20, kStages), bv = bf_window_max(hv >> 20, 1);
+  const int bw = bf_window_max(hw >> 20, 1), bv = bf_window_max(hv >> 20, 1);
   const int Ew = bw - 1022, E = bv - 1022;
-  const int d0 = -(I.bf.sc + E + 1) - 2;   // (2 P + P') -> units of w
-  bool bad = bw < kBfMinE || bw > kBfMaxE || bv < kBfMinE || bv > kBfMaxE || d0 < -3 || !I.bf.ok;
-  bad = bad || (hw ? (hw >> 20) < bw - 6 : lo != 0);
+  const int d0 = -(I.bf.sc + E + 1);   // products (below) -> units of w
+  bool bad = bw < kBfMinE || bw > kBfMaxE || bv < kBfMinE || bv > kBfMaxE || d0 < -1 || !I.bf.ok;
+  bad = bad || (hw ? (hw >> 20) < bw - kBfSpan<false> : lo != 0);
   // ring entries below 2^60 in units of mu
   if (FACES) bad = bad || (rmax >> 20) > I.bf.sc + Ew + 1025;
 
@@ -641,14 +641,16 @@ __global__ void __launch_bounds__(128, NP == 4 ? 5 : 0) k_burgers_adj(const __gr
     auto third = [](long long x) {
       int h, l;
       fx_split(x, h, l);
-      FxAcc t;
-      fx_mac(t, make_int2(kThirdHi, kThirdLo), h, l);
-      return fx_round(t);
+      return fx_scaled(make_int2(kThirdHi, kThirdLo), h, l);
     };
-    // x y 2^-58 for |x|, |y| < 2^60, from the limbs of both
-    auto mul = [](int xh, int xl, int yh, int yl) {
-      return fx_mul(xh, yh) + ((fx_mul(xh, yl) + fx_mul(xl, yh)) >> 29);
+    // x y 2^(k - 58) rounded for |x|, |y| < 2^60, from the limbs of both
+    auto mul = [](int xh, int xl, int yh, int yl, int k) {
+      const long long c = fx_mul(xh, yl) + fx_mul(xl, yh) +
+                          (long long)__umulhi((unsigned)xl << 3, (unsigned)yl);
+      return (fx_mul(xh, yh) << k) + ((c + (1 << (28 - k))) >> (29 - k));
     };
+    // x / 4, halves to even
+    auto quarter = [](long long x) { return (x + 1 + ((x >> 2) & 1)) >> 2; };
 #pragma unroll
     for (int s = kStages - 1; s >= 0; --s) {
       long long v[NP];
@@ -662,39 +664,40 @@ __global__ void __launch_bounds__(128, NP == 4 ? 5 : 0) k_burgers_adj(const __gr
       }
       if (MID) fx_split(w[HP], sh[HP], sl[HP]);
       // a . w = ev + od, b . w = od - ev
-      FxAcc ae, ao;
+      FxAcc ae{0, B.rSt[HP]}, ao{0, B.rDt[HP + MID]};
 #pragma unroll
       for (int i = 0; i < HP + MID; ++i) fx_mac(ae, B.S[i][HP], sh[i], sl[i]);
 #pragma unroll
       for (int i = 0; i < HP; ++i) fx_mac(ao, B.D[i][HP + MID], th[i], tl[i]);
       const long long ev = fx_round(ae), od = fx_round(ao);
-      // (|od - ev| < 2^62: brought with two bits less)
-      const long long bl = bf_bring<kBfTop + 2>(__shfl_up_sync(full, (od - ev + 2) >> 2, 1), dWL, mag);
-      long long mu = ev + od + 4 * bl;
+      // (|ev|, |od| < 2^61)
+      const long long bl = bf_bring<kBfTop + 4>(__shfl_up_sync(full, od - ev, 1), dWL, mag);
+      long long mu = ev + od + bl;
       long long dl, dr;
       bf_llf_partials2(bf_bring(__shfl_up_sync(full, v[NP - 1], 1), dVL, mag), v[0], dl, dr);
       if (FACES && pe) {
         const long long r = bf_from(sR[s][lane], B.sc + Ew + 1025) << 3;
-        mag |= bf_mag(mu) >> 4;   // below 2^62
+        mag |= bf_mag(mu) >> 3;   // below 2^61
         const double m = bf_to(mu, smu);
         post[s] = s == 2 ? m * (2.0 / 3.0) : (s == 1 ? 0.25 * m : m);
         // the ring holds adjoints of the flux with beta: divided by it here
         const long long rb = s == 2 ? r + (r >> 1) : (s == 1 ? 4 * r : r);
         mu = k > 0 ? rb : mu + rb;
       }
-      mag |= bf_mag(mu) >> 4;   // below 2^62
+      mag |= bf_mag(mu) >> 3;   // below 2^61
+      // products in quarters of the unit of mu times that of the stage inputs
       int mh, ml, xh, xl;
-      fx_split((mu + 4) >> 3, mh, ml);
+      fx_split((mu + ((mu >> 1) & 1)) >> 1, mh, ml);
       fx_split(dl, xh, xl);
-      const long long pl = mul(mh, ml, xh, xl);
+      const long long pl = mul(mh, ml, xh, xl, 0);
       fx_split(dr, xh, xl);
-      const long long pr = mul(mh, ml, xh, xl);
+      const long long pr = mul(mh, ml, xh, xl, 0);
       // the left element's part, in units of this lane's w, from the lane above
       const long long pR = bf_bring<kBfTop + 2>(__shfl_down_sync(full, scale(pl + half, mag), 1), dWR, mag);
 #pragma unroll
       for (int j = 0; j < HP + MID; ++j) {
         // half the sum and half the difference of (W^T w)_j and (W^T w)_{p-j}
-        FxAcc a, b;
+        FxAcc a{0, B.rDt[j]}, b{0, j < HP ? B.rSt[j] : 0};
 #pragma unroll
         for (int i = 0; i < HP; ++i) fx_mac(a, B.D[i][j], th[i], tl[i]);
         const long long sum = fx_round(a);
@@ -708,9 +711,11 @@ __global__ void __launch_bounds__(128, NP == 4 ? 5 : 0) k_burgers_adj(const __gr
         for (int m = 0; m < (j < HP ? 2 : 1); ++m) {
           const int q = m ? NP - 1 - j : j;
           int rh, rl, vh, vl;
-          fx_split(((m ? sum - dif : sum + dif) + 2) >> 2, rh, rl);
+          const long long r = m ? sum - dif : sum + dif;
+          mag |= bf_mag(r) >> 2;   // below 2^60
+          fx_split(r, rh, rl);
           fx_split(v[q], vh, vl);
-          long long z = 2 * mul(rh, rl, vh, vl) + half;
+          long long z = mul(rh, rl, vh, vl, 1) + half;
           if (q == 0) z += pr;
           const long long x = w[q] + scale(z, mag) + (q == NP - 1 ? pR : 0);
           mag |= bf_mag(x);
@@ -718,8 +723,8 @@ __global__ void __launch_bounds__(128, NP == 4 ? 5 : 0) k_burgers_adj(const __gr
             acc[q] = third(w[q]);
             w[q] = third(2 * x);
           } else if (s == 1) {
-            acc[q] += (3 * w[q] + 2) >> 2;
-            w[q] = (x + 2) >> 2;
+            acc[q] += quarter(3 * w[q]);
+            w[q] = quarter(x);
           } else {
             w[q] = x + acc[q];
             mag |= bf_mag(w[q]);

@@ -116,11 +116,13 @@ struct FxSlot {
 // rS, rD: what the second accumulator of a row's sum starts from, in units of 2^-29: the rounding
 // half-unit and the mean of the low limb products that fx_mac leaves out (half the sum of the
 // low coefficient limbs, the low limbs of the values being even over [0, 2^29)). Left out, they
-// add up step by step, since a coefficient's low limb keeps its sign.
+// add up step by step, since a coefficient's low limb keeps its sign. rSt, rDt: the same for
+// sums over i (the adjoint's).
 struct BurgersFixed {
   int2 S[(kMaxNp + 1) / 2][kMaxNp / 2 + 1];
   int2 D[kMaxNp / 2][(kMaxNp + 1) / 2 + 1];
   long long rS[(kMaxNp + 1) / 2], rD[kMaxNp / 2];
+  long long rSt[kMaxNp / 2 + 1], rDt[(kMaxNp + 1) / 2 + 1];
   int sc, ok;
   // the 2N coefficients (|c| < 2: limbs of round(c 2^58)), and 2 nu / dt = vn 2^sn (vn <= 1)
   int2 lsA[kMaxStages], lsB[kMaxStages];

@@ -1,7 +1,8 @@
-"""Errors of the fused Burgers step element by element, each over the element's own largest value,
-on rough fields whose patches of four elements differ in size: the step holds an element in
-integers at a scale of its neighbourhood, which must not cost a small element the accuracy that
-FP64 stages give it. Both are measured against the same scheme in extended precision."""
+"""Errors of the fused Burgers step and its adjoint element by element, each over the element's own
+largest value, on rough fields whose patches of four elements differ in size and on waves
+through zero: the steps hold an element in integers at a scale of its neighbourhood, which must
+not cost a small element the accuracy that FP64 stages give it. Both are measured against the
+same scheme in extended precision."""
 import math
 
 import numpy as np
@@ -86,6 +87,31 @@ class Scheme:
         return v
 
 
+    def reverse(self, w, y):
+        """The adjoint of an SSP-RK3 step's result to that of its input; y: its stage inputs."""
+        T, acc = self.T, 0
+        h = T(0.5)
+        for s in (2, 1, 0):
+            al, be = SHU_OSHER[s]
+            (A, l0, lp), v = self.const(be), y[s]
+            sl = sum(l0[i] * w[:, i] for i in range(self.Np))
+            sr = sum(lp[i] * w[:, i] for i in range(self.Np))
+            lv = T(be) * w + 2 * v * sum(A[i][None, :] * w[:, i, None] for i in range(self.Np))
+            lv[:, 0] += v[:, 0] * sl
+            lv[:, -1] += v[:, -1] * sr
+            mu = -sl - np.roll(sr, 1)
+            a, b = np.roll(v[:, -1], 1), v[:, 0]
+            left = abs(a) >= abs(b)
+            lam = np.where(left, abs(a), abs(b))
+            gl = np.where(left, np.where(a >= 0, T(1), T(-1)), T(0))
+            gr = np.where(left, T(0), np.where(b >= 0, T(1), T(-1)))
+            lv[:, 0] += mu * (h * b - h * lam - h * gr * (b - a))
+            lv[:, -1] += np.roll(mu * (h * a + h * lam - h * gl * (b - a)), -1)
+            acc = acc + T(al) * w
+            w = lv
+        return acc + w
+
+
 def _patches(rng, p, ratio):
     u = 0.7 + 0.28 * rng.uniform(-1.0, 1.0, (K, p + 1))
     return u * np.where((np.arange(K) // 4) % 2 == 0, 1.0, 1.0 / ratio)[:, None]
@@ -125,4 +151,36 @@ def _compare(rk, ratio, p, cfl, steps):
         for _ in range(steps):
             f, x = fs.step(f, rk), xs.step(x, rk)
         got, ref = got + _rms(g.astype(X), x), ref + _rms(f.astype(X), x)
+    assert got <= 1.25 * ref
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("field", [1.0, 8.0, 60.0, "wave"])
+def test_gradient_elements_keep_the_accuracy_of_fp64_stages(field, p):
+    # misfits of the final state in patches, or a wave through zero; 1.25 as above
+    dx = 2.0 * math.pi / K
+    dt = 0.01 * dx
+    x = (np.arange(K)[:, None] + np.linspace(0.0, 1.0, p + 1)[None]) * dx
+    got = ref = 0.0
+    for seed in range(SEEDS):
+        u0 = 0.5 + np.sin(x + seed)
+        d = np.sin(3.0 * x + seed) if field == "wave" else _patches(np.random.default_rng(seed), p, field)
+        s = adg.Solver(adg.Config(pde="burgers", K=K, p=p, dt=dt), torch.tensor(u0, device="cuda"))
+        s.step(STEPS)
+        end = s.state().cpu().numpy()
+        s.close()
+        target = end - d
+        s = adg.Solver(adg.Config(pde="burgers", K=K, p=p, dt=dt), torch.tensor(u0, device="cuda"))
+        g = s.grad(torch.tensor(target, device="cuda"), STEPS, STEPS)[1].cpu().numpy()
+        s.close()
+        fs, xs = Scheme(np.float64, p, dt, dx), Scheme(X, p, dt, dx)
+        rec, u = [], u0.astype(X)
+        for _ in range(STEPS):
+            u = xs.step(u, "ssprk3", rec)
+        w = ((end.astype(X) - target.astype(X)) @ xs.M) * (X(dx) / 2)
+        f = w.astype(np.float64)
+        for n in range(STEPS - 1, -1, -1):
+            y = rec[3 * n:3 * n + 3]
+            w, f = xs.reverse(w, y), fs.reverse(f, [v.astype(np.float64) for v in y])
+        got, ref = got + _rms(g.astype(X), w), ref + _rms(f.astype(X), w)
     assert got <= 1.25 * ref
