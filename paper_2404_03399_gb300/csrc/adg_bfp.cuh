@@ -23,14 +23,17 @@
 // elements, integer over FP64): SSP-RK3 0.17 at equal patches, 0.18 to 0.26 at a ratio of 8 and
 // at most 1.00 beyond with a span of 4; the 2N schemes, whose FP64 stages round once or twice,
 // 0.45 (five stages) to 0.72 (RK2) at equal patches, at most 0.89 at 8 and 1.06 beyond with a
-// span of 3. Roundings to the nearest integer that always sent halves up, and the means of the
-// products that sums leave out, would add up step by step (with them, RK2 reached 1.9 after 200
-// steps; with a span of 6 and the scale of the elements up to a stage count away besides, 8.8
-// at a ratio of 50, and SSP-RK3 2.1). The reverse step, whose values' scale and span are those of
-// SSP-RK3: 0.18 to 0.23 with alike elements, at most 0.79 at any ratio and on waves through zero;
-// over 500 steps at most 0.40. (Its products rounded to a unit of 2^-57 of their bound, where smooth
-// fields leave them far below it, without what the low limbs give, it reached 4 on such a wave at
-// a Courant number of 0.01 and p = 3, 22 at 0.05.)
+// span of 3. The means of the products that sums leave out, and (in the 2N schemes) roundings
+// that send every half up, add up step by step: with them RK2 reached 1.9 after 200 steps.
+// SSP-RK3 keeps the latter (2 to 4% of a step to even out), since its FP64 stages lose a unit
+// of 2^-54 a step in 1/3 + 2/3: it stays below 0.1. With a span of 6 and the scale of the
+// elements up to a stage count away, RK2 reached 8.8 at a ratio of 50 and SSP-RK3 2.1.
+// The reverse step, whose scale and span are those of SSP-RK3: 0.18 to 0.23 with alike elements,
+// at most 0.79 at any ratio and on waves through zero, at most 0.40 over 500 steps. (Its
+// products rounded to a unit of 2^-57 of their bound, where smooth fields leave them far
+// below it, and without the low limbs' product, it reached 4 on such a wave at a Courant
+// number of 0.01 and p = 3, 22 at 0.05.)
+//
 // A simple zero of a smooth field leaves its element within a third of its neighbours, inside
 // both spans. Forward Euler takes FP64: its stage is one rounding, which the integer path also
 // ends with. Warps with an element outside the span (or exponents near the ends of the FP64
@@ -93,7 +96,8 @@ __device__ __forceinline__ long long bf_square(int xh, int xl) {
 // Local Lax-Friedrichs flux 1/4 (a^2 + b^2) - 1/2 max(|a|, |b|) (b - a) of the traces a = u^-,
 // b = u^+ with squares ga, gb, in the squares' units. With the larger trace x the last product
 // is +-(a b - x^2): one product and no magnitudes (the sign is x's, and the other one for b);
-// equal traces give a b = a^2 exactly. Halves go up or down by a bit of gb.
+// equal traces give a b = a^2 exactly. EVEN: halves go up or down by a bit of gb.
+template <bool EVEN>
 __device__ __forceinline__ long long bf_llf(long long a, long long b, long long ga, long long gb) {
   int ah, al, bh, bl;
   fx_split(a, ah, al);
@@ -103,7 +107,7 @@ __device__ __forceinline__ long long bf_llf(long long a, long long b, long long 
   const bool left = ga >= gb;
   const long long t = left ? ab - ga : gb - ab;
   const long long s = (long long)((int)((left ? a : b) >> 32) >> 31);   // 0 or -1
-  return (ga + gb - 2 * ((t ^ s) - s) + 2 - ((gb >> 1) & 1)) >> 2;
+  return (ga + gb - 2 * ((t ^ s) - s) + 2 - (EVEN ? (gb >> 1) & 1 : 0)) >> 2;
 }
 
 // 1/3 as limbs of round(2^58 / 3).

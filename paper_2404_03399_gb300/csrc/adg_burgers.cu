@@ -303,7 +303,7 @@ if constexpr (!LS && !VISC) {
         fx_split(vl, xh, xl);
         gl = bf_square(xh, xl);
       }
-      long long FL = bf_llf(vl, v[0], gl, G[0]);
+      long long FL = bf_llf<LS>(vl, v[0], gl, G[0]);
       const size_t at = FACES && pe ? ((size_t)nm * I.ns + s) * I.P + e / I.Kpe : 0;
       if (FACES && pe) {
         if (own) I.ring[at] = make_double2(bf_to(FL, sg), VISC ? bf_to(vl, E - 57) : 0.0);
@@ -364,8 +364,8 @@ if constexpr (!LS && !VISC) {
       if (!LS) d = s == 0 ? d : (s == 1 ? d + 2 : d - 1);
       d = d > 60 ? 60 : d;
       long long r[NP];
-      // (halves of the shift go up or down by a square's last bit)
-      burgers_operator<NP>(B, G, FL, FR, d > 0 ? (1ll << (d - 1)) - (G[0] & 1) : 0, r);
+      // (2N: halves of the shift go up or down by a square's last bit)
+      burgers_operator<NP>(B, G, FL, FR, d > 0 ? (1ll << (d - 1)) - (LS ? G[0] & 1 : 0) : 0, r);
       if (__any_sync(full, d < 0)) {   // large Courant numbers
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
