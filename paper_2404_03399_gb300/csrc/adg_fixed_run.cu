@@ -414,6 +414,11 @@ bool run_shape(const Inst &I, int &nb, int &elems) {
   return !I.async || run_faces(I, most) <= kRunFaces;
 }
 
+// The most dynamic shared memory of a block that an instance's run may take: the kernels' limit,
+// set to this whatever the instance, since it belongs to the kernel and other open instances
+// launch it with their own sizes.
+constexpr size_t kRunSmem = 200 * 1024;
+
 // Dynamic shared memory of a block.
 size_t run_smem(const Inst &I, size_t fixed) {
   int nb, elems;
@@ -429,10 +434,10 @@ cudaError_t run_prepare(const Inst &I) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   if (e == cudaSuccess && !coop) return cudaErrorNotSupported;
   const size_t smem = run_smem(I, sizeof(RunShared<NP, S>));
-  if (smem > 200 * 1024) return cudaErrorNotSupported;
+  if (smem > kRunSmem) return cudaErrorNotSupported;
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_fixed_run<NP, S, FACES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+                             (int)kRunSmem);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fixed_run<NP, S, FACES>,
                                                       kRunBlock, smem);
