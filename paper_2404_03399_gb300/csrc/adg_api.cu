@@ -2080,8 +2080,10 @@ int begin_ctx(adg_ctx *c, void *stream) {
 struct DevBuf {
   void *p = nullptr;
   cudaStream_t s = nullptr;
-  ~DevBuf() {
+  ~DevBuf() { free(); }
+  void free() {
     if (p) cudaFreeAsync(p, s);
+    p = nullptr;
   }
   double *d() const { return static_cast<double *>(p); }
 };
@@ -2277,19 +2279,6 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
   const int64_t n0 = c->n;
   const bool states = I.pde == ADG_BURGERS;
   DevBuf g, ck_u, ck_ring, seg, lam, lring, ck_fx;
-  // a segment's delays are one window of the table; and a run whose recorded stage inputs all
-  // fit in what the pool keeps is one segment, recorded on the way (nothing is recomputed; the
-  // gradient does not depend on C)
-  if (I.async) C = std::min(C, h.TR);
-  if (states && nsteps > C && nsteps <= (I.async ? h.TR : std::numeric_limits<int>::max()) &&
-      ((size_t)nsteps * kStages + 1) * nd * sizeof(double) <= kPoolKeep) {
-    if (pool_alloc(c, seg, ((size_t)nsteps * kStages + 1) * nd * sizeof(double)) == cudaSuccess)
-      C = (int)nsteps;
-    else
-      (void)cudaGetLastError();
-  }
-  const int64_t nseg = nsteps == 0 ? 0 : (nsteps + C - 1) / C;
-  const int64_t nck = states ? nseg : std::min<int64_t>(nseg, 1);
   const size_t ring_n = I.async ? (size_t)I.R * kStages * I.P : 0;
   const int dir = I.a >= 0.0 ? 1 : -1;
 
@@ -2305,12 +2294,36 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
                        3 * sizeof(adg::FxSlot), cudaMemcpyDeviceToDevice, c->stream));
   }
   r = dev_alloc(c, g, nd * sizeof(double));
-  if (!r) r = dev_alloc(c, ck_u, (size_t)nck * nd * sizeof(double));
-  if (!r) r = dev_alloc(c, ck_ring, (size_t)nck * ring_n * sizeof(double2));
-  if (!r && states && !seg.p) r = dev_alloc(c, seg, ((size_t)C * kStages + 1) * nd * sizeof(double));
   if (!r) r = dev_alloc(c, lam, 4 * nd * sizeof(double));
   if (!r) r = dev_alloc(c, lring, ring_n * sizeof(double));
   if (r) return r;
+  // a segment's delays are one window of the table; and a run whose recorded stage inputs all
+  // fit in what the pool keeps is one segment, recorded on the way (nothing is recomputed; the
+  // gradient does not depend on C), if there is room for it besides
+  if (I.async) C = std::min(C, h.TR);
+  const int64_t room = (int64_t)(kPoolKeep / (nd * sizeof(double)));   // fields
+  if (states && nsteps > C && nsteps <= (I.async ? h.TR : std::numeric_limits<int>::max()) &&
+      nsteps <= (room - 1) / kStages) {
+    if (pool_alloc(c, seg, ((size_t)nsteps * kStages + 1) * nd * sizeof(double)) == cudaSuccess &&
+        pool_alloc(c, ck_u, nd * sizeof(double)) == cudaSuccess &&
+        (!ring_n || pool_alloc(c, ck_ring, ring_n * sizeof(double2)) == cudaSuccess)) {
+      C = (int)nsteps;
+    } else {
+      (void)cudaGetLastError();
+      seg.free();
+      ck_u.free();
+      CK(cudaStreamSynchronize(c->stream));
+      CK(cudaMemPoolTrimTo(c->pool, 0));   // what the pool does not use, for the segments
+    }
+  }
+  const int64_t nseg = nsteps == 0 ? 0 : (nsteps + C - 1) / C;
+  const int64_t nck = states ? nseg : std::min<int64_t>(nseg, 1);
+  if (!seg.p) {
+    r = dev_alloc(c, ck_u, (size_t)nck * nd * sizeof(double));
+    if (!r) r = dev_alloc(c, ck_ring, (size_t)nck * ring_n * sizeof(double2));
+    if (!r && states) r = dev_alloc(c, seg, ((size_t)C * kStages + 1) * nd * sizeof(double));
+    if (r) return r;
+  }
   CK(adg::launch_to_internal(target_dev, g.d(), K, Np, c->stream));
 
   // Forward pass with checkpoints (u^n and the forward ring at each segment start). The last
