@@ -262,11 +262,17 @@ int adg_get_fixed_basis(adg_ctx *c, int32_t index, int32_t *basis_out);
  * of the delay table's window when delays are in use), recomputation in between; a run whose
  * recorded states fit in 1 GiB is recorded whole instead (the result does not depend on it).
  * The working memory comes from a pool of the context, which keeps up to 1 GiB of it until
- * adg_destroy. target_dev and grad_u0_dev are device (K, p+1) row-major FP64; J_out is host.
+ * adg_destroy. adg_set_grad_memory sets both limits. target_dev and grad_u0_dev are device (K, p+1) row-major FP64; J_out is host.
  * The paper has no adjoint; this follows the discrete forward scheme exactly.
  */
 int adg_grad(adg_ctx *c, const double *target_dev, int64_t nsteps, int32_t ckpt_every,
              double *grad_u0_dev, double *J_out);
+
+/* Device memory of adg_grad (not a paper quantity): `bytes` (>= 0; 2^30 unless set) is the most
+ * that a run's recorded states may take to be recorded whole instead of in segments of
+ * ckpt_every steps, and what the context keeps of the working memory between calls. 0: always
+ * the segments, nothing kept. What is kept beyond it already is given back. Synchronises. */
+int adg_set_grad_memory(adg_ctx *c, int64_t bytes);
 
 /* Discrete integral sum_e (dx/2) w^T u^e of instance `index` (Section 4.1 conservation
  * check), into *out (host). Synchronises. */

@@ -231,6 +231,11 @@ class Solver:
                               out.data_ptr(), C.byref(J)), self.ctx)
         return J.value, out
 
+    def set_grad_memory(self, nbytes: int) -> None:
+        """What ``grad`` may take to record a run whole and keeps between calls (2**30 unless
+        set; 0: always segments of ``ckpt_every`` steps, nothing kept)."""
+        check(load().adg_set_grad_memory(self.ctx, int(nbytes)), self.ctx)
+
     def close(self) -> None:
         if self._ctx is not None:
             load().adg_destroy(self._ctx)

@@ -78,6 +78,7 @@ def load(require: bool = True):
         "adg_get_variant": (C.c_int, [vp, i32, C.POINTER(i32), C.POINTER(i32)]),
         "adg_get_fixed_basis": (C.c_int, [vp, i32, C.POINTER(i32)]),
         "adg_grad": (C.c_int, [vp, vp, i64, i32, vp, dp]),
+        "adg_set_grad_memory": (C.c_int, [vp, i64]),
         "adg_integral": (C.c_int, [vp, i32, dp]),
         "adg_check_finite": (C.c_int, [vp]),
         "adg_delay_table": (C.c_int, [cfgp, i64, i64, C.POINTER(C.c_uint8)]),

@@ -368,6 +368,7 @@ struct adg_ctx {
   cudaStream_t stream = nullptr;
   cudaStream_t cap = nullptr;
   cudaMemPool_t pool = nullptr;   // working memory of the gradient and the misfit
+  uint64_t grad_keep = uint64_t(1) << 30;   // ... kept between calls; a whole recording's limit
   int device = 0;
   std::vector<InstHost> inst;
   bool batch = false;
@@ -2089,10 +2090,9 @@ struct DevBuf {
 };
 
 // The context's memory pool (the gradient's and the misfit's working fields): it keeps up to
-// kPoolKeep bytes between calls, which a repeated gradient would otherwise allocate and free
-// each time, and is destroyed with the context (with direct launches instead of graphs, 3.92 -> 3.04
-// ms for the gradient of 100 steps on 65536 elements).
-constexpr uint64_t kPoolKeep = uint64_t(1) << 30;
+// grad_keep bytes (adg_set_grad_memory) between calls, which a repeated gradient would otherwise
+// allocate and free each time, and is destroyed with the context (with direct launches instead of
+// graphs, 3.92 -> 3.04 ms for the gradient of 100 steps on 65536 elements).
 
 cudaError_t pool_alloc(adg_ctx *c, DevBuf &b, size_t bytes) {
   if (!c->pool) {
@@ -2105,7 +2105,7 @@ cudaError_t pool_alloc(adg_ctx *c, DevBuf &b, size_t bytes) {
       c->pool = nullptr;
       return e;
     }
-    uint64_t keep = kPoolKeep;
+    uint64_t keep = c->grad_keep;
     e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
     if (e != cudaSuccess) return e;
   }
@@ -2113,6 +2113,13 @@ cudaError_t pool_alloc(adg_ctx *c, DevBuf &b, size_t bytes) {
   if (e != cudaSuccess) b.p = nullptr;
   b.s = c->stream;
   return e;
+}
+
+// After a call that used the pool: with nothing to be kept, its memory back to the device.
+void give_back(adg_ctx *c) {
+  if (!c->pool || c->grad_keep) return;
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess || cudaMemPoolTrimTo(c->pool, 0) != cudaSuccess)
+    (void)cudaGetLastError();
 }
 
 int dev_alloc(adg_ctx *c, DevBuf &b, size_t bytes) {
@@ -2301,7 +2308,7 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
   // fit in what the pool keeps is one segment, recorded on the way (nothing is recomputed; the
   // gradient does not depend on C), if there is room for it besides
   if (I.async) C = std::min(C, h.TR);
-  const int64_t room = (int64_t)(kPoolKeep / (nd * sizeof(double)));   // fields
+  const int64_t room = (int64_t)(c->grad_keep / (nd * sizeof(double)));   // fields
   if (states && nsteps > C && nsteps <= (I.async ? h.TR : std::numeric_limits<int>::max()) &&
       nsteps <= (room - 1) / kStages) {
     if (pool_alloc(c, seg, ((size_t)nsteps * kStages + 1) * nd * sizeof(double)) == cudaSuccess &&
@@ -3067,11 +3074,16 @@ int adg_misfit(adg_ctx *c, int32_t index, const double *target_dev, double *J_ou
     return fail(c, ADG_EINVAL, "bad argument");
   InstHost &h = c->inst[index];
   const size_t nd = (size_t)h.I.K * h.I.Np;
-  DevBuf g;
-  int r = dev_alloc(c, g, nd * sizeof(double));
-  if (r) return r;
-  CK(adg::launch_to_internal(target_dev, g.d(), h.I.K, h.I.Np, c->stream));
-  return reduce(c, h, 3, g.d(), 0.5 * (h.dx / 2.0), J_out);
+  int r;
+  {
+    DevBuf g;
+    r = dev_alloc(c, g, nd * sizeof(double));
+    if (r) return r;
+    CK(adg::launch_to_internal(target_dev, g.d(), h.I.K, h.I.Np, c->stream));
+    r = reduce(c, h, 3, g.d(), 0.5 * (h.dx / 2.0), J_out);
+  }
+  give_back(c);
+  return r;
 }
 
 int adg_check_finite(adg_ctx *c) {
@@ -3138,7 +3150,22 @@ int adg_grad(adg_ctx *c, const double *target_dev, int64_t nsteps, int32_t ckpt_
   if (!target_dev || !grad_u0_dev || !J_out) return fail(c, ADG_EINVAL, "NULL target, gradient or J");
   int r = sync_state(c);
   if (r) return r;
-  return run_gradient(c, target_dev, nsteps, ckpt_every, grad_u0_dev, J_out);
+  r = run_gradient(c, target_dev, nsteps, ckpt_every, grad_u0_dev, J_out);
+  give_back(c);
+  return r;
+}
+
+int adg_set_grad_memory(adg_ctx *c, int64_t bytes) {
+  if (!c) return fail(nullptr, ADG_EINVAL, "ctx is NULL");
+  if (bytes < 0) return fail(c, ADG_EINVAL, "need bytes >= 0");
+  if (c->pool) {
+    uint64_t keep = (uint64_t)bytes;
+    CK(cudaStreamSynchronize(c->stream));
+    CK(cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    CK(cudaMemPoolTrimTo(c->pool, keep));
+  }
+  c->grad_keep = (uint64_t)bytes;
+  return ADG_OK;
 }
 
 }  // extern "C"
