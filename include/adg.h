@@ -46,8 +46,9 @@ typedef enum {
   ADG_ENOMEM = -2,     /* device or host allocation failed */
   ADG_ECUDA = -3,      /* CUDA runtime error (or no device) */
   ADG_ENONFINITE = -4, /* a NaN or Inf was found in the state */
-  ADG_ETIMEOUT = -5,   /* a bounded device wait ran out (reported by the next call that waits
-                          for the stream; the state is lost) */
+  ADG_ETIMEOUT = -5,   /* a bounded device wait ran out (adg_set_wait_limit; reported by the next
+                          call that waits for the stream, and by every adg_step from then on;
+                          the state is lost) */
   ADG_ESTATE = -6      /* call not valid in the context's current state */
 } adg_status;
 
@@ -221,6 +222,12 @@ int adg_batch_init(const adg_config *cfgs, const double *const *u0_devs, int32_t
  * says otherwise; Section 4.2.1 structure, Eq. EulerDG-style explicit updates; Eq.
  * asyncEulerDGconserved at PE faces). Asynchronous: returns once the work is queued. */
 int adg_step(adg_ctx *c, int64_t nsteps);
+
+/* Polls (>= 0) after which a block of the cooperative run kernel gives up its wait for the other
+ * blocks of the launch (fixed-point steps on meshes of up to about 900 elements per SM; 2^22
+ * unless set, some seconds), and adg_step's work ends with ADG_ETIMEOUT. A program whose other
+ * kernels may hold SMs for longer beside a run gives more. For steps queued from then on. */
+int adg_set_wait_limit(adg_ctx *c, int64_t polls);
 
 /* Advance to time t_end: ceil(t_end/dt - 1e-9) - (current step) steps (none if <= 0). */
 int adg_run(adg_ctx *c, double t_end);

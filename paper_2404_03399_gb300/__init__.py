@@ -215,6 +215,10 @@ class Solver:
     def check_finite(self) -> None:
         check(load().adg_check_finite(self.ctx), self.ctx)
 
+    def set_wait_limit(self, polls: int) -> None:
+        """Polls after which a block of a run kernel gives up its wait for the others."""
+        check(load().adg_set_wait_limit(self.ctx, int(polls)), self.ctx)
+
     def misfit(self, target: torch.Tensor) -> float:
         """J = 1/2 ||u - g||_M^2 of the current state against target g."""
         g = _as_field(target, self.cfg.K, self.Np, 3 if self.cfg.pde == "euler" else 1)

@@ -71,6 +71,7 @@ def load(require: bool = True):
         "adg_init_host": (C.c_int, [cfgp, vp, vp, C.POINTER(vp)]),
         "adg_batch_init": (C.c_int, [cfgp, C.POINTER(vp), i32, vp, C.POINTER(vp)]),
         "adg_step": (C.c_int, [vp, i64]),
+        "adg_set_wait_limit": (C.c_int, [vp, i64]),
         "adg_run": (C.c_int, [vp, C.c_double]),
         "adg_get_state": (C.c_int, [vp, i32, vp, C.POINTER(i64)]),
         "adg_get_state_host": (C.c_int, [vp, i32, vp, C.POINTER(i64)]),

@@ -406,6 +406,7 @@ struct adg_ctx {
   int G = 32;                      // steps per graph (128 measured slower: 78.5 against
                                    // 77.2 ms for 2000 steps of the adjoint workload)
   int64_t n = 0;
+  long long polls = adg::kRunPolls;   // of a run kernel's wait for its other blocks
   // set by a kernel whose bounded wait ran out (mapped host memory, read after a synchronisation)
   int *timeout() const { return reinterpret_cast<int *>(pinned + 7); }
 };
@@ -1350,12 +1351,17 @@ int ensure_pinned(adg_ctx *c) {
   return ADG_OK;
 }
 
-// Waits for the context's stream; a bounded device wait that ran out shows here.
-int sync_stream(adg_ctx *c) {
-  CK(cudaStreamSynchronize(c->stream));
+// ADG_ETIMEOUT once a bounded device wait that ran out has shown.
+int check_timeout(adg_ctx *c) {
   if (c->pinned && *static_cast<volatile int *>(c->timeout()))
     return fail(c, ADG_ETIMEOUT, "a run kernel's wait for its other blocks ran out");
   return ADG_OK;
+}
+
+// Waits for the context's stream; a bounded device wait that ran out shows here.
+int sync_stream(adg_ctx *c) {
+  CK(cudaStreamSynchronize(c->stream));
+  return check_timeout(c);
 }
 
 int reduce(adg_ctx *c, InstHost &h, int kind, const double *g, double scale, double *host_out,
@@ -1987,7 +1993,7 @@ int launch_fused_steps(adg_ctx *c, int nsteps, int kind) {
       from = rel = 1;
     }
     const int end = fixed_end(kind == kChunkFP64 ? 0 : kind, nsteps);
-    CK(adg::launch_fixed_run(I, adg::fixed_run(c->inst[0].run, c->timeout()), f[from], f[end], rel,
+    CK(adg::launch_fixed_run(I, adg::fixed_run(c->inst[0].run, c->timeout(), c->polls), f[from], f[end], rel,
                              nsteps - rel, c->stream));
     CK(adg::launch_advance(c->meta, 2, 1, nsteps, c->stream));
     return ADG_OK;
@@ -2937,6 +2943,7 @@ int adg_batch_init(const adg_config *cfgs, const double *const *u0_devs, int32_t
 int adg_step(adg_ctx *c, int64_t nsteps) {
   if (!c) return fail(nullptr, ADG_EINVAL, "ctx is NULL");
   if (nsteps < 0) return fail(c, ADG_EINVAL, "nsteps must be >= 0");
+  if (int r = check_timeout(c)) return r;
   // the fixed-point step carries its int64 state from chunk to chunk and call to call
   const bool carry = fixed_state(c);
   // CUDA graphs of G steps where launches dominate; larger runs launch chunks of up to
@@ -2969,6 +2976,13 @@ int adg_step(adg_ctx *c, int64_t nsteps) {
     c->n += chunk;
     left -= chunk;
   }
+  return ADG_OK;
+}
+
+int adg_set_wait_limit(adg_ctx *c, int64_t polls) {
+  if (!c) return fail(nullptr, ADG_EINVAL, "ctx is NULL");
+  if (polls < 0) return fail(c, ADG_EINVAL, "need polls >= 0");
+  c->polls = polls;
   return ADG_OK;
 }
 

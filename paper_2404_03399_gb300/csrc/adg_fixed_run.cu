@@ -19,7 +19,6 @@ constexpr int kRunTile = 2 * kRunThreads;
 constexpr int kRunFaces = 32;                  // PE faces of a block's tile
 constexpr int kRunFaceWarps = 3;               // at most, in a block of at most 512 threads
 constexpr int kRunBlock = 512;                 // (128 registers)
-constexpr long long kRunPolls = 1ll << 22;     // of the grid barrier: some seconds
 
 // Shared memory of a block; behind it the tile's faces' ring [faces][R][S], their delays
 // [nsteps][faces] and the AT coefficients.
@@ -46,7 +45,7 @@ struct RunWords {
 
 // Arrival of a block whose OR has bit length top (bits: the field's length of the step before),
 // and the wait for all nb: the field's new length, or -1 when the wait ran out.
-__device__ __forceinline__ int run_barrier(RunWords *w, int t, int nb, int top, int bits) {
+__device__ __forceinline__ int run_barrier(RunWords *w, int t, int nb, int top, int bits, long long most) {
   unsigned long long *a = &w->arrived[t];
   if (top != bits)
     asm volatile("red.relaxed.gpu.global.max.u32 [%0], %1;" ::"l"(&w->top[t]), "r"(top) : "memory");
@@ -55,7 +54,7 @@ __device__ __forceinline__ int run_barrier(RunWords *w, int t, int nb, int top, 
       1ull | (top == bits ? 1ull << 16 : 0ull) | (top > bits ? 1ull << 32 : 0ull);
   asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(a), "l"(add) : "memory");
   unsigned long long v = 0;
-  for (long long polls = 0; polls < kRunPolls; ++polls) {
+  for (long long polls = 0; polls < most; ++polls) {
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(a) : "memory");
     if ((int)(v & 0xffffu) == nb) break;
   }
@@ -150,7 +149,7 @@ __device__ __forceinline__ void run_face(const Inst &I, RunShared<NP, S> &sh, co
 //   * the corrections sum_s R_s d_s of the elements around each face are added;
 //   * the block's last 2S-1 elements go to its exchange slot, and the block arrives at the
 //     grid's barrier, whose word also carries the reduction of the next step's scale. The wait
-//     is bounded: after kRunPolls polls a block sets *err and returns.
+//     is bounded: after `polls` polls a block sets *err and returns.
 // Bound by latency: the chain through a tile's elements, the faces' differences and the barrier.
 // K = 65536, p = 3, ADG-AT3 (256 PEs): 8.9 us a step as two kernels in a graph, 5.0 us so
 // with the read of the state (sync steps alone 3.9 -> 3.0 us). (Every block
@@ -160,7 +159,7 @@ template <int NP, int S, bool FACES>
 __global__ void __launch_bounds__(kRunBlock, 1)
     k_fixed_run(const __grid_constant__ Inst I, const long long *__restrict__ in,
                 long long *__restrict__ out, int rel, int nsteps, int elems, RunWords *words,
-                long long *exch, int *err) {
+                long long *exch, int *err, long long polls) {
   constexpr int HL = 2 * S - 1;   // elements left of the tile that the faces' traces reach
   constexpr int G = kFaceLanes<S>;
   extern __shared__ __align__(16) unsigned char smem_[];
@@ -367,7 +366,7 @@ __global__ void __launch_bounds__(kRunBlock, 1)
     if (halo_warp && lane == 0) {
       const unsigned long long m = sh.mag;
       int top = m ? 64 - __clzll((long long)m) : 0;
-      if (nb > 1) top = run_barrier(words, t, nb, top, bits);
+      if (nb > 1) top = run_barrier(words, t, nb, top, bits, polls);
       sh.stop = top < 0;
       sh.bits = top;
     }
@@ -463,7 +462,7 @@ cudaError_t run_launch(const Inst &I, int nb, int elems, const long long *in, lo
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_fixed_run<NP, S, FACES>, I, in, out, rel, nsteps, elems,
-                            static_cast<RunWords *>(R.words), R.exch, R.err);
+                            static_cast<RunWords *>(R.words), R.exch, R.err, R.polls);
 }
 
 template <class F>
@@ -514,8 +513,8 @@ size_t fixed_run_bytes(const Inst &I) {
   return sizeof(RunWords) + 2 * (size_t)nb * (2 * I.ns - 1) * I.Np * sizeof(long long);
 }
 
-FixedRun fixed_run(void *buf, int *err) {
-  return {buf, reinterpret_cast<long long *>(static_cast<char *>(buf) + sizeof(RunWords)), err};
+FixedRun fixed_run(void *buf, int *err, long long polls) {
+  return {buf, reinterpret_cast<long long *>(static_cast<char *>(buf) + sizeof(RunWords)), err, polls};
 }
 
 cudaError_t launch_fixed_run(const Inst &I, const FixedRun &R, const void *in, void *out, int rel,

@@ -301,15 +301,17 @@ cudaError_t launch_fixed_step(const Inst &I, const void *uin, void *uout, int re
 // to about 900 elements per SM): its device buffer's size (0: the instance takes the step and
 // face kernels), the buffer's parts, and nsteps steps from the int64 field in (state of step
 // meta[0] + rel) to out (the same results as launch_fixed_step and launch_face_step). *err
-// (host-mapped) is set when its bounded wait ran out.
+// (host-mapped) is set when its wait of at most `polls` polls ran out.
 struct FixedRun {
   void *words;
   long long *exch;
   int *err;
+  long long polls;
 };
+constexpr long long kRunPolls = 1ll << 22;   // unless set otherwise: some seconds
 constexpr int kRunSteps = 256;   // of one launch
 size_t fixed_run_bytes(const Inst &I);
-FixedRun fixed_run(void *buf, int *err);
+FixedRun fixed_run(void *buf, int *err, long long polls);
 cudaError_t launch_fixed_run(const Inst &I, const FixedRun &R, const void *in, void *out, int rel,
                              int nsteps, cudaStream_t s);
 // A launch with the programmatic-stream-serialization attribute when pdl is set, with smem bytes
