@@ -1714,8 +1714,13 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
   }
 
   if (I.async) {
-    if (I.euler) I.R += adg::kEulerSteps - 1;
-    if (I.pde == ADG_ADVECTION && !I.fused && !I.ls) I.R += adg::kAdvSteps - 1;
+    // spare slots only where a launch takes several steps: the stage kernels load every level of a
+    // ring of up to kPrefetchR at once, and more slots are memory and checkpoints for nothing
+    if (!c->batch) {
+      if (I.euler && adg::euler_steps_per_launch(I)) I.R += adg::kEulerSteps - 1;
+      if (I.pde == ADG_ADVECTION && !I.fused && !I.ls && adg::adv_steps_per_launch(I))
+        I.R += adg::kAdvSteps - 1;
+    }
     const int q = h.q_eff, L = cfg->L;
     std::vector<double> cf((size_t)L * q * q, 0.0);
     for (int k = 0; k < L; ++k)
