@@ -23,7 +23,7 @@ EXPORTS = [
     "adg_get_state", "adg_get_dt", "adg_get_variant", "adg_grad", "adg_integral", "adg_check_finite",
     "adg_delay_table", "adg_eval_modes", "adg_lgl_nodes", "adg_last_error", "adg_destroy",
     "adg_integral_noalloc", "adg_misfit", "adg_comm_stats", "adg_get_fixed_basis",
-    "adg_init_host", "adg_get_state_host",
+    "adg_init_host", "adg_get_state_host", "adg_set_grad_memory", "adg_set_wait_limit",
 ]
 
 
