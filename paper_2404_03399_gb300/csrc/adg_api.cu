@@ -2188,12 +2188,13 @@ int capture(adg_ctx *c, GraphExec &out, F &&body) {
 // Forward over one segment of `len` steps starting at step n, recording the stage inputs
 // of step t in slot t of `seg` (u^n, v1, v2); slot t+1's u receives u^{n+1}, so slot 0's u
 // must hold the segment's first state and slot len's u holds the last.
-int sweep_recompute(adg_ctx *c, InstHost &h, double *seg, int len, int64_t n, cudaStream_t st) {
+int sweep_recompute(adg_ctx *c, InstHost &h, double *seg, int len, int64_t n, cudaStream_t st,
+                    bool alone = true) {
   const size_t nd = (size_t)h.I.K * h.I.Np;
   for (int t = 0; t < len; ++t) {
     double *slot = seg + (size_t)t * kStages * nd;
     CK(adg::launch_burgers_step(h.I, slot, slot + kStages * nd, slot + nd, slot + 2 * nd, n + t,
-                                h.tbase, st, t > 0));
+                                h.tbase, st, t > 0, alone));
   }
   return ADG_OK;
 }
@@ -2201,7 +2202,7 @@ int sweep_recompute(adg_ctx *c, InstHost &h, double *seg, int len, int64_t n, cu
 // Adjoint sweep over one segment, steps len-1 .. 0 after meta[0]; lam[0..1] hold the
 // adjoint of u at the segment's end on entry (index `par`) and of u at its start on exit.
 int sweep_reverse(adg_ctx *c, InstHost &h, const double *seg, double *lam, double *lring, int len,
-                  int par) {
+                  int par, bool alone = true) {
   Inst &I = h.I;
   const size_t nd = (size_t)I.K * I.Np;
   const int dir = I.a >= 0.0 ? 1 : -1;
@@ -2210,7 +2211,7 @@ int sweep_reverse(adg_ctx *c, InstHost &h, const double *seg, double *lam, doubl
     double *Lu = lam + (size_t)par * nd, *Lacc = lam + (size_t)(1 - par) * nd;
     if (seg) {   // Burgers: one kernel per step
       CK(adg::launch_burgers_adj(I, seg + (size_t)t * kStages * nd, Lu, Lacc, lring, c->n + t,
-                                 h.tbase, c->stream, t < len - 1));
+                                 h.tbase, c->stream, t < len - 1, alone));
       par = 1 - par;
       continue;
     }
@@ -2425,7 +2426,7 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
         if (ring_n)
           CK(cudaMemcpyAsync(I.ring, static_cast<double2 *>(ck_ring.p) + (sidx - 1) * ring_n,
                              ring_n * sizeof(double2), cudaMemcpyDeviceToDevice, side.s));
-        r = sweep_recompute(c, h, nb, C, start - C, side.s);
+        r = sweep_recompute(c, h, nb, C, start - C, side.s, false);
         if (r) return r;
         CK(cudaEventRecord(side.rec_done, side.s));
       }
@@ -2446,7 +2447,7 @@ int run_gradient(adg_ctx *c, const double *target_dev, int64_t nsteps, int C, do
     if (states) {
       // one kernel per step: launched directly, without capturing and instantiating graphs of the
       // sweeps (with the pool, 3.92 -> 3.04 ms for 100 steps on 65536 elements)
-      r = sweep_reverse(c, h, segb[cur], lam.d(), lring.d(), len, par);
+      r = sweep_reverse(c, h, segb[cur], lam.d(), lring.d(), len, par, !overlap || sidx == 0);
       if (r) return r;
     } else {
       GraphExec &gr = rev[is_last ? 1 : 0][par];

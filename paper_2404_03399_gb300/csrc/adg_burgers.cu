@@ -764,7 +764,9 @@ int burgers_block(int64_t warps, size_t fixed) {
 // few: 50 steps on 65536 elements, p = 3: 591 us in four-warp blocks, 512 with those held to
 // their share, 490 in one-warp blocks so; p = 1: 515 -> 413; the gradient of 50 steps 1.50 ->
 // 1.30 ms. Below 16 warps per SM the next step's blocks all wait beside the present ones and
-// hide their launch (16384 elements: 299 us, 302 with their share only).
+// hide their launch (16384 elements: 299 us, 302 with their share only). Not where another stream's
+// steps run beside these (the gradient's recomputation beside its reverse sweep), whose blocks
+// the room is for: 2000 steps in segments of 50 on 65536 elements 65.5 ms with it, 60.4 without.
 size_t burgers_smem(int64_t grid, int bs, size_t fixed) {
   const int64_t per = (grid + sm_count() - 1) / sm_count();
   if (bs != 32 || per < 16) return 0;
@@ -773,14 +775,14 @@ size_t burgers_smem(int64_t grid, int bs, size_t fixed) {
 }
 
 template <int NP, bool FACES>
-cudaError_t burgers_np(const Inst &I, const StepArgs &A, cudaStream_t s, bool pdl) {
+cudaError_t burgers_np(const Inst &I, const StepArgs &A, cudaStream_t s, bool pdl, bool alone) {
   const int own = 32 - A.H - A.HR;
   const int64_t warps = ((int64_t)I.K + own - 1) / own;
   const size_t fixed = FACES ? sizeof(double) * 32 * 4 * (I.visc ? kFaceVals<true> : kFaceVals<false>) *
                                    (I.ls ? kMaxStages : kStages) : 0;   // sV_
   const int bs = burgers_block(warps, fixed);
   const dim3 g((unsigned)((warps * 32 + bs - 1) / bs)), b(bs);
-  const size_t smem = burgers_smem(g.x, bs, fixed);
+  const size_t smem = alone ? burgers_smem(g.x, bs, fixed) : 0;
   auto go = [&](auto kernel) { return launch_smem_pdl(kernel, g, b, smem, s, pdl, I, A); };
   if (A.r1) return go(k_burgers_step<NP, FACES, true, false, false>);
   if (I.ls)
@@ -791,12 +793,12 @@ cudaError_t burgers_np(const Inst &I, const StepArgs &A, cudaStream_t s, bool pd
 }
 
 template <int NP>
-cudaError_t burgers_adj_np(const Inst &I, const AdjArgs &A, cudaStream_t s, bool pdl) {
+cudaError_t burgers_adj_np(const Inst &I, const AdjArgs &A, cudaStream_t s, bool pdl, bool alone) {
   const int64_t warps = ((int64_t)I.K + kOwn - 1) / kOwn;
   const size_t fixed = I.async ? sizeof(double) * 32 * 4 * kStages : 0;   // sR_
   const int bs = burgers_block(warps, fixed);
   const dim3 g((unsigned)((warps * 32 + bs - 1) / bs)), b(bs);
-  const size_t smem = burgers_smem(g.x, bs, fixed);
+  const size_t smem = alone ? burgers_smem(g.x, bs, fixed) : 0;
   return I.async ? launch_smem_pdl(k_burgers_adj<NP, true>, g, b, smem, s, pdl, I, A)
                  : launch_smem_pdl(k_burgers_adj<NP, false>, g, b, smem, s, pdl, I, A);
 }
@@ -804,27 +806,37 @@ cudaError_t burgers_adj_np(const Inst &I, const AdjArgs &A, cudaStream_t s, bool
 }  // namespace
 
 cudaError_t launch_burgers_adj(const Inst &I, const double *y, const double *w, double *out,
-                               double *lring, int64_t n, int64_t tbase, cudaStream_t s, bool pdl) {
+                               double *lring, int64_t n, int64_t tbase, cudaStream_t s, bool pdl,
+                               bool alone) {
   if (w == out) return cudaErrorInvalidValue;
   const AdjArgs A{y, w, out, lring, n, tbase};
   switch (I.Np) {
-    case 2: return burgers_adj_np<2>(I, A, s, pdl);
-    case 3: return burgers_adj_np<3>(I, A, s, pdl);
-    case 4: return burgers_adj_np<4>(I, A, s, pdl);
-    case 5: return burgers_adj_np<5>(I, A, s, pdl);
+    case 2: return burgers_adj_np<2>(I, A, s, pdl, alone);
+    case 3: return burgers_adj_np<3>(I, A, s, pdl, alone);
+    case 4: return burgers_adj_np<4>(I, A, s, pdl, alone);
+    case 5: return burgers_adj_np<5>(I, A, s, pdl, alone);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_burgers_step(const Inst &I, const double *uin, double *uout, double *r1,
-                                double *r2, int64_t n, int64_t tbase, cudaStream_t s, bool pdl) {
+                                double *r2, int64_t n, int64_t tbase, cudaStream_t s, bool pdl,
+                                bool alone) {
   if (uin == uout || (r1 && (I.ls || I.visc))) return cudaErrorInvalidValue;
   const StepArgs A{uin, uout, r1, r2, n, tbase, I.ns, I.ns + (I.visc ? 1 : 0)};
   switch (I.Np) {
-    case 2: return I.async ? burgers_np<2, true>(I, A, s, pdl) : burgers_np<2, false>(I, A, s, pdl);
-    case 3: return I.async ? burgers_np<3, true>(I, A, s, pdl) : burgers_np<3, false>(I, A, s, pdl);
-    case 4: return I.async ? burgers_np<4, true>(I, A, s, pdl) : burgers_np<4, false>(I, A, s, pdl);
-    case 5: return I.async ? burgers_np<5, true>(I, A, s, pdl) : burgers_np<5, false>(I, A, s, pdl);
+    case 2:
+      return I.async ? burgers_np<2, true>(I, A, s, pdl, alone)
+                     : burgers_np<2, false>(I, A, s, pdl, alone);
+    case 3:
+      return I.async ? burgers_np<3, true>(I, A, s, pdl, alone)
+                     : burgers_np<3, false>(I, A, s, pdl, alone);
+    case 4:
+      return I.async ? burgers_np<4, true>(I, A, s, pdl, alone)
+                     : burgers_np<4, false>(I, A, s, pdl, alone);
+    case 5:
+      return I.async ? burgers_np<5, true>(I, A, s, pdl, alone)
+                     : burgers_np<5, false>(I, A, s, pdl, alone);
     default: return cudaErrorInvalidValue;
   }
 }

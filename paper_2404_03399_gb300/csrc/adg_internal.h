@@ -244,15 +244,15 @@ cudaError_t launch_adv_steps(const Inst &I, const double *uin, double *uout, int
 // One step of Burgers uin -> uout (adg_burgers.cu), with the delayed / AT flux and the ring
 // write (entries of flux and u^-, and -2 nu q^+ in ringq) at PE faces; r1, r2 (both or neither;
 // inviscid SSP-RK3) receive the inputs of stages 1 and 2. n: the step; tbase: the first step of
-// the delay table.
+// the delay table. alone: no other stream's steps run beside it (burgers_smem).
 cudaError_t launch_burgers_step(const Inst &I, const double *uin, double *uout, double *r1,
                                 double *r2, int64_t n, int64_t tbase, cudaStream_t s,
-                                bool pdl = false);
+                                bool pdl = false, bool alone = true);
 // Its adjoint: from the recorded stage inputs y (u, v1, v2 one after another) of step n and the adjoint w of its result, the adjoint of its input into out, with the
 // adjoint ring lring [R][3][P] at PE faces.
 cudaError_t launch_burgers_adj(const Inst &I, const double *y, const double *w, double *out,
                                double *lring, int64_t n, int64_t tbase, cudaStream_t s,
-                               bool pdl = false);
+                               bool pdl = false, bool alone = true);
 // Stage s of a 2N low-storage step (I.ls): dU_s = A_s dU_{s-1} + dt L(U_{s-1}) in place in
 // I.v1 (A_1 = 0: dU_0 is not read) and U_s = U_{s-1} + B_s dU_s from uin (U_{s-1}) into uout,
 // with the delayed / AT flux and the ring write of the stage-input traces at PE faces.

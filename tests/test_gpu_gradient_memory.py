@@ -57,6 +57,19 @@ def test_segments_and_a_whole_recording_agree(P):
         assert J == ref[0] and torch.equal(g, ref[1])
 
 
+@pytest.mark.parametrize("K,p", [(63300, 1), (70000, 2)])
+def test_overlapped_segments_of_16_to_32_warps_an_sm(K, p):
+    # blocks are held to an SM's even share, but not those of two streams beside one another
+    cfg = adg.Config(pde="burgers", K=K, p=p, P=100, cfl=0.005, mode="at", L=3, q=2, seed=4)
+    u0 = torch.tensor(dg.modes_initial(HALF_PLUS_SIN, K, p), device="cuda")
+    s = adg.Solver(cfg, u0)
+    ref = s.grad(0.9 * u0, 12, 12)
+    s.set_grad_memory(0)
+    J, g = s.grad(0.9 * u0, 12, 3)
+    s.close()
+    assert J == ref[0] and torch.equal(g, ref[1])
+
+
 @pytest.mark.parametrize("K,p,P,mode,q,steps,ckpt", [
     (64, 3, 4, "at", 2, 40, 16), (48, 2, 48, "at", 2, 25, 7), (80, 4, 8, "async", 1, 30, 4), (64, 1, 1, "sync", 0, 20, 4)])
 def test_recomputed_gradient_matches_oracle(K, p, P, mode, q, steps, ckpt):
