@@ -419,12 +419,16 @@ int fail(adg_ctx *c, int code, const std::string &msg) {
   return code;
 }
 
+// A failed call's error is taken off the thread's record: the next kernel launch, of whatever
+// context, would report it as its own.
 #define CK(call)                                                                          \
   do {                                                                                    \
     cudaError_t e_ = (call);                                                              \
-    if (e_ != cudaSuccess)                                                                \
+    if (e_ != cudaSuccess) {                                                              \
+      (void)cudaGetLastError();                                                           \
       return fail(c, e_ == cudaErrorMemoryAllocation ? ADG_ENOMEM : ADG_ECUDA,            \
                   std::string(#call) + ": " + cudaGetErrorString(e_));                    \
+    }                                                                                     \
   } while (0)
 
 // The device address of a caller's host buffer where kernels can use it in place: pinned

@@ -1,10 +1,13 @@
 """Several solvers open at once: what one needs of a kernel that they share (its limit of shared
 memory) leaves the others' launches as they were."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 import paper_2404_03399_gb300 as adg  # noqa: E402
+from paper_2404_03399_gb300 import _abi  # noqa: E402
 from workloads import random_nodal  # noqa: E402
 
 pytestmark = pytest.mark.gpu
@@ -29,3 +32,16 @@ def test_a_run_of_more_faces_steps_after_one_of_fewer_is_made(p, rk):
         ref = s.state().cpu().numpy()
         s.close()
         assert np.array_equal(got, ref)
+
+
+def test_a_solver_that_does_not_fit_leaves_the_next_one_alone():
+    # four fields of 3 x 2^30 x 5 values, 515 GB: refused before u0 is read
+    lib, ctx = adg.load(), C.c_void_p()
+    u0 = torch.zeros(1, dtype=torch.float64, device="cuda")
+    c, keep = adg.Config(pde="euler", K=1 << 30, p=4, dt=1e-9, rk="rk2").to_c()
+    assert lib.adg_init(C.byref(c), u0.data_ptr(), None, C.byref(ctx)) == _abi.ADG_ENOMEM
+    cfg = adg.Config(pde="advection", K=64, p=2, cfl=0.002)
+    s = adg.Solver(cfg, torch.ones((64, 3), dtype=torch.float64, device="cuda"))
+    s.step(3)
+    assert s.integral() == pytest.approx(cfg.x1 - cfg.x0)
+    s.close()
