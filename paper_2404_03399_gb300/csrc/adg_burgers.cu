@@ -551,10 +551,12 @@ __device__ __noinline__ void burgers_adj_fp64(const Inst &I, const AdjArgs &A, i
 // steps) with this kernel: 6.3 -> 3.9 ms, against three FP64 stage kernels of 14 us each, bound
 // by the FP64 pipe (11.3 -> 2.9 ms with the forward's step and without recomputation). Bound by
 // the latency of a warp's chain: 65536 elements are 17 warps per SM, and the 5 million warp
-// instructions of a launch some 4 of its 12 us. At p = 3 the compiler's own choice was 80
-// registers with spills (2.92 against 2.75 ms at the 96 of five blocks).
+// instructions of a launch some 4 of its 12 us. The compiler's own choices are 64 to 80
+// registers, with spills at p = 1 and 2 (and 3, 2.92 ms); the 96 of five blocks hold every degree
+// but p = 4, which takes 128, without them (p = 3 2.75 ms; p = 2 on 65536 elements 2.157 -> 2.139
+// ms, p = 1 1.879 -> 1.866).
 template <int NP, bool FACES>
-__global__ void __launch_bounds__(128, NP == 4 ? 5 : 0) k_burgers_adj(const __grid_constant__ Inst I,
+__global__ void __launch_bounds__(128, NP <= 4 ? 5 : 0) k_burgers_adj(const __grid_constant__ Inst I,
                                                      const __grid_constant__ AdjArgs A) {
   constexpr int HP = NP / 2, MID = NP % 2;
   __shared__ double sR_[FACES ? 4 * kStages : 1][32];
