@@ -103,7 +103,7 @@ __device__ __noinline__ void burgers_step_fp64(const Inst &I, const StepArgs &A,
   for (int s = 0; s < S; ++s) {
     const StageConsts &C = I.sc[LS ? 0 : s];
     const double vl = __shfl_up_sync(full, v[NP - 1], 1);
-    double FL = num_flux<1>(0.0, vl, v[0]);
+    double FL = llf_flux(vl, v[0]);
     const size_t at = FACES && pe ? ((size_t)nm * I.ns + s) * I.P + e / I.Kpe : 0;
     if (FACES && pe) {
       if (own) I.ring[at] = make_double2(FL, vl);
@@ -131,8 +131,8 @@ __device__ __noinline__ void burgers_step_fp64(const Inst &I, const StepArgs &A,
       jqR = __shfl_down_sync(full, qL, 1) - q[NP - 1];
     }
     const double FR = __shfl_down_sync(full, FL, 1);
-    const double jL = __dsub_rn(phys_flux<1>(0.0, v[0]), FL);
-    const double jR = __dsub_rn(phys_flux<1>(0.0, v[NP - 1]), FR);
+    const double jL = __dsub_rn(burgers_flux(v[0]), FL);
+    const double jR = __dsub_rn(burgers_flux(v[NP - 1]), FR);
     double g[NP], out[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) g[i] = v[i] * v[i];

@@ -16,16 +16,10 @@ __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Physical flux f(u): a u (advection) or u^2/2 (Burgers). Explicit round-to-nearest
-// intrinsics keep every evaluation of a face flux bit-identical wherever it is computed.
-template <int PDE>
-__device__ __forceinline__ double phys_flux(double a, double u) {
-  if (PDE == 0) return __dmul_rn(a, u);
-  return __dmul_rn(0.5, __dmul_rn(u, u));
-}
+// Physical flux u^2/2 of Burgers. Explicit round-to-nearest intrinsics keep every evaluation of
+// a face flux bit-identical wherever it is computed.
+__device__ __forceinline__ double burgers_flux(double u) { return __dmul_rn(0.5, __dmul_rn(u, u)); }
 
-// Numerical flux (Section 6.1): upwind a u^- (a >= 0) or a u^+ (a < 0); local
-// Lax-Friedrichs 1/2 (f(u^-) + f(u^+)) - 1/2 max(|u^-|, |u^+|) (u^+ - u^-) for Burgers.
 // Comparisons and max/abs on FP64 values done on their IEEE bit patterns with integer
 // instructions (exact for finite values; on this part FP64 compares and min/max occupy the
 // FP64 pipe). |x| as bits, max(|a|, |b|), and "x >= 0" (true for +0 and -0).
@@ -40,11 +34,11 @@ __device__ __forceinline__ bool nonneg(double x) {
   return __double_as_longlong(x) >= 0 || abs_bits(x) == 0;
 }
 
-template <int PDE>
-__device__ __forceinline__ double num_flux(double a, double uL, double uR) {
-  if (PDE == 0) return __dmul_rn(a, a >= 0.0 ? uL : uR);
+// Local Lax-Friedrichs flux of Burgers (Section 6.1),
+// 1/2 (f(u^-) + f(u^+)) - 1/2 max(|u^-|, |u^+|) (u^+ - u^-).
+__device__ __forceinline__ double llf_flux(double uL, double uR) {
   const double lam = abs_max(uL, uR);
-  const double avg = __dmul_rn(0.5, __dadd_rn(phys_flux<1>(a, uL), phys_flux<1>(a, uR)));
+  const double avg = __dmul_rn(0.5, __dadd_rn(burgers_flux(uL), burgers_flux(uR)));
   return __dsub_rn(avg, __dmul_rn(__dmul_rn(0.5, lam), __dsub_rn(uR, uL)));
 }
 
