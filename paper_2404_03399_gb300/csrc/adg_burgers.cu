@@ -376,10 +376,6 @@ if constexpr (!LS && !VISC) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) r[k] >>= d;
       }
-      // 2^58 / 3 lies a third above an integer: the next one is taken a third of the time, by a
-      // square's low bits, so that the field does not shrink by 2^-58 a step (500 steps: 1.2e-15
-      // to 1.8e-15 off, 1.4e-15 to 2.5e-15 without)
-      const int third = kThirdLo + (((unsigned)G[0] & 255u) < 85u ? 1 : 0);
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
         const long long x = r[k];
@@ -409,7 +405,7 @@ if constexpr (!LS && !VISC) {
           mag |= bf_mag(T) >> 2;   // below 2^60: its high limb fits 32 bits
           int th, tl;
           fx_split(T, th, tl);
-          v[k] = fx_scaled(make_int2(kThirdHi, third), th, tl);
+          v[k] = fx_scaled(make_int2(kThirdHi, kThirdLo), th, tl);
         }
         mag |= bf_mag(v[k]);
       }
