@@ -1555,9 +1555,9 @@ int setup_instance(adg_ctx *c, InstHost &h, const adg_config *cfg, const double 
         a += o.M[i * Np + j];
         b += o.M[j * Np + i] * o.x[i];
       }
-      I.avg_w[j] = (double)(0.5L * a);
-      I.p1_w[j] = (double)(1.5L * b);
-      I.xi[j] = (double)o.x[j];
+      I.lim.avg[j] = (double)(0.5L * a);
+      I.lim.p1[j] = (double)(1.5L * b);
+      I.lim.xi[j] = (double)o.x[j];
     }
   }
   if (I.visc || I.euler) {

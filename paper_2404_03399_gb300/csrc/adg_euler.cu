@@ -212,17 +212,17 @@ __device__ __forceinline__ double limited_slope(double a1, double dp, double dm,
 
 template <int NP>
 __device__ __forceinline__ double cell_average(const Inst &I, const double *v) {
-  double a = I.avg_w[0] * v[0];
+  double a = I.lim.avg[0] * v[0];
 #pragma unroll
-  for (int j = 1; j < NP; ++j) a = fma(I.avg_w[j], v[j], a);
+  for (int j = 1; j < NP; ++j) a = fma(I.lim.avg[j], v[j], a);
   return a;
 }
 
 template <int NP>
 __device__ __forceinline__ double first_moment(const Inst &I, const double *v) {
-  double a = I.p1_w[0] * v[0];
+  double a = I.lim.p1[0] * v[0];
 #pragma unroll
-  for (int j = 1; j < NP; ++j) a = fma(I.p1_w[j], v[j], a);
+  for (int j = 1; j < NP; ++j) a = fma(I.lim.p1[j], v[j], a);
   return a;
 }
 
@@ -235,7 +235,7 @@ __device__ __forceinline__ void limit_element(const Inst &I, const double *v, do
   if ((__double_as_longlong(a1) & 0x7fffffffffffffffLL) <= __double_as_longlong(keep)) a1n = a1;
   const bool change = a1n != a1;
 #pragma unroll
-  for (int i = 0; i < NP; ++i) out[i] = change ? fma(a1n, I.xi[i], a0) : v[i];
+  for (int i = 0; i < NP; ++i) out[i] = change ? fma(a1n, I.lim.xi[i], a0) : v[i];
 }
 
 template <int NP, bool PES>
