@@ -866,7 +866,7 @@ def main():
                     f"lanes per clock per SM sub-partition ({sms} SMs x 4, {sm_mhz:.0f} MHz)",
             "pipe_bound_ms": pipe_s * 1e3, "frac": pipe_s / step_s}
     else:
-        roofline["kernel"] = f"k_step_fused / k_stage ({variant}, FP64)"
+        roofline["kernel"] = f"k_step_fused / k_stage_halo ({variant}, FP64)"
         roofline["fp64"] = {"achieved_tflops": ndof * FLOP_PER_DOF_STEP / step_s / 1e12,
                             "peak_tflops": fp64_tflops,
                             "frac": ndof * FLOP_PER_DOF_STEP / step_s / 1e12 / fp64_tflops}
@@ -910,8 +910,8 @@ def main():
         # solution after the same steps
         line["accuracy"] = {"advection_16m": {"at": acc_at, "sync": acc_sync,
                                               "norm": "max |u - u_exact| / max |u_exact|"}}
-        # the Burgers workload (LLF, K = 2^20, p = 4, 1024 PEs, AT2, L = 4): the staged
-        # stage kernels, at the stated Courant number 0.05 and at 0.005, inside the stability
+        # the Burgers workload (LLF, K = 2^20, p = 4, 1024 PEs, AT2, L = 4),
+        # one launch a step, at the stated Courant number 0.05 and at 0.005, inside the stability
         # bound of the delayed self-feedback
         bline = {"workload": "Burgers u0 = 0.5 + sin x, K = 2^20, p = 4, LLF, SSP-RK3, 1024 PEs, "
                              "delays uniform in {0..3} (L = 4), AT order 2",

@@ -85,12 +85,11 @@ enum {
  *               error is no larger than that of FP64 stages.
  *   rk        : ADG_SSPRK3 (default; every variant, adg_grad and batches), or one of the
  *               low-storage schemes of the kind Section 6 integrates with, run in Williamson's
- *               2N form (dU_s = A_s dU_{s-1} + dt L(U_{s-1}), U_s = U_{s-1} + B_s dU_s) by the
- *               staged kernels: ADG_RK1, ADG_RK2 (Eq. dg2-rk2 as A = (0, -1),
- *               B = (1, 1/2)), ADG_LSRK3, ADG_LSRK4. At PE faces stage s of a step reads the
- *               stage-s inputs of the delayed step. A low-storage scheme is a single-instance
- *               option: adg_batch_init and adg_grad reject it (ADG_EINVAL), and so does a
- *               composed variant (ADG_VARIANT_COMPOSED, ADG_VARIANT_COMPOSED_FIXED).
+ *               2N form (dU_s = A_s dU_{s-1} + dt L(U_{s-1}), U_s = U_{s-1} + B_s dU_s), for
+ *               upwind advection with a > 0 also composed (variant): ADG_RK1, ADG_RK2 (Eq.
+ *               dg2-rk2 as A = (0, -1), B = (1, 1/2)), ADG_LSRK3, ADG_LSRK4. At PE faces stage s
+ *               of a step reads the stage-s inputs of the delayed step. A low-storage scheme is
+ *               a single-instance option: adg_batch_init and adg_grad reject it (ADG_EINVAL).
  *   K, p, P   : elements, polynomial degree (1..ADG_MAX_P), PEs; K % P == 0, P >= 1.
  *   x0, x1    : periodic domain [x0, x1], x1 > x0.
  *   a         : advection speed (advection only).
@@ -115,8 +114,8 @@ enum {
  *               (Eq. burgers; pde ADG_BURGERS, nu > 0, finite) by the local DG method of
  *               Section 6: q = u_x with the alternating flux uhat = u^-, the viscous flux
  *               qhat = q^+, Lax-Friedrichs for u u_x; at PE faces uhat, the Lax-Friedrichs
- *               flux and qhat all take the AT sum over the common delayed level. Staged
- *               kernels, any rk; dt from cfl uses max|u0| only (the diffusive limit
+ *               flux and qhat all take the AT sum over the common delayed level.
+ *               Any rk; dt from cfl uses max|u0| only (the diffusive limit
  *               nu dt / dx^2 is the caller's: give dt or a small cfl). Single instances only
  *               (adg_batch_init, adg_grad: ADG_EINVAL).
  *   pde ADG_EULER (flux ADG_LLF): the one-dimensional Euler equations of Section 6's Sod
@@ -127,9 +126,12 @@ enum {
  *               components one after another). limiter = 1 applies the TVB-minmod (MUSCL)
  *               slope limiter to every stage output, keeping slopes |a1| <= tvb_m dx^2 / 2
  *               (tvb_m = 0: minmod); its stencil ends at PE faces. dt must be given (> 0).
- *               adg_integral reports the integral of rho. Single instances, staged kernels;
+ *               adg_integral reports the integral of rho. Single instances;
  *               batches, adg_grad and the composed variants reject it (ADG_EINVAL).
- *   variant   : ADG_VARIANT_AUTO (0), ADG_VARIANT_STAGED (1): one kernel per RK stage, or
+ *   variant   : ADG_VARIANT_AUTO (0), ADG_VARIANT_STAGED (1): stage by stage (advection in FP64, a
+ *               kernel per RK stage or, on small meshes, several steps a launch with the same
+ *               results; Burgers and Euler take no other variant: a kernel per step of Burgers,
+ *               see pde), or
  *               ADG_VARIANT_COMPOSED (2): the stages of one step of upwind advection with a > 0
  *               (SSP-RK3, or a low-storage scheme of up to three stages) composed into one
  *               stencil per step in FP64, with the delayed / AT flux at PE faces added as a

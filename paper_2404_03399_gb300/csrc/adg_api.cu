@@ -403,8 +403,8 @@ struct adg_ctx {
   cudaGraphExec_t gexec[4] = {};   // one graph of G steps per chunk kind (kChunk*)
   int fx_live = 0;                 // fixed-point state: 0 in u (FP64), 1 in v1, 2 in v2 (int64)
   bool u_fresh = true;             // u holds the state of step n (FP64)
-  int G = 32;                      // steps per graph (128 measured slower: 78.5 against
-                                   // 77.2 ms for 2000 steps of the adjoint workload)
+  int G = 32;                      // steps per graph (128: 0.1 us a step less at 2.4 to 20 us a
+                                   // step, for runs of 128 steps and more only)
   int64_t n = 0;
   long long polls = adg::kRunPolls;   // of a run kernel's wait for its other blocks
   // set by a kernel whose bounded wait ran out (mapped host memory, read after a synchronisation)
@@ -1820,8 +1820,10 @@ int launch_fused_steps(adg_ctx *c, int nsteps, int kind);
 // Steps are launched directly (not through CUDA graphs) from 2^20 DOF in all: a step there
 // takes hundreds of microseconds, and programmatic launches overlapped better outside a graph
 // (0.2315 -> 0.2276 ms per fixed-point step on the 2^26-DOF mesh). Below, the host's launch
-// rate is the bound: 2000 staged Burgers steps on 262144 DOF took 99.6 ms launched directly
-// and 77.1 ms as graphs.
+// rate is the bound (us a step as graphs and launched directly, advection, p = 3, 16384
+// elements: five 2N stages 23.6, 34.9; the FP64 composed step 11.3, 16.1; SSP-RK3 stages several
+// steps a launch 8.0, 9.3). Burgers steps and the run kernel, one launch a step or less, go
+// directly whatever the size (adg_step).
 bool direct_launches(const adg_ctx *c) {
   int64_t dof = 0;
   for (const auto &h : c->inst) dof += (int64_t)h.I.K * h.I.Np;

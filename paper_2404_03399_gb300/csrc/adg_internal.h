@@ -20,9 +20,10 @@ int sm_count();
 
 // Block size of the stage kernels: 256, or one warp when the mesh gives fewer than two
 // 256-blocks per SM. Small meshes are latency-bound and make a single wave, whose length is
-// set by the SMs holding the most warps: one-warp blocks spread them evenly (K = 65536, 2185
-// warps of the halo-lane kernels: forward 78.1 -> 77.2 ms and gradient 209 -> 205 ms over
-// 2000 steps, against 128-thread blocks; 64-thread blocks gave no gain).
+// set by the SMs holding the most warps: one-warp blocks spread them evenly (us a step with
+// one-warp blocks and with 256: five 2N stages of advection, p = 3, on 16384 elements 23.6, 31.2,
+// on 65536 41.0, 45.2; SSP-RK3 stages on 65536 20.3, 21.6; advection's gradient on 16384
+// 24.9, 27.0; Euler on 32768 32.9, 33.4).
 inline int stage_block(int K) { return K < 2 * sm_count() * 256 ? 32 : 256; }
 
 // Folded constants of one SSP-RK3 stage in Shu-Osher form, v_out = alpha u + beta (v + dt L(v)),
@@ -172,7 +173,7 @@ struct alignas(16) Inst {
   int ns;               // stages per step: the ring holds [R][ns][P] stage-input traces; the
                         // composed steps' S (3, or 5 for the five-stage scheme)
   int ls;               // 1: a 2N low-storage scheme (k_lsrk_stage, coefficients lsA, lsB)
-  int visc;             // 1: viscous Burgers by the local DG method (k_ldg_q, then the stage)
+  int visc;             // 1: viscous Burgers by the local DG method (k_burgers_step)
   double lsA[kMaxStages], lsB[kMaxStages];
   // viscous Burgers: nu, the PE faces' -2 nu q^+ [R][ns][P], and
   // q = QD v + qlL (uhat_L - v_0) + qlR (uhat_R - v_p)

@@ -1,6 +1,7 @@
 """Several solvers open at once: what one needs of a kernel that they share (its limit of shared
 memory) leaves the others' launches as they were."""
 import ctypes as C
+import threading
 
 import numpy as np
 import pytest
@@ -45,3 +46,35 @@ def test_a_solver_that_does_not_fit_leaves_the_next_one_alone():
     s.step(3)
     assert s.integral() == pytest.approx(cfg.x1 - cfg.x0)
     s.close()
+
+
+@pytest.mark.parametrize("kind", ["run", "burgers"])
+def test_two_streams_and_threads_side_by_side(kind):
+    # cooperative runs that fill the chip, and Burgers steps launched as programmatic dependents,
+    # each solver stepped by a thread of its own on a stream of its own
+    cfgs = [adg.Config(pde="advection", K=65536, p=p, P=256, cfl=0.002, mode="at", L=5, q=2, seed=p) if kind == "run" else
+            adg.Config(pde="burgers", K=40000, p=p, P=100, cfl=0.005, mode="at", L=4, q=2, seed=p) for p in (3, 2)]
+    u0 = [torch.tensor(0.5 + 0.1 * random_nodal(c.K, c.p, 4), device="cuda") for c in cfgs]
+
+    def steps(s):
+        for _ in range(40):
+            s.step(17)
+
+    ref = []
+    for c, u in zip(cfgs, u0):
+        s = adg.Solver(c, u)
+        steps(s)
+        ref.append(s.state())
+        s.close()
+    torch.cuda.synchronize()
+    solvers = [adg.Solver(c, u, stream=torch.cuda.Stream()) for c, u in zip(cfgs, u0)]
+    for s in solvers:
+        s.set_wait_limit(1 << 20)
+    threads = [threading.Thread(target=steps, args=(s,)) for s in solvers]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for s, r in zip(solvers, ref):
+        assert torch.equal(s.state(), r)
+        s.close()
